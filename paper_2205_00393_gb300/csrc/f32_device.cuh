@@ -16,7 +16,7 @@ __device__ __forceinline__ void bar_sync() {
     else asm volatile("bar.sync 1, 256;" ::: "memory");
 }
 
-constexpr int BM = 64, BN = 64, BK = 16, NT = 256;
+constexpr int BK = 16, NT = 256;
 constexpr int LOG_BK = 4;
 
 __device__ __forceinline__ int64_t slice_offset(const Operand& op, int64_t s) {
@@ -33,14 +33,53 @@ __device__ __forceinline__ int64_t bits_offset(int64_t x, const int64_t* str, in
     return off;
 }
 
-__device__ __forceinline__ void cmac(float2& acc, float2 a, float2 b) {
-    acc.x = fmaf(a.x, b.x, acc.x);
-    acc.x = fmaf(-a.y, b.y, acc.x);
-    acc.y = fmaf(a.x, b.y, acc.y);
-    acc.y = fmaf(a.y, b.x, acc.y);
+// Packed pairs of FP32 values in one 64-bit register: fma.rn.f32x2 rounds each
+// half like fmaf, with one instruction (two cycles of the FMA pipe) for both.
+using f32x2 = unsigned long long;
+
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 swap2(f32x2 v) {
+    const float2 f = unpack2(v);
+    return pack2(f.y, f.x);
 }
 
-// C[m][n] = sum_k A(m,k) B(k,n), one 64x64 tile per CTA, 4x4 complex per thread.
+// C[m][n] = sum_k A(m,k) B(k,n), one BM x 64 tile per CTA of 256 threads, RM x 4
+// complex per thread (BM = 16 RM).
+//
+// What bounds it: the FMA pipe and the 128 bytes per clock that shared memory
+// returns to registers (a broadcast does not make a load cheaper). Real and
+// imaginary parts are accumulated for pairs of rows by packed FMAs,
+//     Cr += Ar (br, br);  Cr += Ai (-bi, -bi);  Ci += Ar (bi, bi);  Ci += Ai (br, br),
+// with Ar, Ai the parts of rows m, m + 1: for every element the four roundings
+// of four scalar FMAs, in the same order. A is staged as two planes (parts), so
+// its pairs are loaded as they are; the doubled factors of B's four columns are
+// made in registers. Per k and thread the 8 x 4 tile issues 64 packed FMAs (128
+// pipe cycles), 6 16-byte loads (24 cycles of shared memory) and 20 moves.
+//
 // Shared-memory stages are double buffered: the gather of tile t+1 goes to
 // registers while tile t is multiplied, then to the other stage (one barrier
 // per tile). Accumulation is two-level: each group of GROUP_TILES k-tiles is
@@ -48,182 +87,367 @@ __device__ __forceinline__ void cmac(float2& acc, float2 a, float2 b) {
 // (Knuth's error-free addition), whose rounding errors are collected in a
 // per-thread compensation kept in shared memory and added once at the end.
 // The FP32 rounding error thus grows like the 64-term partial sums alone
-// instead of also with the K / 64 additions of partials, and the register
-// budget (128 per thread) still keeps two CTAs per SM.
-constexpr int PAD = 2;           // keeps 16-byte alignment of fragment rows
+// instead of also with the K / 64 additions of partials.
 constexpr int GROUP_TILES = 4;   // 64 k-terms per partial sum
 
-
-// B columns are stored interleaved: column n goes to half (n >> 1) & 1 at
-// position (n >> 2) * 2 + (n & 1), so the two 16-byte halves of the four
-// columns a thread owns are contiguous across the warp (one 256-byte span per
-// load instead of a 512-byte stride).
-constexpr int BH = BN / 2 + PAD;
-struct GemmSmem {
-    float2 As[2][BK][BM + PAD];
-    float2 Bs[2][BK][2][BH];
-    int64_t rowA[BM], colB[BN], klA[BK], klB[BK];
-    float2 comp[16][NT];  // TwoSum compensation of each thread's 4 x 4 outputs
+// Tile shape: NTH threads, WN warps along n (the others along m), RM x 4
+// complex per thread.
+template <int NTH, int RM, int WN> struct TileCfg {
+    static constexpr int BM = NTH / 32 / WN * 4 * RM, BN = 32 * WN;
 };
+
+// Staged operands and offset tables of one tile.
+template <int NTH, int RM, int WN> struct GemmStage {
+    static constexpr int BM = TileCfg<NTH, RM, WN>::BM, BN = TileCfg<NTH, RM, WN>::BN;
+    float Ar[2][BK][BM + 4], Ai[2][BK][BM + 4];  // 16-byte aligned rows
+    float2 Bs[2][BK][BN + 2];
+    int64_t rowA[BM], colB[BN], klA[BK], klB[BK];
+    // kstep[b]: offset of k-tile t + 1 minus that of k-tile t when b bits of t
+    // carry (bit b of t + 1 is its lowest set bit)
+    int64_t kstepA[kMaxBits], kstepB[kMaxBits];
+};
+template <int NTH, int RM, int WN> struct GemmSmemT : GemmStage<NTH, RM, WN> {
+    f32x2 comp[4 * RM][NTH];       // TwoSum compensation of each thread's outputs
+};
+using GemmSmem = GemmSmemT<256, 4, 2>;
 
 // a += b with the rounding error of the addition added to c (TwoSum: the
 // error term is exact whatever the magnitudes of a and b)
-__device__ __forceinline__ void two_sum_into(float& a, float b, float& c) {
-    const float s = a + b;
-    const float bv = s - a;
-    const float e = (a - (s - bv)) + (b - bv);
+__device__ __forceinline__ void two_sum_into(f32x2& a, f32x2 b, f32x2& c) {
+    const f32x2 s = add2(a, b);
+    const f32x2 bv = sub2(s, a);
+    const f32x2 e = add2(sub2(a, sub2(s, bv)), sub2(b, bv));
     a = s;
-    c += e;
+    c = add2(c, e);
 }
 
-// Operand pointer of gemm_tile. Alone in a launch (BAR 0) the operands were
+// Operand pointer of a tile. Alone in a launch (BAR 0) the operands were
 // written by earlier launches and may be read through the read-only path;
 // inside the persistent executor (BAR 1) other CTAs of the same launch wrote
 // them, so the loads stay on the coherent path.
 template <int BAR> struct OperandPtr { using type = const float2* __restrict__; };
 template <> struct OperandPtr<1> { using type = const float2*; };
 
-// One 64x64 output tile `tile` of slice z (slice id slice0 + z) of the
-// contraction described by p.
-template <int BAR = 0>
-__device__ __forceinline__ void gemm_tile(const GemmParams& p, int64_t tile, int z, int64_t slice0,
-                                          GemmSmem& sm) {
-    auto& As = sm.As;
-    auto& Bs = sm.Bs;
-    auto& rowA = sm.rowA;
-    auto& colB = sm.colB;
-    auto& klA = sm.klA;
-    auto& klB = sm.klB;
-    const int tid = threadIdx.x;
-    const int64_t M = 1ll << p.mb, N = 1ll << p.nb, K = 1ll << p.kb;
-    const int64_t tiles_n = (N + BN - 1) / BN;
-    const int64_t m0 = (tile / tiles_n) * BM, n0 = (tile % tiles_n) * BN;
-    const int64_t s = slice0 + z;
-    const typename OperandPtr<BAR>::type A = p.A.ptr + z * p.A.batch_stride + slice_offset(p.A, s);
-    const typename OperandPtr<BAR>::type B = p.B.ptr + z * p.B.batch_stride + slice_offset(p.B, s);
+// The gather, staging and products of one output tile (slice z, slice id
+// slice0 + z) of the contraction described by p.
+template <int BAR, int NTH, int RM, int WN> struct TileWork {
+    using Cfg = TileCfg<NTH, RM, WN>;
+    static constexpr int EA = Cfg::BM * BK / NTH, EB = Cfg::BN * BK / NTH;  // elements a thread gathers per k-tile
+    static constexpr int RP = RM / 2;                                      // row pairs of a thread
+    GemmStage<NTH, RM, WN>& sm;
+    int64_t M, N, K, m0, n0;
+    typename OperandPtr<BAR>::type A, B;
+    bool a_kfast, b_nfast;
+    int tm, tn;
+    int64_t khA = 0, khB = 0;  // offsets of the k-tile to gather
+    float2 ra[EA], rb[EB];
 
-    if (tid < BM) rowA[tid] = (m0 + tid < M) ? bits_offset(m0 + tid, p.am, p.mb, 0) : 0;
-    else if (tid < BM + BN) {
-        int t = tid - BM;
-        colB[t] = (n0 + t < N) ? bits_offset(n0 + t, p.bn, p.nb, 0) : 0;
-    } else if (tid < BM + BN + BK) {
-        int t = tid - BM - BN;
-        klA[t] = bits_offset(t, p.ak, p.kb < LOG_BK ? p.kb : LOG_BK, 0);
-    } else if (tid < BM + BN + 2 * BK) {
-        int t = tid - BM - BN - BK;
-        klB[t] = bits_offset(t, p.bk, p.kb < LOG_BK ? p.kb : LOG_BK, 0);
+    // Fills the offset tables; a barrier must follow before the first gather.
+    __device__ __forceinline__ TileWork(const GemmParams& p, int64_t tile, int z, int64_t slice0,
+                                        GemmStage<NTH, RM, WN>& stage)
+        : sm(stage) {
+        const int tid = threadIdx.x;
+        M = 1ll << p.mb;
+        N = 1ll << p.nb;
+        K = 1ll << p.kb;
+        const int64_t tiles_n = (N + Cfg::BN - 1) / Cfg::BN;
+        m0 = (tile / tiles_n) * Cfg::BM;
+        n0 = (tile % tiles_n) * Cfg::BN;
+        A = p.A.ptr + z * p.A.batch_stride + slice_offset(p.A, slice0 + z);
+        B = p.B.ptr + z * p.B.batch_stride + slice_offset(p.B, slice0 + z);
+        for (int t = tid; t < Cfg::BM + Cfg::BN + 2 * BK; t += NTH) {
+            const int kl = p.kb < LOG_BK ? p.kb : LOG_BK;
+            if (t < Cfg::BM) sm.rowA[t] = (m0 + t < M) ? bits_offset(m0 + t, p.am, p.mb, 0) : 0;
+            else if (t < Cfg::BM + Cfg::BN) {
+                const int n = t - Cfg::BM;
+                sm.colB[n] = (n0 + n < N) ? bits_offset(n0 + n, p.bn, p.nb, 0) : 0;
+            } else if (t < Cfg::BM + Cfg::BN + BK) sm.klA[t - Cfg::BM - Cfg::BN] = bits_offset(t - Cfg::BM - Cfg::BN, p.ak, kl, 0);
+            else sm.klB[t - Cfg::BM - Cfg::BN - BK] = bits_offset(t - Cfg::BM - Cfg::BN - BK, p.bk, kl, 0);
+        }
+        if (tid < p.kb - LOG_BK) {
+            int64_t da = p.ak[LOG_BK + tid], db = p.bk[LOG_BK + tid];
+            for (int j = 0; j < tid; ++j) {
+                da -= p.ak[LOG_BK + j];
+                db -= p.bk[LOG_BK + j];
+            }
+            sm.kstepA[tid] = da;
+            sm.kstepB[tid] = db;
+        }
+        // load mapping: walk the operand's unit-stride mode with consecutive threads
+        a_kfast = p.kb > 0 && p.ak[0] == 1;
+        b_nfast = p.nb > 0 && p.bn[0] == 1;
+        // lanes 4 (m) x 8 (n): thread rows tm .. tm + 3 (and, for RM = 8, tm + 16 ..
+        // tm + 19), columns tn, tn + 1, tn + 16, tn + 17
+        const int lane = tid & 31, warp = tid >> 5;
+        tm = (warp / WN) * (4 * RM) + 4 * (lane >> 3);
+        tn = (warp % WN) * 32 + 2 * (lane & 7);
     }
-    // load mapping: walk the operand's unit-stride mode with consecutive threads
-    const bool a_kfast = p.kb > 0 && p.ak[0] == 1;
-    const bool b_nfast = p.nb > 0 && p.bn[0] == 1;
-    int la_k[4], la_m[4], lb_k[4], lb_n[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        int e = tid + i * NT;
-        if (a_kfast) { la_k[i] = e % BK; la_m[i] = e / BK; }
-        else { la_m[i] = e % BM; la_k[i] = e / BM; }
-        if (b_nfast) { lb_n[i] = e % BN; lb_k[i] = e / BN; }
-        else { lb_k[i] = e % BK; lb_n[i] = e / BK; }
+    __device__ __forceinline__ void a_mk(int i, int& m, int& k) const {
+        const int e = threadIdx.x + i * NTH;
+        m = a_kfast ? e / BK : e % Cfg::BM;
+        k = a_kfast ? e % BK : e / Cfg::BM;
     }
-    bar_sync<BAR>();
-
-    float2 ra[4], rb[4];
-    auto gather = [&](int64_t k0) {
-        const int64_t khA = bits_offset(k0, p.ak, p.kb, LOG_BK);
-        const int64_t khB = bits_offset(k0, p.bk, p.kb, LOG_BK);
+    __device__ __forceinline__ void b_nk(int i, int& n, int& k) const {
+        const int e = threadIdx.x + i * NTH;
+        n = b_nfast ? e % Cfg::BN : e / BK;
+        k = b_nfast ? e / Cfg::BN : e % BK;
+    }
+    // moves khA, khB from k-tile t to k-tile t + 1
+    __device__ __forceinline__ void next_tile(int64_t t) {
+        const int carry = __ffsll(t + 1) - 1;
+        khA += sm.kstepA[carry];
+        khB += sm.kstepB[carry];
+    }
+    __device__ __forceinline__ void gather() {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < EA; ++i) {
+            int m, k;
+            a_mk(i, m, k);
             ra[i] = make_float2(0.f, 0.f);
-            if (m0 + la_m[i] < M && k0 + la_k[i] < K) ra[i] = A[rowA[la_m[i]] + khA + klA[la_k[i]]];
+            if (m0 + m < M && k < K) ra[i] = A[khA + sm.rowA[m] + sm.klA[k]];
+        }
+#pragma unroll
+        for (int i = 0; i < EB; ++i) {
+            int n, k;
+            b_nk(i, n, k);
             rb[i] = make_float2(0.f, 0.f);
-            if (n0 + lb_n[i] < N && k0 + lb_k[i] < K) rb[i] = B[colB[lb_n[i]] + khB + klB[lb_k[i]]];
+            if (n0 + n < N && k < K) rb[i] = B[khB + sm.colB[n] + sm.klB[k]];
         }
-    };
-    auto stage_store = [&](int st) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            As[st][la_k[i]][la_m[i]] = ra[i];
-            Bs[st][lb_k[i]][(lb_n[i] >> 1) & 1][(lb_n[i] >> 2) * 2 + (lb_n[i] & 1)] = rb[i];
-        }
-    };
-
-    const int tx = tid & 15, ty = tid >> 4;
-    float2 acc[4][4], part[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            acc[i][j] = make_float2(0.f, 0.f);
-            part[i][j] = make_float2(0.f, 0.f);
-            sm.comp[4 * i + j][tid] = make_float2(0.f, 0.f);  // this thread's own slots
-        }
-
-    const int64_t ntiles = (K + BK - 1) / BK;
-    // K is a power of two: below BK, the one k-tile has K nonzero rows and the
-    // zero-padded rest is skipped
-    const int kmax = K < BK ? (int)K : BK;
-    gather(0);
-    stage_store(0);
-    bar_sync<BAR>();
-    for (int64_t t = 0; t < ntiles; ++t) {
-        const int st = (int)(t & 1);
-        if (t + 1 < ntiles) gather((t + 1) * BK);
-#pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            if (kk >= kmax) break;
-            float4 a01 = *reinterpret_cast<const float4*>(&As[st][kk][4 * ty]);
-            float4 a23 = *reinterpret_cast<const float4*>(&As[st][kk][4 * ty + 2]);
-            float4 b01 = *reinterpret_cast<const float4*>(&Bs[st][kk][0][2 * tx]);
-            float4 b23 = *reinterpret_cast<const float4*>(&Bs[st][kk][1][2 * tx]);
-            float2 a[4] = {make_float2(a01.x, a01.y), make_float2(a01.z, a01.w),
-                           make_float2(a23.x, a23.y), make_float2(a23.z, a23.w)};
-            float2 b[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w),
-                           make_float2(b23.x, b23.y), make_float2(b23.z, b23.w)};
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) cmac(part[i][j], a[i], b[j]);
-        }
-        if ((t + 1) % GROUP_TILES == 0 || t + 1 == ntiles) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    float2 c = sm.comp[4 * i + j][tid];
-                    two_sum_into(acc[i][j].x, part[i][j].x, c.x);
-                    two_sum_into(acc[i][j].y, part[i][j].y, c.y);
-                    sm.comp[4 * i + j][tid] = c;
-                    part[i][j] = make_float2(0.f, 0.f);
-                }
-        }
-        if (t + 1 < ntiles) stage_store(st ^ 1);
-        bar_sync<BAR>();
     }
+    __device__ __forceinline__ void stage_store(int st) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < EA; ++i) {
+            int m, k;
+            a_mk(i, m, k);
+            sm.Ar[st][k][m] = ra[i].x;
+            sm.Ai[st][k][m] = ra[i].y;
+        }
+#pragma unroll
+        for (int i = 0; i < EB; ++i) {
+            int n, k;
+            b_nk(i, n, k);
+            sm.Bs[st][k][n] = rb[i];
+        }
+    }
+    // part[h][row pair][column] += the products of row kk of stage st (h: 0 Re, 1 Im)
+    __device__ __forceinline__ void step(int st, int kk, f32x2 (&part)[2][RP][4]) const {
+        f32x2 ar[RP], ai[RP];
+#pragma unroll
+        for (int q = 0; q < RM / 4; ++q) {
+            const ulonglong2 r = *reinterpret_cast<const ulonglong2*>(&sm.Ar[st][kk][tm + 16 * q]);
+            const ulonglong2 i = *reinterpret_cast<const ulonglong2*>(&sm.Ai[st][kk][tm + 16 * q]);
+            ar[2 * q] = r.x;
+            ar[2 * q + 1] = r.y;
+            ai[2 * q] = i.x;
+            ai[2 * q + 1] = i.y;
+        }
+        const float4 b01 = *reinterpret_cast<const float4*>(&sm.Bs[st][kk][tn]);
+        const float4 b23 = *reinterpret_cast<const float4*>(&sm.Bs[st][kk][tn + 16]);
+        const float br[4] = {b01.x, b01.z, b23.x, b23.z}, bi[4] = {b01.y, b01.w, b23.y, b23.w};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const float2 c = sm.comp[4 * i + j][tid];
-            acc[i][j].x += c.x;
-            acc[i][j].y += c.y;
-        }
-    float2* C = p.C + z * p.c_batch_stride;
+            const f32x2 brr = pack2(br[j], br[j]), bii = pack2(bi[j], bi[j]), bin = pack2(-bi[j], -bi[j]);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        int64_t m = m0 + 4 * ty + i;
-        if (m >= M) continue;
-        if (n0 + 4 * tx + 3 < N) {
-            float4* dst = reinterpret_cast<float4*>(C + m * N + n0 + 4 * tx);
-            dst[0] = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
-            dst[1] = make_float4(acc[i][2].x, acc[i][2].y, acc[i][3].x, acc[i][3].y);
-        } else {
+            for (int i = 0; i < RP; ++i) {
+                part[0][i][j] = fma2(ar[i], brr, part[0][i][j]);
+                part[1][i][j] = fma2(ar[i], bii, part[1][i][j]);
+            }
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                int64_t n = n0 + 4 * tx + j;
-                if (n < N) C[m * N + n] = acc[i][j];
+            for (int i = 0; i < RP; ++i) {
+                part[0][i][j] = fma2(ai[i], bin, part[0][i][j]);
+                part[1][i][j] = fma2(ai[i], brr, part[1][i][j]);
             }
         }
     }
+    // every row of stage st (K is a power of two: below BK, the one k-tile's
+    // zero-padded rows are skipped)
+    __device__ __forceinline__ void multiply(int st, f32x2 (&part)[2][RP][4]) const {
+        if (K >= BK) {
+#pragma unroll
+            for (int kk = 0; kk < BK; ++kk) step(st, kk, part);
+        } else {
+            for (int kk = 0; kk < (int)K; kk += 2) {  // (K = 1: a zero row of both operands)
+                step(st, kk, part);
+                step(st, kk + 1, part);
+            }
+        }
+    }
+    // row of the tile of row pair i, half h
+    __device__ __forceinline__ int64_t row(int i, int h) const { return m0 + tm + 16 * (i / 2) + 2 * (i % 2) + h; }
+};
+
+// One output tile `tile` of slice z (slice id slice0 + z) of the contraction
+// described by p.
+template <int BAR = 0, int NTH = 256, int RM = 4, int WN = 2>
+__device__ __forceinline__ void gemm_tile(const GemmParams& p, int64_t tile, int z, int64_t slice0,
+                                          GemmSmemT<NTH, RM, WN>& sm) {
+    using W = TileWork<BAR, NTH, RM, WN>;
+    constexpr int RP = W::RP;
+    const int tid = threadIdx.x;
+    W w(p, tile, z, slice0, sm);
+    bar_sync<BAR>();
+    f32x2 acc[2][RP][4], part[2][RP][4];
+#pragma unroll
+    for (int i = 0; i < RP; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                acc[h][i][j] = 0;
+                part[h][i][j] = 0;
+            }
+    const int64_t ntiles = (w.K + BK - 1) / BK;
+    w.gather();
+    w.stage_store(0);
+    bar_sync<BAR>();
+    for (int64_t t = 0; t < ntiles; ++t) {
+        const int st = (int)(t & 1);
+        if (t + 1 < ntiles) {
+            w.next_tile(t);
+            w.gather();
+        }
+        w.multiply(st, part);
+        if (t + 1 == ntiles) break;
+        if ((t + 1) % GROUP_TILES == 0) {  // comp: this thread's own slots, written by its first group
+#pragma unroll
+            for (int i = 0; i < RP; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        f32x2 c = t < GROUP_TILES ? 0 : sm.comp[8 * i + 2 * j + h][tid];
+                        two_sum_into(acc[h][i][j], part[h][i][j], c);
+                        sm.comp[8 * i + 2 * j + h][tid] = c;
+                        part[h][i][j] = 0;
+                    }
+        }
+        w.stage_store(st ^ 1);
+        bar_sync<BAR>();
+    }
+    // the last group, then the compensation
+#pragma unroll
+    for (int i = 0; i < RP; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                f32x2 c = ntiles <= GROUP_TILES ? 0 : sm.comp[8 * i + 2 * j + h][tid];
+                two_sum_into(acc[h][i][j], part[h][i][j], c);
+                acc[h][i][j] = add2(acc[h][i][j], c);
+            }
+    float2* C = p.C + z * p.c_batch_stride;
+#pragma unroll
+    for (int i = 0; i < RP; ++i)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {  // columns tn + 16 q, + 1
+            float2 re[2], im[2];  // of the two columns, both rows
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                re[j] = unpack2(acc[0][i][2 * q + j]);
+                im[j] = unpack2(acc[1][i][2 * q + j]);
+            }
+            const int64_t n = w.n0 + w.tn + 16 * q;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int64_t m = w.row(i, h);
+                if (m >= w.M) continue;
+                const float4 v = h ? make_float4(re[0].y, im[0].y, re[1].y, im[1].y)
+                                   : make_float4(re[0].x, im[0].x, re[1].x, im[1].x);
+                if (n + 1 < w.N) *reinterpret_cast<float4*>(C + m * w.N + n) = v;
+                else if (n < w.N) C[m * w.N + n] = make_float2(v.x, v.y);
+            }
+        }
+}
+
+// The same tile by a cluster of CL CTAs, for contractions of few output tiles
+// and a long K. CTA r of the cluster forms the 64-term partials of the k groups
+// r, r + CL, ...; after each round of CL groups the partials are exchanged
+// through distributed shared memory, and the CTA that owns an output adds the
+// CL partials in group order with TwoSum: the sums, and so the bits, of
+// gemm_tile. Thread t's partials live at xch[.][e][t], e = 8 * row pair +
+// 2 * column + h; CTA r owns e in [r E, (r + 1) E), E = 4 RM / CL. Two exchange
+// buffers, so one cluster barrier per round is enough: a CTA refills a buffer
+// after the next round's barrier, which follows every read of it.
+template <int NTH, int WN> struct GemmClusterSmem : GemmStage<NTH, 4, WN> {
+    f32x2 xch[2][16][NTH];
+};
+
+__device__ __forceinline__ f32x2 ld_cluster(const f32x2* p, uint32_t rank) {
+    uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p)), ra;
+    f32x2 v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
+    asm volatile("ld.shared::cluster.b64 %0, [%1];" : "=l"(v) : "r"(ra) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+template <int NTH, int WN, int CL>
+__device__ __forceinline__ void gemm_tile_cluster(const GemmParams& p, int64_t tile, uint32_t rank, int z, int64_t slice0,
+                                                  GemmClusterSmem<NTH, WN>& sm) {
+    static_assert(CL == 2 || CL == 4 || CL == 8, "a CTA owns whole complex outputs");
+    using W = TileWork<0, NTH, 4, WN>;
+    constexpr int E = 16 / CL;
+    const int tid = threadIdx.x;
+    W w(p, tile, z, slice0, sm);
+    f32x2 part[2][2][4], acc[E], comp[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) acc[e] = comp[e] = 0;
+    const int64_t rounds = w.K / (BK * GROUP_TILES) / CL;  // K is a multiple of 64 CL
+    auto seek = [&](int64_t round) {  // the first k-tile of this CTA's group of the round
+        const int64_t k = (round * CL + rank) * (BK * GROUP_TILES);
+        w.khA = bits_offset(k, p.ak, p.kb, LOG_BK);
+        w.khB = bits_offset(k, p.bk, p.kb, LOG_BK);
+    };
+    __syncthreads();
+    seek(0);
+    w.gather();
+    w.stage_store(0);
+    __syncthreads();
+    for (int64_t r = 0; r < rounds; ++r) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) part[0][i][j] = part[1][i][j] = 0;
+#pragma unroll 1
+        for (int t = 0; t < GROUP_TILES; ++t) {
+            const bool more = t + 1 < GROUP_TILES || r + 1 < rounds;
+            if (more) {
+                if (t + 1 < GROUP_TILES) w.next_tile(t);
+                else seek(r + 1);
+                w.gather();
+            }
+            w.multiply(t & 1, part);
+            if (more) w.stage_store((t & 1) ^ 1);
+            __syncthreads();
+        }
+        f32x2(*x)[NTH] = sm.xch[r & 1];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                x[8 * i + 2 * j][tid] = part[0][i][j];
+                x[8 * i + 2 * j + 1][tid] = part[1][i][j];
+            }
+        cluster_barrier();
+#pragma unroll
+        for (int q = 0; q < CL; ++q)
+#pragma unroll
+            for (int e = 0; e < E; ++e) two_sum_into(acc[e], ld_cluster(&x[rank * E + e][tid], q), comp[e]);
+    }
+    float2* C = p.C + z * p.c_batch_stride;
+#pragma unroll
+    for (int e = 0; e < E; e += 2) {
+        const int i = (rank * E + e) / 8, j = (rank * E + e) / 2 % 4;
+        const int64_t n = w.n0 + w.tn + 16 * (j / 2) + j % 2;
+        const float2 re = unpack2(add2(acc[e], comp[e])), im = unpack2(add2(acc[e + 1], comp[e + 1]));
+        if (n < w.N) {
+            if (w.row(i, 0) < w.M) C[w.row(i, 0) * w.N + n] = make_float2(re.x, im.x);
+            if (w.row(i, 1) < w.M) C[w.row(i, 1) * w.N + n] = make_float2(re.y, im.y);
+        }
+    }
+    cluster_barrier();  // this CTA's exchange buffers are read until every CTA is here
 }
 
 // Sum over this thread's k in [k_lo, k_hi) (k = k_lo + lane, + lanes, ...) of

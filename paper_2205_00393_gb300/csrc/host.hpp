@@ -118,7 +118,7 @@ struct Arena {
 struct Group {
     bool per_slice = false;
     std::vector<int> fp32;   // node tensor ids run by one grouped FP32 launch
-    std::vector<int> tc;     // nodes launched one by one: tensor-core nodes and large FP32 nodes
+    std::vector<int> tc;     // nodes launched one by one: tensor-core nodes, and FP32 nodes that are large or of long K
     std::vector<int> stems;  // fused stem groups ending at this level (Plan::stems indices)
     int first = 0;           // first entry of the group's parameters in the table
     int off_first = 0;       // first entry of its n + 1 tile offsets

@@ -244,7 +244,7 @@ tnc_status many_build(ManyCall& mc, cudaStream_t s) {
                     params.push_back(net->groups.params[g.first + k]);
                     netidx.push_back(i);
                     tile_off.push_back(tiles);
-                    tiles += tnc::gemm_f32_tiles(np.mb, np.nb);
+                    tiles += tnc::gemm_f32_group_tiles(np.mb, np.nb);
                 }
                 for (int v : g.tc) mg.singles.emplace_back(i, v);
                 if (per_slice) mg.max_b = std::max<int>(mg.max_b, (int)mc.nb[i]);

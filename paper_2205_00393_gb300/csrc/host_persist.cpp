@@ -225,7 +225,8 @@ static void level_cost_uncached(tnc_net* net, int mode, int64_t b, bool with_inv
 // Launches and estimated seconds of one batch of b slices on the per-level
 // executor (the slice-invariant levels included when with_inv), added to
 // *launches and *seconds: one grouped launch per level for its FP32
-// contractions, three per tensor-core contraction (two operand splits and the
+// contractions of fewer than 256 tiles (those of long K count with it), one for
+// each larger one, three per tensor-core contraction (two operand splits and the
 // GEMM), two for the final contraction. A contraction's time is estimated as
 // the larger of its flops at 300 TFLOP/s and its operand and result bytes,
 // 8 (MK + KN + MN) per slice, at 6 TB/s. Cached by plan_key, since the
@@ -253,11 +254,14 @@ static void level_cost_uncached(tnc_net* net, int mode, int64_t b, bool with_inv
     for (bool per : {false, true}) {
         if (!per && !with_inv) continue;
         for (const Group& g : level_groups(net, mode, per)) {
-            if (!g.fp32.empty()) *launches += 1;
+            bool grouped = !g.fp32.empty();
             for (int v : g.tc) {
                 const NodePlan& np = P.nodes[v - net->n_leaves];
-                *launches += shape_choice(net, mode, np.mb, np.nb, np.kb, np.is_root) ? 3 : 1;
+                if (shape_choice(net, mode, np.mb, np.nb, np.kb, np.is_root)) *launches += 3;
+                else if (tnc::gemm_f32_tiles(np.mb, np.nb) >= 256) *launches += 1;
+                else grouped = true;
             }
+            if (grouped) *launches += 1;
             for (auto* list : {&g.fp32, &g.tc})
                 for (int v : *list) *seconds += node_s(P.nodes[v - net->n_leaves], per ? (double)b : 1.0);
         }

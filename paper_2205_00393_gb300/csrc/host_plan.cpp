@@ -659,10 +659,11 @@ std::vector<Group> level_groups(const tnc_net* net, int mode, bool per_slice) {
             if (P.stems[gi].steps.back() == (int)ni) g.stems.push_back(gi);
             continue;
         }
-        // large contractions keep their own launch (parameters in kernel parameter space)
+        // large contractions and those of long K keep their own launch (parameters
+        // in kernel parameter space)
         if (shape_choice(net, mode, np.mb, np.nb, np.kb, np.is_root) ||
             (net->tuning && tc_node(mode, np.mb, np.nb, np.kb, np.is_root)) ||
-            tnc::gemm_f32_tiles(np.mb, np.nb) >= 256)
+            tnc::gemm_f32_tiles(np.mb, np.nb) >= 256 || tnc::gemm_f32_long(np.kb))
             g.tc.push_back(np.v);
         else
             g.fp32.push_back(np.v);
@@ -705,7 +706,7 @@ tnc_status ensure_groups(tnc_net* net, const Arena& ar, char* ws, int mode, int6
                 gp.slice0 = 0;
                 G.params.push_back(gp);
                 G.tile_off.push_back(tiles);
-                tiles += tnc::gemm_f32_tiles(np.mb, np.nb);
+                tiles += tnc::gemm_f32_group_tiles(np.mb, np.nb);
                 g.cmacs += std::ldexp(1.0, np.mb + np.nb + np.kb);
             }
             G.tile_off.push_back(tiles);

@@ -295,6 +295,14 @@ void set_last_error(const std::string& msg);
 cudaError_t launch_gemm_f32(const GemmParams& p, int batch, cudaStream_t s);
 // 64x64 output tiles of one FP32 contraction of 2^mb x 2^nb outputs.
 int64_t gemm_f32_tiles(int mb, int nb);
+// CTAs of one contraction in a grouped launch (32x64 tiles).
+int64_t gemm_f32_group_tiles(int mb, int nb);
+// K from which a contraction of few tiles is worth a launch of its own, where
+// clusters share its K (launch_gemm_f32), rather than a place in its level's
+// grouped launch: 256, four 64-term groups. (M, N, K) = (2^5, 2^5, 2^8) takes
+// 35 us on one CTA and 14 us on a cluster; at K = 128 the difference (22 against
+// 18 us) is that of one more launch.
+bool gemm_f32_long(int kb);
 // Independent FP32 contractions in one launch; params and tile_off (n + 1
 // prefix offsets of their tile counts) are device arrays.
 cudaError_t launch_gemm_f32_group(const GemmParams* d_params, const int64_t* d_tile_off, int n,

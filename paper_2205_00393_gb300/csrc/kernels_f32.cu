@@ -17,19 +17,33 @@ namespace {
 
 using namespace f32dev;
 
-__global__ void __launch_bounds__(NT, 2) k_gemm_f32(const __grid_constant__ GemmParams p) {
+template <int NTH, int RM, int WN, int MINB>
+__global__ void __launch_bounds__(NTH, MINB) k_gemm_f32(const __grid_constant__ GemmParams p) {
     extern __shared__ __align__(16) uint8_t gemm_dyn[];
-    GemmSmem& sm = *reinterpret_cast<GemmSmem*>(gemm_dyn);
-    gemm_tile(p, blockIdx.x, blockIdx.z, p.slice0, sm);
+    gemm_tile<0, NTH, RM, WN>(p, blockIdx.x, blockIdx.z, p.slice0, *reinterpret_cast<GemmSmemT<NTH, RM, WN>*>(gemm_dyn));
 }
+
+template <int NTH, int WN, int CL>
+__global__ void __launch_bounds__(NTH, 3) k_gemm_f32_cluster(const __grid_constant__ GemmParams p) {
+    extern __shared__ __align__(16) uint8_t gemm_dyn[];
+    gemm_tile_cluster<NTH, WN, CL>(p, blockIdx.x / CL, blockIdx.x % CL, blockIdx.z, p.slice0,
+                                   *reinterpret_cast<GemmClusterSmem<NTH, WN>*>(gemm_dyn));
+}
+
+// Grouped contractions run on 32 x 64 tiles by 128 threads, four CTAs per SM:
+// most nodes of a level have a few tiles at most, and the smaller tile shortens
+// the chain of each (K = 512, M = 2^8, N = 2^6: 58 us against 74 us on the
+// 64 x 64 tile of 256 threads).
+constexpr int GT = 128;
+using GroupSmem = GemmSmemT<GT, 4, 2>;
 
 // Many independent contractions in one launch (nodes of one tree level): CTA
 // b serves tile b - tile_off[i] of node i, tile_off[i] <= b < tile_off[i+1].
-__global__ void __launch_bounds__(NT, 2) k_gemm_f32_group(const GemmParams* __restrict__ params,
+__global__ void __launch_bounds__(GT, 4) k_gemm_f32_group(const GemmParams* __restrict__ params,
                                                        const int64_t* __restrict__ tile_off, int n,
                                                        int64_t slice0) {
     extern __shared__ __align__(16) uint8_t gemm_dyn[];
-    GemmSmem& sm = *reinterpret_cast<GemmSmem*>(gemm_dyn);
+    GroupSmem& sm = *reinterpret_cast<GroupSmem*>(gemm_dyn);
     const int64_t b = blockIdx.x;
     int lo = 0, hi = n - 1;
     while (lo < hi) {
@@ -37,7 +51,7 @@ __global__ void __launch_bounds__(NT, 2) k_gemm_f32_group(const GemmParams* __re
         if (tile_off[mid] <= b) lo = mid;
         else hi = mid - 1;
     }
-    gemm_tile(params[lo], b - tile_off[lo], blockIdx.z, slice0, sm);
+    gemm_tile<0, GT, 4, 2>(params[lo], b - tile_off[lo], blockIdx.z, slice0, sm);
 }
 
 // FP64 partial sums of a contraction with R = M*N <= 64 outputs.
@@ -87,48 +101,112 @@ __global__ void k_slice_sum_f32(const __grid_constant__ SumParams p, int batch, 
 
 }  // namespace
 
-__global__ void __launch_bounds__(NT, 2) k_gemm_f32_group_multi(const GemmParams* __restrict__ params,
+__global__ void __launch_bounds__(GT, 4) k_gemm_f32_group_multi(const GemmParams* __restrict__ params,
                                                              const int64_t* __restrict__ tile_off, int n,
                                                              const int* __restrict__ net,
                                                              const int64_t* __restrict__ rs0,
                                                              const int* __restrict__ rb);
 
-// The FP32 GEMM kernels take GemmSmem (over 48 KB) as dynamic shared memory;
+// The grouped FP32 kernels take GroupSmem (over 48 KB) as dynamic shared memory;
 // the limit is raised once per process (a host-side setting, not a stream
 // operation, so it is safe before or during graph capture).
 cudaError_t gemm_smem_attr() {
     static cudaError_t done = [] {
-        cudaError_t e = cudaFuncSetAttribute(k_gemm_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GemmSmem));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_gemm_f32_group, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GemmSmem));
+        cudaError_t e = cudaFuncSetAttribute(k_gemm_f32_group, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GroupSmem));
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_gemm_f32_group_multi, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)sizeof(GemmSmem));
+                                     (int)sizeof(GroupSmem));
         return e;
     }();
     return done;
 }
 
-cudaError_t launch_gemm_f32(const GemmParams& p, int batch, cudaStream_t s) {
-    int64_t M = 1ll << p.mb, N = 1ll << p.nb;
-    int64_t tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
+template <int NTH, int RM, int WN, int MINB>
+static cudaError_t launch_gemm_f32_tiles(const GemmParams& p, int batch, cudaStream_t s) {
+    using Cfg = TileCfg<NTH, RM, WN>;
+    using Smem = GemmSmemT<NTH, RM, WN>;
+    static const cudaError_t attr = cudaFuncSetAttribute(k_gemm_f32<NTH, RM, WN, MINB>,
+                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
+    if (attr != cudaSuccess) return attr;
+    const int64_t M = 1ll << p.mb, N = 1ll << p.nb;
+    const int64_t tiles = ((M + Cfg::BM - 1) / Cfg::BM) * ((N + Cfg::BN - 1) / Cfg::BN);
     if (tiles > 0x7fffffffll || batch < 1 || batch > 65535) return cudaErrorInvalidConfiguration;
-    cudaError_t e = gemm_smem_attr();
-    if (e != cudaSuccess) return e;
-    k_gemm_f32<<<dim3((unsigned)tiles, 1, batch), NT, sizeof(GemmSmem), s>>>(p);
+    k_gemm_f32<NTH, RM, WN, MINB><<<dim3((unsigned)tiles, 1, batch), NTH, sizeof(Smem), s>>>(p);
     return cudaGetLastError();
+}
+
+template <int NTH, int WN, int CL>
+static cudaError_t launch_gemm_f32_cluster(const GemmParams& p, int batch, cudaStream_t s) {
+    using Cfg = TileCfg<NTH, 4, WN>;
+    using Smem = GemmClusterSmem<NTH, WN>;
+    static const cudaError_t attr = cudaFuncSetAttribute(k_gemm_f32_cluster<NTH, WN, CL>,
+                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
+    if (attr != cudaSuccess) return attr;
+    const int64_t M = 1ll << p.mb, N = 1ll << p.nb;
+    const int64_t tiles = ((M + Cfg::BM - 1) / Cfg::BM) * ((N + Cfg::BN - 1) / Cfg::BN);
+    if (tiles > 0x7fffffffll / CL || batch < 1 || batch > 65535) return cudaErrorInvalidConfiguration;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(tiles * CL), 1, batch);
+    cfg.blockDim = dim3(NTH);
+    cfg.dynamicSmemBytes = sizeof(Smem);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = CL;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_gemm_f32_cluster<NTH, WN, CL>, p);
+}
+
+// Choice of the tile, by the number T of CTAs that 32 x 64 tiles (64 x 32 where
+// N <= 32: half of a 64-wide tile would be padding) give, all slices of the
+// batch together. Every choice gives the same bits.
+//  - few tiles and K >= 128: clusters, whose CTAs share the k groups of one
+//    tile. 152 SMs hold 456 such CTAs, and while T is below an SM each, eight
+//    per tile fill the chip: (M, N, K) = (2^10, 2^6, 2^14) 350 us against 1486
+//    on one CTA per tile, (2^6, 2^6, 2^12) 67 against 379, (2^9, 2^9, 2^9)
+//    55 against 62; at T = 256, four: (2^10, 2^9, 2^10) 148 us, against 158 with
+//    eight and 155 without. Beyond that clusters lose ((2^10, 2^10, 2^10),
+//    T = 512: 274 against 244).
+//  - two SMs' worth of tiles or more: 64 x 64 tiles with 8 x 4 outputs per thread,
+//    which load fewer bytes per product from shared memory: (2^11, 2^11, 2^11)
+//    1515 us (45.4 TFLOP/s, 0.62 of the FFMA rate) against 1677.
+//  - otherwise 32 x 64 tiles (K < 128, or narrow outputs): (2^10, 2^8, 2^7) 30 us
+//    against 34.
+cudaError_t launch_gemm_f32(const GemmParams& p, int batch, cudaStream_t s) {
+    const bool narrow = p.nb <= 5;
+    const int64_t T = narrow ? (int64_t)batch << (p.mb > 6 ? p.mb - 6 : 0)
+                             : (int64_t)batch << ((p.mb > 5 ? p.mb - 5 : 0) + p.nb - 6);
+    const int cl = T <= 152 ? (p.kb >= 9 ? 8 : p.kb == 8 ? 4 : p.kb == 7 ? 2 : 1)
+                            : T <= 304 ? (p.kb >= 8 ? 4 : p.kb == 7 ? 2 : 1) : 1;
+    if (narrow) {
+        switch (cl) {
+            case 8: return launch_gemm_f32_cluster<128, 1, 8>(p, batch, s);
+            case 4: return launch_gemm_f32_cluster<128, 1, 4>(p, batch, s);
+            case 2: return launch_gemm_f32_cluster<128, 1, 2>(p, batch, s);
+            default: return launch_gemm_f32_tiles<128, 4, 1, 4>(p, batch, s);
+        }
+    }
+    switch (cl) {
+        case 8: return launch_gemm_f32_cluster<128, 2, 8>(p, batch, s);
+        case 4: return launch_gemm_f32_cluster<128, 2, 4>(p, batch, s);
+        case 2: return launch_gemm_f32_cluster<128, 2, 2>(p, batch, s);
+        default: break;
+    }
+    return T > 304 ? launch_gemm_f32_tiles<128, 8, 2, 2>(p, batch, s) : launch_gemm_f32_tiles<128, 4, 2, 4>(p, batch, s);
 }
 
 // Grouped contractions of several networks: node i belongs to network
 // net[i]; slice z of the launch maps to slice rs0[net] + z of that network and
 // exists only for z < rb[net] (networks batch different numbers of slices).
-__global__ void __launch_bounds__(NT, 2) k_gemm_f32_group_multi(const GemmParams* __restrict__ params,
+__global__ void __launch_bounds__(GT, 4) k_gemm_f32_group_multi(const GemmParams* __restrict__ params,
                                                              const int64_t* __restrict__ tile_off, int n,
                                                              const int* __restrict__ net,
                                                              const int64_t* __restrict__ rs0,
                                                              const int* __restrict__ rb) {
     extern __shared__ __align__(16) uint8_t gemm_dyn[];
-    GemmSmem& sm = *reinterpret_cast<GemmSmem*>(gemm_dyn);
+    GroupSmem& sm = *reinterpret_cast<GroupSmem*>(gemm_dyn);
     const int64_t b = blockIdx.x;
     int lo = 0, hi = n - 1;
     while (lo < hi) {
@@ -138,7 +216,7 @@ __global__ void __launch_bounds__(NT, 2) k_gemm_f32_group_multi(const GemmParams
     }
     const int w = net[lo];
     if ((int)blockIdx.z >= rb[w]) return;
-    gemm_tile(params[lo], b - tile_off[lo], blockIdx.z, rs0[w], sm);
+    gemm_tile<0, GT, 4, 2>(params[lo], b - tile_off[lo], blockIdx.z, rs0[w], sm);
 }
 
 // Root reductions of several networks in one launch: block x serves chunk
@@ -186,9 +264,16 @@ __global__ void k_accumulate_multi(const RootParams* __restrict__ roots, double2
     }
 }
 
+bool gemm_f32_long(int kb) { return kb >= 8; }
+
+int64_t gemm_f32_group_tiles(int mb, int nb) {
+    using Cfg = TileCfg<GT, 4, 2>;
+    return (((1ll << mb) + Cfg::BM - 1) / Cfg::BM) * (((1ll << nb) + Cfg::BN - 1) / Cfg::BN);
+}
+
 int64_t gemm_f32_tiles(int mb, int nb) {
     int64_t M = 1ll << mb, N = 1ll << nb;
-    return ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
+    return ((M + 63) / 64) * ((N + 63) / 64);
 }
 
 cudaError_t launch_gemm_f32_group(const GemmParams* d_params, const int64_t* d_tile_off, int n,
@@ -197,7 +282,7 @@ cudaError_t launch_gemm_f32_group(const GemmParams* d_params, const int64_t* d_t
         return cudaErrorInvalidConfiguration;
     cudaError_t e = gemm_smem_attr();
     if (e != cudaSuccess) return e;
-    k_gemm_f32_group<<<dim3((unsigned)total_tiles, 1, batch), NT, sizeof(GemmSmem), s>>>(d_params, d_tile_off, n,
+    k_gemm_f32_group<<<dim3((unsigned)total_tiles, 1, batch), GT, sizeof(GroupSmem), s>>>(d_params, d_tile_off, n,
                                                                                        slice0);
     return cudaGetLastError();
 }
@@ -209,7 +294,7 @@ cudaError_t launch_gemm_f32_group_multi(const GemmParams* d_params, const int64_
         return cudaErrorInvalidConfiguration;
     cudaError_t e = gemm_smem_attr();
     if (e != cudaSuccess) return e;
-    k_gemm_f32_group_multi<<<dim3((unsigned)total_tiles, 1, max_batch), NT, sizeof(GemmSmem), s>>>(
+    k_gemm_f32_group_multi<<<dim3((unsigned)total_tiles, 1, max_batch), GT, sizeof(GroupSmem), s>>>(
         d_params, d_tile_off, n, d_net, d_rs0, d_rb);
     return cudaGetLastError();
 }
