@@ -62,9 +62,10 @@ __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
-__device__ __forceinline__ f32x2 swap2(f32x2 v) {
-    const float2 f = unpack2(v);
-    return pack2(f.y, f.x);
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
 }
 
 // C[m][n] = sum_k A(m,k) B(k,n), one BM x 64 tile per CTA of 256 threads, RM x 4

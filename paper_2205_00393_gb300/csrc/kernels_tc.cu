@@ -22,7 +22,8 @@
 //     so the complex tile lives in 256 TMEM columns and two such buffers
 //     alternate per 128-wide K chunk; eight epilogue warps move each chunk's
 //     Cr, Ci into FP32 registers while the tensor cores fill the other
-//     buffer, and finally write C.
+//     buffer, and finally write C. k_cgemm_pair is the same on pairs of CTAs
+//     (256 x 128 tiles, cta_group::2), for all but the smallest contractions.
 //
 // Split FP16x2 scaling: every row of A and every column of B is scaled by its
 // own power of two per 256-wide K chunk (the largest |Re|, |Im| of that row
@@ -132,34 +133,42 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
 }
 
 // Shared-memory matrix descriptor: K-major, ROWB-byte swizzle (layout type
-// 4 = 64B, 6 = 32B), 8-row groups 8*ROWB bytes apart, descriptor version 1.
+// 4 = 64B, 6 = 32B), 8-row groups 8*ROWB bytes apart, descriptor version 1. The
+// high word is a constant; the low word is linear in the address, so an MMA's
+// descriptors are one addition each from the stage's.
 template <int ROWB>
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-    d |= (uint64_t)1 << 16;                    // leading byte offset (unused for swizzled K-major)
-    d |= (uint64_t)((8 * ROWB) >> 4) << 32;    // stride byte offset
-    d |= (uint64_t)1 << 46;                    // version
-    d |= (uint64_t)(ROWB == 64 ? 4 : 6) << 61;
-    return d;
+__host__ __device__ constexpr uint32_t desc_hi() {
+    return (uint32_t)((8 * ROWB) >> 4) | (1u << 14) | ((ROWB == 64 ? 4u : 6u) << 29);
+}
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) {
+    return ((saddr >> 4) & 0x3FFFu) | (1u << 16);  // leading byte offset (unused for swizzled K-major)
 }
 
-template <int KIND>
-__device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    if constexpr (KIND != 1) {
-        asm volatile(
-            "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-            "l"(a), "l"(b), "r"(idesc), "r"(acc)
-            : "memory");
-    } else {
-        asm volatile(
-            "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-            "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-            "l"(a), "l"(b), "r"(idesc), "r"(acc)
-            : "memory");
-    }
+// one lane of a converged warp
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.b32 %0, 1, 0, p;\n}\n"
+        : "=r"(p));
+    return p != 0;
 }
+
+#define TNC_MMA(group, kind)                                                                                   \
+    asm volatile(                                                                                              \
+        "{\n.reg .pred p;\n.reg .b64 da, db;\nsetp.ne.b32 p, %5, 0;\nmov.b64 da, {%1, %3};\nmov.b64 db, {%2, %3};\n" \
+        "tcgen05.mma.cta_group::" group ".kind::" kind " [%0], da, db, %4, p;\n}\n" ::"r"(d_tmem),           \
+        "r"(a), "r"(b), "r"(hi), "r"(idesc), "r"(acc)                                                          \
+        : "memory")
+
+// D (+)= A B over 32 bytes of K; a, b: low descriptor words, hi: the common high word
+template <int KIND, int GROUP>
+__device__ __forceinline__ void mma(uint32_t d_tmem, uint32_t a, uint32_t b, uint32_t hi, uint32_t idesc, uint32_t acc) {
+    if constexpr (GROUP == 1 && KIND != 1) TNC_MMA("1", "f16");
+    else if constexpr (GROUP == 1) TNC_MMA("1", "tf32");
+    else if constexpr (KIND != 1) TNC_MMA("2", "f16");
+    else TNC_MMA("2", "tf32");
+}
+#undef TNC_MMA
 
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
@@ -168,16 +177,11 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// 16 consecutive 32-bit TMEM columns of this warp's 32 lanes (one per lane)
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+// 8 consecutive 32-bit TMEM columns of this warp's 32 lanes (one per lane)
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
 }
 
 // Instruction descriptor: FP32 accumulator (bit 4), A/B format at bits 7 and
@@ -194,9 +198,26 @@ __host__ __device__ constexpr uint32_t instr_desc(bool negate_a) {
            ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
 }
 
-// Part pairs, smallest magnitudes first.
-__constant__ int kPairsBF16[6][2] = {{1, 1}, {0, 2}, {2, 0}, {0, 1}, {1, 0}, {0, 0}};
-__constant__ int kPairs2[3][2] = {{0, 1}, {1, 0}, {0, 0}};
+// the pair's: M = 256 over two CTAs
+template <int KIND>
+__host__ __device__ constexpr uint32_t pair_desc(bool negate_a) {
+    return (instr_desc<KIND>(negate_a) & ~(31u << 24)) | ((uint32_t)(2 * TM >> 4) << 24);
+}
+
+// Part pairs (of A, of B), smallest magnitudes first.
+template <int KIND>
+__host__ __device__ constexpr int part_a(int q) {
+    return KIND == 0 ? (q == 2 ? 2 : (q == 0 || q == 4) ? 1 : 0) : (q == 1 ? 1 : 0);
+}
+template <int KIND>
+__host__ __device__ constexpr int part_b(int q) {
+    return KIND == 0 ? (q == 1 ? 2 : (q == 0 || q == 3) ? 1 : 0) : (q == 0 ? 1 : 0);
+}
+static_assert(part_a<0>(0) == 1 && part_b<0>(0) == 1 && part_a<0>(1) == 0 && part_b<0>(1) == 2 && part_a<0>(2) == 2 &&
+                  part_b<0>(2) == 0 && part_a<0>(3) == 0 && part_b<0>(3) == 1 && part_a<0>(4) == 1 && part_b<0>(4) == 0 &&
+                  part_a<0>(5) == 0 && part_b<0>(5) == 0 && part_a<1>(0) == 0 && part_b<1>(0) == 1 && part_a<1>(1) == 1 &&
+                  part_b<1>(1) == 0 && part_a<1>(2) == 0 && part_b<1>(2) == 0,
+              "(1,1) (0,2) (2,0) (0,1) (1,0) (0,0); (0,1) (1,0) (0,0)");
 
 // K is processed in chunks of KD_ELEMS. Each chunk accumulates in one of two
 // TMEM buffers of 256 columns (Cr in the first 128, Ci in the last 128); when
@@ -213,12 +234,62 @@ constexpr int EPI_LDW = 66;    // float2 per row of a warp's staged 32 x 64 outp
 static_assert(EPI_WARPS * 32 * EPI_LDW * 8 <= SMEM_PIPE, "staged epilogue fits the pipeline ring");
 constexpr int PRODUCER_WARP = 8, MMA_WARP = 9, NTHREADS = 320;
 
+using f32dev::add2;
+using f32dev::f32x2;
+using f32dev::fma2;
+using f32dev::pack2;
+using f32dev::unpack2;
+
+// Adds a chunk's accumulators (this warp's 32 rows x 64 complex columns at
+// taddr, Ci TN columns further) to the FP32 sums, 8 columns at a time by packed
+// operations. Split FP16x2 undoes the scales first: sa of this lane's row, then
+// the column's factor in the same FMA as the addition (both are powers of two,
+// so every product is exact). The drain takes 128 packed operations a lane
+// instead of 384 scalar ones.
+template <int KIND>
+__device__ __forceinline__ void drain_chunk(uint32_t taddr, float sa, const float* colf, f32x2 (&cr)[32], f32x2 (&ci)[32]) {
+    const f32x2 sa2 = pack2(sa, sa);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        uint32_t re[8], im[8];
+        tmem_ld8(taddr + 8 * q, re);
+        tmem_ld8(taddr + TN + 8 * q, im);
+        f32x2 f[4];
+        if constexpr (KIND == 3) {
+            const ulonglong2* t = reinterpret_cast<const ulonglong2*>(colf + 8 * q);
+            f[0] = t[0].x;
+            f[1] = t[0].y;
+            f[2] = t[1].x;
+            f[3] = t[1].y;
+        }
+        tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const f32x2 r = pack2(__uint_as_float(re[2 * j]), __uint_as_float(re[2 * j + 1]));
+            const f32x2 i = pack2(__uint_as_float(im[2 * j]), __uint_as_float(im[2 * j + 1]));
+            if constexpr (KIND == 3) {
+                cr[4 * q + j] = fma2(f32dev::mul2(r, sa2), f[j], cr[4 * q + j]);
+                ci[4 * q + j] = fma2(f32dev::mul2(i, sa2), f[j], ci[4 * q + j]);
+            } else {
+                cr[4 * q + j] = add2(cr[4 * q + j], r);
+                ci[4 * q + j] = add2(ci[4 * q + j], i);
+            }
+        }
+    }
+}
+
+// two adjacent complex columns as they are stored
+__device__ __forceinline__ float4 complex_pair(f32x2 re, f32x2 im) {
+    const float2 r = unpack2(re), i = unpack2(im);
+    return make_float4(r.x, i.x, r.y, i.y);
+}
+
 // Shared-memory state of one CTA's tensor-core pipeline.
 struct TcShared {
     uint64_t full_bar[8], empty_bar[8], tfull[2], tfree[2], drain_bar;
     uint32_t tmem_base;
     int abort;
-    float colscale[EPI_WARPS][64];  // split FP16x2: per-warp column factors of a chunk
+    alignas(16) float colscale[EPI_WARPS][64];  // split FP16x2: per-warp column factors of a chunk
 };
 
 // k-blocks and TMEM chunks a CTA's tensor-core roles have processed so far:
@@ -227,6 +298,35 @@ struct TcShared {
 struct TcPipe {
     uint32_t it = 0, ch = 0;
 };
+
+// The MMAs of one stage: for every part pair and 32 bytes of K, the four real
+// products of the complex tile (Cr at d, Ci at d + TN). A's planes start at sa
+// (part tiles of 128 ROWB bytes), B's a_bytes further (part tiles of b_tile
+// bytes). more: the chunk's accumulator already holds a stage.
+template <int KIND, int ROWB, int GROUP>
+__device__ __forceinline__ void issue_stage(uint32_t sa, int a_bytes, int b_tile, uint32_t d, bool more, uint32_t idesc,
+                                            uint32_t idesc_neg) {
+    using C_ = Cfg<KIND, ROWB>;
+    constexpr uint32_t hi = desc_hi<ROWB>();
+    const uint32_t la = desc_lo(sa), lb = desc_lo(sa + a_bytes);
+    const uint32_t dr = d, di = d + TN;
+#pragma unroll
+    for (int q = 0; q < C_::NPAIRS; ++q) {
+        const int pa = part_a<KIND>(q), pb = part_b<KIND>(q);
+#pragma unroll
+        for (int j = 0; j < C_::KSTEPS; ++j) {  // MMAs of 32 bytes of K per swizzle row
+            const uint32_t ar = la + ((pa * C_::PART_TILE + j * 32) >> 4);
+            const uint32_t ai = la + (((C_::PARTS + pa) * C_::PART_TILE + j * 32) >> 4);
+            const uint32_t br = lb + ((pb * b_tile + j * 32) >> 4);
+            const uint32_t bi = lb + (((C_::PARTS + pb) * b_tile + j * 32) >> 4);
+            const uint32_t acc = (more || q > 0 || j > 0) ? 1u : 0u;
+            mma<KIND, GROUP>(dr, ar, br, hi, idesc, acc);
+            mma<KIND, GROUP>(dr, ai, bi, hi, idesc_neg, 1u);
+            mma<KIND, GROUP>(di, ar, bi, hi, idesc, acc);
+            mma<KIND, GROUP>(di, ai, br, hi, idesc, 1u);
+        }
+    }
+}
 
 // thread 0, before the CTA-wide barrier that precedes the first tile
 __device__ __forceinline__ void tc_init(TcShared& sh) {
@@ -309,63 +409,51 @@ __device__ __forceinline__ void tc_tile(const CUtensorMap* tmA, const CUtensorMa
                 }
             }
         }
-    } else if (warp == MMA_WARP && lane == 0) {
-        // ---------------- MMA issuer
+    } else if (warp == MMA_WARP) {
+        // ---------------- MMA issuer: the whole warp waits and computes the descriptors, one
+        // elected lane issues. With the loop in a single lane the descriptors went from
+        // vector to uniform registers before every MMA, and issuing took longer than the
+        // MMAs themselves: about 960 clocks a k-block on top of their 1536 (FP16x2).
         constexpr uint32_t idesc = instr_desc<KIND>(false), idesc_neg = instr_desc<KIND>(true);
         bool any = false;
-        for (int it = 0; it < nkb && !*abort_flag; ++it) {
+        for (int it = 0; it < nkb; ++it) {
             const uint32_t g = pipe.it + it;
             const int s = g % C_::STAGES;
             const uint32_t ph = (g / C_::STAGES) & 1u;
             const int kbi = it % kpc;
             const uint32_t cgl = pipe.ch + it / kpc;  // chunk over all tiles of this CTA
             const int buf = cgl & 1;
-            if ((kbi == 0 && cgl >= 2 &&
-                 !mbar_wait(smem_u32(&sh.tfree[buf]), ((cgl - 2) >> 1) & 1u, abort_flag, spin)) ||
-                !mbar_wait(smem_u32(&sh.full_bar[s]), ph, abort_flag, spin)) {
+            const bool ready = !*abort_flag &&
+                               (kbi != 0 || cgl < 2 ||
+                                mbar_wait(smem_u32(&sh.tfree[buf]), ((cgl - 2) >> 1) & 1u, abort_flag, spin)) &&
+                               mbar_wait(smem_u32(&sh.full_bar[s]), ph, abort_flag, spin);
+            if (!__all_sync(0xffffffffu, ready)) {
                 sh.abort = 1;
                 atomicExch(p.err, kErrTimeout);
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t sa = smem_u32(smem + s * C_::STAGE_BYTES);
-            const uint32_t sb = sa + C_::OP_BYTES;
-            const uint32_t dr = tmem + (uint32_t)(buf * 2 * TN), di = dr + TN;
-#pragma unroll
-            for (int q = 0; q < C_::NPAIRS; ++q) {
-                const int pa = KIND == 0 ? kPairsBF16[q][0] : kPairs2[q][0];
-                const int pb = KIND == 0 ? kPairsBF16[q][1] : kPairs2[q][1];
-#pragma unroll
-                for (int j = 0; j < C_::KSTEPS; ++j) {  // MMAs of 32 bytes of K per swizzle row
-                    const uint64_t ar = smem_desc<ROWB>(sa + pa * PT + j * 32);
-                    const uint64_t ai = smem_desc<ROWB>(sa + (C_::PARTS + pa) * PT + j * 32);
-                    const uint64_t br = smem_desc<ROWB>(sb + pb * PT + j * 32);
-                    const uint64_t bi = smem_desc<ROWB>(sb + (C_::PARTS + pb) * PT + j * 32);
-                    const uint32_t acc = (kbi > 0 || q > 0 || j > 0) ? 1u : 0u;
-                    mma<KIND>(dr, ar, br, idesc, acc);
-                    mma<KIND>(dr, ai, bi, idesc_neg, 1u);
-                    mma<KIND>(di, ar, bi, idesc, acc);
-                    mma<KIND>(di, ai, br, idesc, 1u);
-                }
+            if (elect_one()) {
+                issue_stage<KIND, ROWB, 1>(smem_u32(smem + s * C_::STAGE_BYTES), C_::OP_BYTES, C_::PART_TILE,
+                                           tmem + (uint32_t)(buf * 2 * TN), kbi > 0, idesc, idesc_neg);
+                mma_commit(smem_u32(&sh.empty_bar[s]));
+                if (kbi == kpc - 1) mma_commit(smem_u32(&sh.tfull[buf]));
             }
             any = true;
-            mma_commit(smem_u32(&sh.empty_bar[s]));
-            if (kbi == kpc - 1) mma_commit(smem_u32(&sh.tfull[buf]));
+            __syncwarp();
         }
-        if (*abort_flag && any) {
+        if (*abort_flag && any && elect_one()) {
             mma_commit(smem_u32(&sh.drain_bar));
             for (uint32_t i = 0; i < spin && !mbar_try(smem_u32(&sh.drain_bar), 0); ++i) {
             }
         }
+        __syncwarp();
     } else if (warp < EPI_WARPS) {
         // ---------------- epilogue: chunk sums TMEM -> FP32 registers -> C
         const int g = warp & 3, h = warp >> 2;
-        float cr[64], ci[64];
+        f32x2 cr[32], ci[32];  // pairs of adjacent columns
 #pragma unroll
-        for (int j = 0; j < 64; ++j) {
-            cr[j] = 0.f;
-            ci[j] = 0.f;
-        }
+        for (int j = 0; j < 32; ++j) cr[j] = ci[j] = 0;
         // split FP16x2: per-chunk scale exponents of this lane's row and of the warp's 64 columns;
         // the columns' factors 2^-e go through a warp-private table in shared memory
         const int64_t sk = K < KC_ELEMS ? K : KC_ELEMS;  // K per scale chunk
@@ -399,23 +487,7 @@ __device__ __forceinline__ void tc_tile(const CUtensorMap* tmA, const CUtensorMa
                 colf[2 * lane + 1] = pow2f(-(int)e2.y);
                 __syncwarp();
             }
-            const uint32_t tbase = tmem + ((uint32_t)(32 * g) << 16) + (uint32_t)(buf * 2 * TN + 64 * h);
-#pragma unroll
-            for (int q4 = 0; q4 < 4; ++q4) {                // 16 columns at a time
-#pragma unroll
-                for (int part = 0; part < 2; ++part) {      // 0: Cr columns, 1: Ci columns
-                    float v[16];
-                    tmem_ld16(tbase + (uint32_t)(part * TN + 16 * q4), v);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        float x = v[j];
-                        if constexpr (KIND == 3) x = x * sa * colf[16 * q4 + j];
-                        if (part == 0) cr[16 * q4 + j] += x;
-                        else ci[16 * q4 + j] += x;
-                    }
-                }
-            }
+            drain_chunk<KIND>(tmem + ((uint32_t)(32 * g) << 16) + (uint32_t)(buf * 2 * TN + 64 * h), sa, colf, cr, ci);
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&sh.tfree[buf]));
@@ -431,8 +503,7 @@ __device__ __forceinline__ void tc_tile(const CUtensorMap* tmA, const CUtensorMa
             // with coalesced 16-byte stores.
             float2* stg = reinterpret_cast<float2*>(smem) + (size_t)warp * 32 * EPI_LDW;
 #pragma unroll
-            for (int j = 0; j < 64; j += 2)
-                reinterpret_cast<float4*>(stg + lane * EPI_LDW + j)[0] = make_float4(cr[j], ci[j], cr[j + 1], ci[j + 1]);
+            for (int j = 0; j < 32; ++j) reinterpret_cast<float4*>(stg + lane * EPI_LDW + 2 * j)[0] = complex_pair(cr[j], ci[j]);
             __syncwarp();
             const int64_t ld = p.ksplit_bits ? N : (p.c_ld ? p.c_ld : N);
             float2* cb = p.ksplit_bits ? p.partial + ((int64_t)ky * nbatch + z) * (N << p.mb)
@@ -486,6 +557,312 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         __syncwarp();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+    }
+}
+
+// ------------------------------------------------------------ CTA-pair GEMM
+//
+// k_cgemm_pair computes the same tiles two at a time: a cluster of two CTAs
+// shares a 256 x 128 complex tile, and every MMA (cta_group::2, M = 256, N = 128)
+// spans both SMs. What bounds the one-CTA kernel is shared memory: a 128 x 128 x 16
+// MMA reads 8 KB of operands in its 64 clocks, the full 128 bytes per clock that
+// an SM's shared memory delivers, and the TMA fill (41 bytes per clock at full rate
+// for FP16x2) comes on top. A pair holds half of B per SM: 6 KB of operands per 64
+// clocks and SM, and 48 KB instead of 64 KB of fill per k-block.
+//
+// The kernel is persistent: one pair per two SMs walks over the tiles (and K
+// splits and batch entries), and the producer and the MMA issuer run ahead into
+// the next tile while the epilogue warps write the last one, whose staging has
+// shared memory of its own.
+//
+// Measured on (M, N, K) = (2^14, 2^12, 2^12), split FP16x2: 3.45-3.54 ms = 1862-1914
+// TFLOP/s, tensor pipe 93% at 1.66 GHz under the power cap, against 3.99 ms (one-CTA
+// tiles) and 4.34 ms (those before the issuing warp kept its descriptors in uniform
+// registers, below); split BF16 6.18 ms (tensor pipe 98%) against 6.91 and 7.10, split
+// TF32 5.95 ms (1109 TFLOP/s) against 7.31 and 8.15.
+template <int KIND, int ROWB> struct PairCfg : Cfg<KIND, ROWB> {
+    using C_ = Cfg<KIND, ROWB>;
+    static constexpr int A_BYTES = C_::PLANES * 128 * ROWB, B_BYTES = C_::PLANES * 64 * ROWB;
+    static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;  // of one CTA
+    static constexpr int STAGES = SMEM_PIPE / STAGE_BYTES > 8 ? 8 : SMEM_PIPE / STAGE_BYTES;
+    static constexpr int STG_LD = 5;                        // 16-byte units per staged row of 8 complex values
+    static constexpr int STG_BYTES = EPI_WARPS * 32 * STG_LD * 16;
+    static constexpr int SMEM = STAGES * STAGE_BYTES + STG_BYTES + 1024;
+    static_assert(STAGES >= 2 && SMEM + (int)sizeof(TcShared) <= 227 * 1024, "shared memory");
+};
+
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+
+// arrive on a barrier of any CTA of the cluster (address from mapa)
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+// As mbar_wait, acquiring what CTAs of the cluster released.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint32_t limit) {
+    for (uint32_t i = 0; i < limit; ++i) {
+        uint32_t ok;
+        asm volatile(
+            "{\n.reg .pred p;\n"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+            "selp.b32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (ok) return true;
+        if ((i & 255) == 255 && *abort_flag) return false;
+    }
+    return false;
+}
+
+// load into this CTA's shared memory, completing on a barrier of the pair
+__device__ __forceinline__ void tma_load_pair(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
+                                              uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
+        : "memory");
+}
+
+// completion of the MMAs issued so far, on this barrier of both CTAs
+__device__ __forceinline__ void mma_commit_pair(uint32_t bar) {
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+        "h"((uint16_t)3)
+        : "memory");
+}
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Work item of the pair kernel: an output tile of a K split of a batch entry.
+struct PairItem {
+    int m0, n0, ky, z;  // m0: the pair's first row
+};
+__device__ __forceinline__ PairItem pair_item(const TcGemmParams& p, int64_t item) {
+    const int GROUP_M = p.group_m < 1 ? 1 : p.group_m;
+    const int64_t tiles_n = 1ll << (p.nb - 7), tiles_m = 1ll << (p.mb - 8), tiles = tiles_m * tiles_n;
+    const int64_t cta = item % tiles, rest = item / tiles;
+    const int64_t per_group = (int64_t)GROUP_M * tiles_n;
+    const int64_t grp = cta / per_group, in_grp = cta % per_group;
+    const int64_t gm = (tiles_m - grp * GROUP_M) < GROUP_M ? (tiles_m - grp * GROUP_M) : GROUP_M;
+    PairItem it;
+    it.m0 = (int)((grp * GROUP_M + in_grp % gm) * 2 * TM);
+    it.n0 = (int)((in_grp / gm) * TN);
+    it.ky = (int)(rest & ((1 << p.ksplit_bits) - 1));
+    it.z = (int)(rest >> p.ksplit_bits);
+    return it;
+}
+
+template <int KIND, int ROWB>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
+    k_cgemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                 const __grid_constant__ TcGemmParams p, int nbatch) {
+    using C_ = PairCfg<KIND, ROWB>;
+    extern __shared__ __align__(1024) uint8_t dsmem[];
+    __shared__ TcShared sh;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dsmem) + 1023) & ~uintptr_t(1023));
+    const uint32_t rank = blockIdx.x & 1;  // of the CTA in its pair
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < C_::STAGES; ++s) {
+            mbar_init(smem_u32(&sh.full_bar[s]), 1);
+            mbar_init(smem_u32(&sh.empty_bar[s]), 1);
+        }
+        for (int t = 0; t < 2; ++t) {
+            mbar_init(smem_u32(&sh.tfull[t]), 1);
+            mbar_init(smem_u32(&sh.tfree[t]), 2 * EPI_WARPS);  // used in CTA 0: both CTAs' epilogue warps
+        }
+        mbar_init(smem_u32(&sh.drain_bar), 1);
+        sh.abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == MMA_WARP) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem_base)),
+                     "r"(512u)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    cluster_sync();  // both CTAs' barriers are initialised
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = sh.tmem_base;
+
+    const int64_t M = 1ll << p.mb, N = 1ll << p.nb, K = 1ll << p.kb;
+    const int64_t items = ((int64_t)nbatch << p.ksplit_bits) << (p.mb - 8 + p.nb - 7);
+    const int64_t first = blockIdx.x >> 1, stride = gridDim.x >> 1;
+    const int nkb = (int)((K >> p.ksplit_bits) / C_::BK);               // k-blocks of one item
+    const int kpc = nkb < KD_ELEMS / C_::BK ? nkb : KD_ELEMS / C_::BK;  // k-blocks per chunk
+    const int nchunks = nkb / kpc;
+    volatile int* abort_flag = &sh.abort;
+    const uint32_t spin = p.spin_limit ? p.spin_limit : kSpinLimit;
+    auto give_up = [&]() {  // stop this CTA's roles and the peer's
+        sh.abort = 1;
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(mapa(smem_u32(&sh.abort), rank ^ 1u)), "r"(1) : "memory");
+        atomicExch(p.err, kErrTimeout);
+    };
+
+    if (warp == PRODUCER_WARP && lane == 0) {
+        // ---------------- TMA producer of this CTA: its 128 rows of A, its 64 rows of B, on CTA 0's barrier
+        asm volatile("fence.proxy.async.global;" ::: "memory");  // planes written by generic stores
+        uint32_t g = 0;                                          // k-blocks issued over all items
+        bool ok = true;
+        for (int64_t item = first; item < items && ok && !p.test_stall; item += stride) {
+            const PairItem w = pair_item(p, item);
+            const int za = p.a_shared ? 0 : w.z, zb = p.b_shared ? 0 : w.z;
+            const int m0 = w.m0 + TM * (int)rank, n0 = w.n0 + 64 * (int)rank;
+            for (int it = 0; it < nkb; ++it, ++g) {
+                const int s = g % C_::STAGES;
+                const uint32_t ph = (g / C_::STAGES) & 1u;
+                if (!mbar_wait_cluster(smem_u32(&sh.empty_bar[s]), ph ^ 1u, abort_flag, spin)) {
+                    give_up();
+                    ok = false;
+                    break;
+                }
+                const uint32_t sa = smem_u32(smem + s * C_::STAGE_BYTES);
+                if (rank == 0) mbar_expect_tx(smem_u32(&sh.full_bar[s]), 2 * C_::STAGE_BYTES);
+                const uint32_t fb = mapa(smem_u32(&sh.full_bar[s]), 0);
+                tma_load_pair(sa, &tmA, (it + w.ky * nkb) * C_::BK, m0, 0, za, fb);
+                tma_load_pair(sa + C_::A_BYTES, &tmB, (it + w.ky * nkb) * C_::BK, n0, 0, zb, fb);
+            }
+        }
+        if (*abort_flag) {
+            // drain: a millisecond for the loads still in flight (they take microseconds), then,
+            // in CTA 0, wait (bounded) on the barriers that its own and CTA 1's loads complete on
+            for (int i = 0; i < 50; ++i) __nanosleep(20000);
+            for (uint32_t h = g > (uint32_t)C_::STAGES ? g - C_::STAGES : 0; h < g && rank == 0; ++h)
+                for (uint32_t i = 0; i < spin && !mbar_try(smem_u32(&sh.full_bar[h % C_::STAGES]), (h / C_::STAGES) & 1u); ++i) {
+                }
+        }
+    } else if (warp == MMA_WARP && rank == 0) {
+        // ---------------- MMA issuer of the pair (as in tc_tile)
+        constexpr uint32_t idesc = pair_desc<KIND>(false), idesc_neg = pair_desc<KIND>(true);
+        uint32_t g = 0, cgl = 0;                        // k-blocks and chunks over all items
+        bool any = false, ok = true;
+        for (int64_t item = first; item < items && ok; item += stride)
+            for (int it = 0; it < nkb; ++it, ++g) {
+                const int s = g % C_::STAGES;
+                const uint32_t ph = (g / C_::STAGES) & 1u;
+                const int kbi = it % kpc, buf = cgl & 1;
+                const bool ready = !*abort_flag &&
+                                   (kbi != 0 || cgl < 2 ||
+                                    mbar_wait_cluster(smem_u32(&sh.tfree[buf]), ((cgl - 2) >> 1) & 1u, abort_flag, spin)) &&
+                                   mbar_wait_cluster(smem_u32(&sh.full_bar[s]), ph, abort_flag, spin);
+                if (!__all_sync(0xffffffffu, ready)) {
+                    if (lane == 0) give_up();
+                    ok = false;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (elect_one()) {
+                    issue_stage<KIND, ROWB, 2>(smem_u32(smem + s * C_::STAGE_BYTES), C_::A_BYTES, 64 * ROWB,
+                                               tmem + (uint32_t)(buf * 2 * TN), kbi > 0, idesc, idesc_neg);
+                    mma_commit_pair(smem_u32(&sh.empty_bar[s]));
+                    if (kbi == kpc - 1) mma_commit_pair(smem_u32(&sh.tfull[buf]));
+                }
+                any = true;
+                __syncwarp();
+                if (kbi == kpc - 1) ++cgl;
+            }
+        if (*abort_flag && any && elect_one()) {
+            mma_commit_pair(smem_u32(&sh.drain_bar));
+            for (uint32_t i = 0; i < spin && !mbar_try(smem_u32(&sh.drain_bar), 0); ++i) {
+            }
+        }
+        __syncwarp();
+    } else if (warp < EPI_WARPS) {
+        // ---------------- epilogue of this CTA's 128 rows: chunk sums TMEM -> FP32 registers -> C
+        const int gq = warp & 3, h = warp >> 2;
+        uint8_t* stg = smem + C_::STAGES * C_::STAGE_BYTES + warp * 32 * C_::STG_LD * 16;
+        float* colf = sh.colscale[warp];
+        const int64_t sk = K < KC_ELEMS ? K : KC_ELEMS;  // K per scale chunk
+        const int64_t nch = K / sk;                       // scale chunks over the whole K of the planes
+        const uint32_t tfree0[2] = {mapa(smem_u32(&sh.tfree[0]), 0), mapa(smem_u32(&sh.tfree[1]), 0)};
+        uint32_t cgl = 0;
+        bool ok = true;
+        for (int64_t item = first; item < items && ok; item += stride) {
+            const PairItem w = pair_item(p, item);
+            const int m0 = w.m0 + TM * (int)rank;
+            f32x2 cr[32], ci[32];  // pairs of adjacent columns
+#pragma unroll
+            for (int j = 0; j < 32; ++j) cr[j] = ci[j] = 0;
+            const int8_t* ea_row = nullptr;
+            const int8_t* eb_col = nullptr;
+            if constexpr (KIND == 3) {
+                ea_row = p.sexp_a + (int64_t)(p.a_shared ? 0 : w.z) * nch * M + m0 + 32 * gq + lane;
+                eb_col = p.sexp_b + (int64_t)(p.b_shared ? 0 : w.z) * nch * N + w.n0 + 64 * h;
+            }
+            for (int c = 0; c < nchunks; ++c, ++cgl) {
+                const int buf = cgl & 1;
+                // scale chunk of this TMEM chunk; its factors are loaded before the wait
+                const int64_t cg = ((int64_t)w.ky * nchunks + c) * (kpc * C_::BK) / sk;
+                float sa = 1.f;
+                char2 e2 = make_char2(0, 0);
+                if constexpr (KIND == 3) {
+                    sa = pow2f(-(int)ea_row[cg * M]);
+                    e2 = reinterpret_cast<const char2*>(eb_col + cg * N)[lane];
+                }
+                int got = 0;
+                if (lane == 0) got = mbar_wait_cluster(smem_u32(&sh.tfull[buf]), (cgl >> 1) & 1u, abort_flag, spin) ? 1 : 0;
+                got = __shfl_sync(0xffffffffu, got, 0);
+                if (!got) {
+                    if (lane == 0) give_up();
+                    ok = false;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if constexpr (KIND == 3) {
+                    colf[2 * lane] = pow2f(-(int)e2.x);
+                    colf[2 * lane + 1] = pow2f(-(int)e2.y);
+                    __syncwarp();
+                }
+                drain_chunk<KIND>(tmem + ((uint32_t)(32 * gq) << 16) + (uint32_t)(buf * 2 * TN + 64 * h), sa, colf, cr, ci);
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(tfree0[buf]);
+            }
+            if (!ok) break;
+            // 8 columns at a time through this warp's staging: rows leave in 64-byte pieces
+            const int64_t ld = p.ksplit_bits ? N : (p.c_ld ? p.c_ld : N);
+            float2* cb = p.ksplit_bits ? p.partial + ((int64_t)w.ky * nbatch + w.z) * (N << p.mb)
+                                       : p.C + (int64_t)w.z * p.c_batch_stride;
+            float2* cbase = cb + (int64_t)(m0 + 32 * gq) * ld + w.n0 + 64 * h;
+#pragma unroll
+            for (int c8 = 0; c8 < 8; ++c8) {
+                float4* own = reinterpret_cast<float4*>(stg) + lane * C_::STG_LD;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) own[u] = complex_pair(cr[4 * c8 + u], ci[4 * c8 + u]);
+                __syncwarp();
+#pragma unroll
+                for (int r4 = 0; r4 < 4; ++r4) {
+                    const int r = 8 * r4 + (lane >> 2);
+                    float4 v = reinterpret_cast<const float4*>(stg)[r * C_::STG_LD + (lane & 3)];
+                    float4* dst = reinterpret_cast<float4*>(cbase + (int64_t)r * ld + 8 * c8) + (lane & 3);
+                    if (p.accumulate) {
+                        const float4 o = *dst;
+                        v = make_float4(o.x + v.x, o.y + v.y, o.z + v.z, o.w + v.w);
+                    }
+                    *dst = v;
+                }
+                __syncwarp();
+            }
+        }
+    }
+    __syncwarp();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    cluster_sync();  // the peer's MMAs, loads and arrivals on this CTA's shared memory are done
+    if (warp == MMA_WARP) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
     }
 }
 
@@ -870,9 +1247,9 @@ EncodeFn encoder() {
     return fn;
 }
 
-// 4D map over planes [batch][PLANES][rows][K]; box = (BK, 128 rows, PLANES, 1).
+// 4D map over planes [batch][PLANES][rows][K]; box = (BK, box_rows, PLANES, 1).
 template <int KIND, int ROWB>
-bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int batch) {
+bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int batch, unsigned box_rows = 128u) {
     using C_ = Cfg<KIND, ROWB>;
     EncodeFn enc = encoder();
     if (!enc) return false;
@@ -880,7 +1257,7 @@ bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int b
     cuuint64_t dims[4] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)Q, (cuuint64_t)batch};
     cuuint64_t strides[3] = {(cuuint64_t)(K * C_::ELEM), (cuuint64_t)(rows * K * C_::ELEM),
                              (cuuint64_t)(Q * rows * K * C_::ELEM)};
-    cuuint32_t box[4] = {(cuuint32_t)C_::BK, 128u, (cuuint32_t)Q, 1u};  // BK * ELEM = ROWB bytes
+    cuuint32_t box[4] = {(cuuint32_t)C_::BK, box_rows, (cuuint32_t)Q, 1u};  // BK * ELEM = ROWB bytes
     cuuint32_t estr[4] = {1, 1, 1, 1};
     const CUtensorMapDataType dt = KIND == 1   ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                    : KIND == 3 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
@@ -916,8 +1293,39 @@ cudaError_t launch_tc_impl(const TcGemmParams& p, const void* planesA, const voi
     return cudaGetLastError();
 }
 
+template <int KIND, int ROWB>
+cudaError_t launch_pair_impl(const TcGemmParams& p, const void* planesA, const void* planesB, int batch, cudaStream_t s) {
+    using C_ = PairCfg<KIND, ROWB>;
+    const int64_t M = 1ll << p.mb, N = 1ll << p.nb, K = 1ll << p.kb;
+    CUtensorMap ta, tb;
+    if (!make_map<KIND, ROWB>(&ta, planesA, M, K, batch) || !make_map<KIND, ROWB>(&tb, planesB, N, K, batch, 64u))
+        return cudaErrorInvalidValue;
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(k_cgemm_pair<KIND, ROWB>, cudaFuncAttributeMaxDynamicSharedMemorySize, C_::SMEM);
+    if (attr != cudaSuccess) return attr;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int64_t kcta = K >> p.ksplit_bits;  // K of one item: whole k-blocks, whole chunks
+    if (kcta < C_::BK || (kcta > KC_ELEMS && kcta % KC_ELEMS) || (p.ksplit_bits && (!p.partial || p.accumulate)))
+        return cudaErrorInvalidValue;
+    const int64_t items = ((int64_t)batch << p.ksplit_bits) << (p.mb - 8 + p.nb - 7);
+    const int64_t pairs = items < sms / 2 ? items : sms / 2;
+    k_cgemm_pair<KIND, ROWB><<<dim3((unsigned)(2 * pairs)), NTHREADS, C_::SMEM, s>>>(ta, tb, p, batch);
+    return cudaGetLastError();
+}
+
+// Pairs from one item per two SMs on, or for K of at least 1024 per item: below
+// both, the cluster's longer start is not made up for ((M, N, K) = (2^11, 2^10, 2^7),
+// 64 items, FP16x2: 18.4 us on pairs, 16.3 on single CTAs; (2^9, 2^8, 2^10), 2 items:
+// 38.9 against 44.9; (2^12, 2^11, 2^7), 256 items: 40.9 against 47.3). Either gives
+// the same bits.
 template <int KIND>
 cudaError_t launch_tc_rows(const TcGemmParams& p, const void* pa, const void* pb, int batch, cudaStream_t s) {
+    const int64_t items = p.mb < 8 ? 0 : ((int64_t)batch << p.ksplit_bits) << (p.mb - 8 + p.nb - 7);
+    if (items >= 76 || (items && p.kb - p.ksplit_bits >= 10))
+        return p.row_bytes == 32 ? launch_pair_impl<KIND, 32>(p, pa, pb, batch, s) : launch_pair_impl<KIND, 64>(p, pa, pb, batch, s);
     if (p.row_bytes == 32) return launch_tc_impl<KIND, 32>(p, pa, pb, batch, s);
     return launch_tc_impl<KIND, 64>(p, pa, pb, batch, s);
 }
