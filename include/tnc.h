@@ -328,10 +328,9 @@ tnc_status tnc_worklist_many_json(int n, const tnc_net_t* nets, int64_t batch, i
  *                  launch when every tensor of the sub-path, without the stem
  *                  modes that live through all of its steps, fits 2^value
  *                  elements: one CTA per assignment of those long-lived modes
- *                  keeps its sub-tensor in shared memory across the steps
- *                  (a group with a step whose contracted and new elements
- *                  differ holds two buffers and stays within 2^min(value, 12)
- *                  elements). A narrow step that starts no longer group runs
+ *                  keeps its sub-tensor on chip across the steps (groups
+ *                  stay within 2^min(value, 12) elements, which is faster
+ *                  than 2^13). A narrow step that starts no longer group runs
  *                  alone in the same kernel. 0 turns fusion off: every
  *                  contraction then runs on the GEMM kernels
  *                  (tnc_contract_many never fuses)

@@ -131,6 +131,7 @@ struct GroupPlan {
     std::vector<tnc::GemmParams> params;
     std::vector<int64_t> tile_off;
     std::vector<tnc::StemParams> stem_params;  // per Plan::stems entry (device copy in d_stem)
+    std::vector<std::unique_ptr<tnc::StemRegParams>> stem_reg;  // the groups that run in registers (else null)
 };
 
 // Device copy of a work list: one allocation holding the tables, the initial
@@ -212,6 +213,8 @@ struct tnc_net {
     bool in_many = false;        // building a many-network call: no fused stem groups
     tnc::StemParams* d_stem = nullptr;
     size_t d_stem_cap = 0;
+    tnc::StemRegBranches* d_stem_reg = nullptr;  // per Plan::stems entry
+    size_t d_stem_reg_cap = 0;
     bool cache_invariants = false;  // keep slice-invariant inputs of per-slice nodes across calls
     std::string inv_key;            // state under which the cached invariants were computed
     uint64_t leaf_version = 0;      // bumped whenever leaf data changes
@@ -251,6 +254,7 @@ struct tnc_net {
         if (d_tile_off) cudaFree(d_tile_off);
         if (d_pg) cudaFree(d_pg);
         if (d_stem) cudaFree(d_stem);
+        if (d_stem_reg) cudaFree(d_stem_reg);
         if (ws_own) cudaFree(ws_own);
         if (d_prof) cudaFree(d_prof);
         if (d_var) cudaFree(d_var);

@@ -172,7 +172,12 @@ bool stem_step(const tnc_net* net, const NodePlan& np) {
            (int)net->plan.layout[np.A].size() > net->stem_cap_log2;
 }
 
-constexpr int kStemTwoBufferCap = 12;
+// Groups stay within 2^12 elements whatever the cap: four CTAs of 128 threads
+// share an SM, and their phases (loads, products, exchanges) overlap better
+// than those of the two CTAs of 256 threads that 2^13 elements allow, although
+// the groups are fewer then. The 28-qubit stem path takes 75.0 ms (67 launches)
+// against 80.0 ms (59), a 24-qubit one 5.22 against 5.64 ms.
+constexpr int kStemGroupCap = 12;
 
 void plan_stems(tnc_net* net) {
     Plan& P = net->plan;
@@ -223,15 +228,7 @@ void plan_stems(tnc_net* net) {
                 if (!Us.count(m)) ++inner;
             mx = std::max(mx, inner);
         }
-        // a step that is not in place (contracted and new elements differ) makes
-        // the kernel hold two buffers of the inner size: such groups stay within
-        // 2^kStemTwoBufferCap elements, so that three CTAs still share an SM
-        bool two = false;
-        for (size_t j = i; j < i + n; ++j) {
-            const NodePlan& np = P.nodes[chain[j]];
-            two |= !(np.kb == np.nb && np.kb > 0);
-        }
-        const int lim = two ? std::min(cap, kStemTwoBufferCap) : cap;
+        const int lim = std::min(cap, kStemGroupCap);
         if (mx > lim || (int)U.size() < net->stem_min_outer || U.size() > 30) return false;
         g = StemGroupPlan();
         g.steps.assign(chain.begin() + i, chain.begin() + i + n);
@@ -713,11 +710,28 @@ tnc_status ensure_groups(tnc_net* net, const Arena& ar, char* ws, int mode, int6
             g.tiles = tiles;
         }
     }
+    std::vector<tnc::StemRegBranches> branches;
     if (stem_fusion(net)) {
         G.stem_params.resize(net->plan.stems.size());
         for (const auto* list : {&G.inv, &G.ps})
             for (const Group& g : *list)
                 for (int gi : g.stems) G.stem_params[gi] = stem_params(net, ar, ws, gi, g.per_slice ? nb : 1);
+        for (const tnc::StemParams& sp : G.stem_params) {
+            auto r = std::make_unique<tnc::StemRegParams>();
+            branches.emplace_back();
+            if (!tnc::stem_reg_params(sp, *r, branches.back())) r.reset();
+            G.stem_reg.push_back(std::move(r));
+        }
+        if (branches.size() > net->d_stem_reg_cap) {
+            if (net->d_stem_reg) CUDA_TRY(cudaFree(net->d_stem_reg));
+            net->d_stem_reg = nullptr;
+            net->d_stem_reg_cap = 0;
+            CUDA_TRY(cudaMalloc(&net->d_stem_reg, branches.size() * sizeof(tnc::StemRegBranches)));
+            net->d_stem_reg_cap = branches.size();
+        }
+        if (!branches.empty())
+            CUDA_TRY(cudaMemcpyAsync(net->d_stem_reg, branches.data(), branches.size() * sizeof(tnc::StemRegBranches),
+                                     cudaMemcpyHostToDevice, s));
         if (G.stem_params.size() > net->d_stem_cap) {
             if (net->d_stem) CUDA_TRY(cudaFree(net->d_stem));
             net->d_stem = nullptr;
@@ -885,7 +899,8 @@ tnc_status run_group(tnc_net* net, const Arena& ar, char* ws, const Group& g, in
         double cm = 0.0;
         for (int k : sg.steps) cm += node_cmacs(net, net->plan.nodes[k].v);
         CUDA_TRY(timed_begin(net, sg.out, K_STEM, b, s, cm * b));
-        CUDA_TRY(tnc::launch_stem_fused(net->d_stem + gi, net->groups.stem_params[gi], sg.max_inner, slice0, b, s));
+        if (net->groups.stem_reg[gi]) CUDA_TRY(tnc::launch_stem_reg(*net->groups.stem_reg[gi], net->d_stem_reg + gi, slice0, b, s));
+        else CUDA_TRY(tnc::launch_stem_fused(net->d_stem + gi, net->groups.stem_params[gi], sg.max_inner, slice0, b, s));
         CUDA_TRY(timed_end(net, s));
     }
     return TNC_OK;

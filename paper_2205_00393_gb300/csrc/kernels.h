@@ -184,6 +184,60 @@ struct StemParams {
     StemStep steps[kStemMaxSteps];
 };
 
+// The same group for k_stem_reg, when every step is a one- or two-mode gate
+// (nk = nn), projects one mode away (nk = 1, nn = 0) or adds modes (nk = 1 or 0,
+// nn = 2). A position is a bit of the sub-tensor's address: X_0's bits, then one
+// for every mode that is added. A gate's new mode takes its contracted mode's
+// position, a projected mode's position dies and an added mode's is born, so the
+// group runs in place. The steps are cut into passes: a thread holds the
+// 2^kStemRegBits elements of its pass's register positions and applies the
+// pass's steps to them in registers.
+constexpr int kStemRegBits = 5;
+constexpr int kStemRegMaxN = 13;         // positions
+constexpr int kStemRegMinN = 9;
+constexpr int kStemRegMaxEntries = 192;  // elements of all dense branch copies
+
+enum StemRegKind : int8_t { SR_GATE1 = 0, SR_PROJECT = 1, SR_GATE2 = 2, SR_GROW1 = 3, SR_GROW0 = 4 };
+
+struct StemRegStep {
+    int8_t kind;   // StemRegKind
+    int8_t reg;    // gate or projection of one mode: its register bit; others: register bits 2 reg, 2 reg + 1
+    int16_t b_off; // the step's dense branch copy
+};
+
+struct StemRegPass {
+    int8_t step0, step1;                      // steps [step0, step1)
+    int8_t nt;                                // thread bits
+    int8_t unborn;                            // register bits without data when the pass begins
+    int8_t dead;                              // register bits projected away in this pass
+    uint16_t rslot[kStemRegBits];             // shared-memory slots (bytes, XOR-combined) of the register positions
+    uint16_t tslot[kStemRegMaxN - kStemRegBits];  // and of the thread bits' (0 past nt)
+};
+
+struct StemRegParams {
+    Operand in;
+    float2* out;
+    int64_t out_batch_stride;
+    int n, nu, npass, nentries;
+    int64_t ustr_in[32], ustr_out[32];
+    // strides in bytes of the first pass's register and thread bits in T_0, the last pass's in T_n
+    int64_t rstr_in[kStemRegBits], tstr_in[kStemRegMaxN - kStemRegBits];
+    int64_t rstr_out[kStemRegBits], tstr_out[kStemRegMaxN - kStemRegBits];
+    StemRegPass pass[kStemMaxSteps + 2];
+    StemRegStep step[kStemMaxSteps];
+};
+
+// The branches of a group, in device memory (threads index it, each its own entry).
+struct StemRegBranches {
+    int2 entry[kStemRegMaxEntries];           // dense branch entry e: its step and its element offset in the branch
+    Operand br[kStemMaxSteps];
+};
+
+// Fills r from a group's parameters; false if k_stem_reg cannot run it.
+bool stem_reg_params(const StemParams& sp, StemRegParams& r, StemRegBranches& rb);
+cudaError_t launch_stem_reg(const StemRegParams& p, const StemRegBranches* d_branches, int64_t slice0, int batch,
+                            cudaStream_t s);
+
 // Launch fused stem groups: params is a device array of n groups; group g
 // runs 2^nu[g] CTAs per slice (their maximum is max_outer_log2) with
 // 2 * 2^cap_log2 + b_total complex elements of shared memory.
