@@ -469,7 +469,7 @@ __device__ void root_dot(const GemmParams& p, const float2* A, const float2* B, 
         // thread); the offsets of j's bits come from shared-memory tables, one
         // per 8-bit group. Products are summed in FP32 over runs of 16 j and
         // the runs in FP64.
-        const int jb = p.kb - lb, ng = (jb + 7) / 8;
+        const int jb = p.kb - lb, ng = jb > 0 ? (jb + 7) / 8 : 1;  // (K = lanes: one table of zeros)
         for (int idx = threadIdx.x; idx < ng * 256; idx += 256) {
             const int g = idx >> 8, e = idx & 255;
             int64_t oa = 0, ob = 0;
@@ -487,21 +487,36 @@ __device__ void root_dot(const GemmParams& p, const float2* A, const float2* B, 
         const float2* Al = A + bits_offset(lane, p.ak, lb, 0);
         const float2* Bl = B + bits_offset(lane, p.bk, lb, 0);
         const int64_t j_lo = k_lo >> lb, j_hi = k_hi >> lb;
+        // eight j at a time (j_hi - j_lo is a power of two), all their loads in flight
+        // before the first product: one at a time, a chunk of 64 j waited 64 times. (One
+        // at a time inside the persistent executor, where the registers are short.)
+        constexpr int RB = BAR == 0 ? 8 : 1;
         for (int64_t j0 = j_lo; j0 < j_hi; j0 += 16) {
-            const int64_t je = j0 + 16 < j_hi ? j0 + 16 : j_hi;
             float sr = 0.f, si = 0.f;
-            for (int64_t j = j0; j < je; ++j) {
+            for (int64_t jb = j0; jb < j0 + 16 && jb < j_hi; jb += RB) {
+                const int nj = j_hi - jb < RB ? (int)(j_hi - jb) : RB;
                 int64_t oa = 0, ob = 0;
-                for (int g = 0; g < ng; ++g) {
-                    const int e = (int)((j >> (8 * g)) & 255);
+                for (int g = 1; g < ng; ++g) {
+                    const int e = (int)((jb >> (8 * g)) & 255);
                     oa += root_ta[g][e];
                     ob += root_tb[g][e];
                 }
-                const float2 a = Al[oa], b = Bl[ob];
-                sr = fmaf(a.x, b.x, sr);
-                sr = fmaf(-a.y, b.y, sr);
-                si = fmaf(a.x, b.y, si);
-                si = fmaf(a.y, b.x, si);
+                const int e0 = (int)(jb & 255);
+                float2 a[RB], b[RB];
+#pragma unroll
+                for (int t = 0; t < RB; ++t)
+                    if (t < nj) {
+                        a[t] = Al[oa + root_ta[0][e0 + t]];
+                        b[t] = Bl[ob + root_tb[0][e0 + t]];
+                    }
+#pragma unroll
+                for (int t = 0; t < RB; ++t)
+                    if (t < nj) {
+                        sr = fmaf(a[t].x, b[t].x, sr);
+                        sr = fmaf(-a[t].y, b[t].y, sr);
+                        si = fmaf(a[t].x, b[t].y, si);
+                        si = fmaf(a[t].y, b[t].x, si);
+                    }
             }
             re += sr;
             im += si;
@@ -547,6 +562,51 @@ __device__ __forceinline__ void root_chunk(const RootParams& rp, int chunk, int 
         bar_sync<BAR>();
     }
     if (lane == 0) out[r] = red[threadIdx.x];
+}
+
+// Ordered FP64 sum of a final contraction's `count` partial sums per output,
+// added to out: output r's are shared by L lanes (a power of two of at most 128, at
+// least 8 values each), lane l adding values l, l + L, ... and the lanes' sums
+// being added as a tree. L depends on count alone, so every caller adds in the
+// same order. (One lane per output read count values one after another: 67 us for
+// 8 slices of 64 chunks and 16 outputs.) Items are (r, l) pairs; threads 0-255 serve
+// items [item0, item0 + 256); red is shared-memory scratch of 256 entries.
+__host__ __device__ inline int acc_lanes(int count) {
+    int L = 1;
+    while (L < 128 && 16 * L <= count) L *= 2;
+    return L;
+}
+template <int BAR = 0>
+__device__ __forceinline__ void accumulate_items(const double2* partials, int count, const PermParams& pp, int64_t item0,
+                                                 double2* out, double2* red) {
+    const int L = acc_lanes(count), tid = threadIdx.x;
+    const int64_t R = 1ll << pp.obits, item = item0 + tid, r = item / L;
+    const int l = (int)(item % L);
+    const bool on = r < R;
+    double2 acc = make_double2(0.0, 0.0);
+    if (on) {
+        const double2* src = partials + bits_offset(r, pp.ostride, pp.obits, 0);
+#pragma unroll(BAR == 0 ? 8 : 2)
+        for (int i = l; i < count; i += L) {
+            const double2 v = src[(int64_t)i * R];
+            acc.x += v.x;
+            acc.y += v.y;
+        }
+    }
+    for (int st = L / 2; st > 0; st >>= 1) {
+        red[tid] = acc;
+        bar_sync<BAR>();
+        if (l < st) {
+            const double2 o = red[tid + st];
+            acc.x += o.x;
+            acc.y += o.y;
+        }
+        bar_sync<BAR>();
+    }
+    if (on && l == 0) {
+        out[r].x += acc.x;
+        out[r].y += acc.y;
+    }
 }
 
 }  // namespace f32dev

@@ -207,8 +207,9 @@ bool wl_root(tnc_net* net, const Arena& ar, char* ws, const NodePlan& np, int b,
     st.out = reinterpret_cast<double2*>(out);
     const int si = (int)W.sum.size();
     W.sum.push_back(st);
-    const int cdone = W.new_counter(1);
-    W.task(tnc::PT_SUM, si, 0, 0, netidx, 0, cg, -1, -1, cdone);
+    const int64_t R = 1ll << P.obits;
+    const int cdone = W.new_counter((int)((R + tnc::kSumOutputs - 1) / tnc::kSumOutputs));
+    for (int64_t r = 0; r < R; r += tnc::kSumOutputs) W.task(tnc::PT_SUM, si, r, 0, netidx, 0, cg, -1, -1, cdone);
     return true;
 }
 

@@ -65,21 +65,12 @@ __global__ void __launch_bounds__(256) k_root_partials(const __grid_constant__ R
                   root_tb);
 }
 
-// out[r] += sum_i partials[i][perm(r)], i ascending (fixed order)
-__global__ void k_accumulate_partials(const double2* __restrict__ partials, int count,
-                                      const __grid_constant__ PermParams pp, double2* __restrict__ out) {
-    const int64_t R = 1ll << pp.obits;
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R) return;
-    const int64_t src = bits_offset(r, pp.ostride, pp.obits, 0);
-    double2 acc = make_double2(0.0, 0.0);
-    for (int i = 0; i < count; ++i) {
-        double2 v = partials[(int64_t)i * R + src];
-        acc.x += v.x;
-        acc.y += v.y;
-    }
-    out[r].x += acc.x;
-    out[r].y += acc.y;
+// out[r] += sum_i partials[i][perm(r)] (a fixed order: accumulate_items)
+__global__ void __launch_bounds__(256) k_accumulate_partials(const double2* __restrict__ partials, int count,
+                                                             const __grid_constant__ PermParams pp,
+                                                             double2* __restrict__ out) {
+    __shared__ double2 red[256];
+    accumulate_items<0>(partials, count, pp, (int64_t)blockIdx.x * 256, out, red);
 }
 
 // out[r] += sum_z src_z[perm(r)] in FP64, z ascending
@@ -243,25 +234,18 @@ __global__ void __launch_bounds__(256) k_root_partials_multi(const RootParams* _
     root_chunk<0>(rp, chunk, z, rs0[lo], partials[lo] + ((int64_t)z * rp.chunks + chunk) * R, red, root_ta, root_tb);
 }
 
-// out_i[r] += sum over network i's partial sums (slices in order, then chunks).
-__global__ void k_accumulate_multi(const RootParams* __restrict__ roots, double2* const* __restrict__ partials,
-                                   const PermParams* __restrict__ perms, double2* const* __restrict__ outs,
-                                   const int* __restrict__ rb) {
+// out_i[r] += sum over network i's partial sums (slices in order, then chunks; as
+// accumulate_items adds them), one block per network.
+__global__ void __launch_bounds__(256) k_accumulate_multi(const RootParams* __restrict__ roots,
+                                                          double2* const* __restrict__ partials,
+                                                          const PermParams* __restrict__ perms,
+                                                          double2* const* __restrict__ outs, const int* __restrict__ rb) {
+    __shared__ double2 red[256];
     const int i = blockIdx.x;
     const PermParams& pp = perms[i];
-    const int64_t R = 1ll << pp.obits;
     const int count = rb[i] * roots[i].chunks;
-    for (int64_t r = threadIdx.x; r < R; r += blockDim.x) {
-        const int64_t src = bits_offset(r, pp.ostride, pp.obits, 0);
-        double2 acc = make_double2(0.0, 0.0);
-        for (int c = 0; c < count; ++c) {
-            double2 v = partials[i][(int64_t)c * R + src];
-            acc.x += v.x;
-            acc.y += v.y;
-        }
-        outs[i][r].x += acc.x;
-        outs[i][r].y += acc.y;
-    }
+    const int64_t items = (int64_t)acc_lanes(count) << pp.obits;
+    for (int64_t it = 0; it < items; it += 256) accumulate_items<0>(partials[i], count, pp, it, outs[i], red);
 }
 
 bool gemm_f32_long(int kb) { return kb >= 8; }
@@ -320,8 +304,8 @@ cudaError_t launch_root_partials(const RootParams& p, int batch, double2* partia
 
 cudaError_t launch_accumulate_partials(const double2* partials, int count, const PermParams& pp,
                                        double2* out, cudaStream_t s) {
-    int64_t R = 1ll << pp.obits;
-    k_accumulate_partials<<<(unsigned)((R + 255) / 256), 256, 0, s>>>(partials, count, pp, out);
+    const int64_t items = (int64_t)acc_lanes(count) << pp.obits;
+    k_accumulate_partials<<<(unsigned)((items + 255) / 256), 256, 0, s>>>(partials, count, pp, out);
     return cudaGetLastError();
 }
 

@@ -177,8 +177,13 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// 8 consecutive 32-bit TMEM columns of this warp's 32 lanes (one per lane)
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+// 4 or 8 consecutive 32-bit TMEM columns of this warp's 32 lanes (one per lane)
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                  : "r"(taddr));
@@ -241,38 +246,34 @@ using f32dev::pack2;
 using f32dev::unpack2;
 
 // Adds a chunk's accumulators (this warp's 32 rows x 64 complex columns at
-// taddr, Ci TN columns further) to the FP32 sums, 8 columns at a time by packed
-// operations. Split FP16x2 undoes the scales first: sa of this lane's row, then
-// the column's factor in the same FMA as the addition (both are powers of two,
-// so every product is exact). The drain takes 128 packed operations a lane
-// instead of 384 scalar ones.
-template <int KIND>
+// taddr, Ci TN columns further) to the FP32 sums, by packed operations. Split
+// FP16x2 undoes the scales first: sa of this lane's row, then the column's factor
+// in the same FMA as the addition (both are powers of two, so every product is
+// exact). The drain takes 128 packed operations a lane instead of 384 scalar
+// ones.
+template <int KIND, int CW>
 __device__ __forceinline__ void drain_chunk(uint32_t taddr, float sa, const float* colf, f32x2 (&cr)[32], f32x2 (&ci)[32]) {
     const f32x2 sa2 = pack2(sa, sa);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        uint32_t re[8], im[8];
-        tmem_ld8(taddr + 8 * q, re);
-        tmem_ld8(taddr + TN + 8 * q, im);
-        f32x2 f[4];
-        if constexpr (KIND == 3) {
-            const ulonglong2* t = reinterpret_cast<const ulonglong2*>(colf + 8 * q);
-            f[0] = t[0].x;
-            f[1] = t[0].y;
-            f[2] = t[1].x;
-            f[3] = t[1].y;
-        }
+    for (int q = 0; q < 64 / CW; ++q) {
+        uint32_t re[CW], im[CW];
+        tmem_ld(taddr + CW * q, re);
+        tmem_ld(taddr + TN + CW * q, im);
         tmem_wait_ld();
+        if constexpr (KIND == 3) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const f32x2 r = pack2(__uint_as_float(re[2 * j]), __uint_as_float(re[2 * j + 1]));
-            const f32x2 i = pack2(__uint_as_float(im[2 * j]), __uint_as_float(im[2 * j + 1]));
-            if constexpr (KIND == 3) {
-                cr[4 * q + j] = fma2(f32dev::mul2(r, sa2), f[j], cr[4 * q + j]);
-                ci[4 * q + j] = fma2(f32dev::mul2(i, sa2), f[j], ci[4 * q + j]);
-            } else {
-                cr[4 * q + j] = add2(cr[4 * q + j], r);
-                ci[4 * q + j] = add2(ci[4 * q + j], i);
+            for (int j = 0; j < CW / 2; ++j) {
+                const f32x2 f = *reinterpret_cast<const f32x2*>(colf + CW * q + 2 * j);
+                const f32x2 r = pack2(__uint_as_float(re[2 * j]), __uint_as_float(re[2 * j + 1]));
+                const f32x2 i = pack2(__uint_as_float(im[2 * j]), __uint_as_float(im[2 * j + 1]));
+                cr[CW / 2 * q + j] = fma2(f32dev::mul2(r, sa2), f, cr[CW / 2 * q + j]);
+                ci[CW / 2 * q + j] = fma2(f32dev::mul2(i, sa2), f, ci[CW / 2 * q + j]);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < CW / 2; ++j) {
+                cr[CW / 2 * q + j] = add2(cr[CW / 2 * q + j], pack2(__uint_as_float(re[2 * j]), __uint_as_float(re[2 * j + 1])));
+                ci[CW / 2 * q + j] = add2(ci[CW / 2 * q + j], pack2(__uint_as_float(im[2 * j]), __uint_as_float(im[2 * j + 1])));
             }
         }
     }
@@ -487,7 +488,7 @@ __device__ __forceinline__ void tc_tile(const CUtensorMap* tmA, const CUtensorMa
                 colf[2 * lane + 1] = pow2f(-(int)e2.y);
                 __syncwarp();
             }
-            drain_chunk<KIND>(tmem + ((uint32_t)(32 * g) << 16) + (uint32_t)(buf * 2 * TN + 64 * h), sa, colf, cr, ci);
+            drain_chunk<KIND, KIND == 3 ? 4 : 8>(tmem + ((uint32_t)(32 * g) << 16) + (uint32_t)(buf * 2 * TN + 64 * h), sa, colf, cr, ci);
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&sh.tfree[buf]));
@@ -824,7 +825,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                     colf[2 * lane + 1] = pow2f(-(int)e2.y);
                     __syncwarp();
                 }
-                drain_chunk<KIND>(tmem + ((uint32_t)(32 * gq) << 16) + (uint32_t)(buf * 2 * TN + 64 * h), sa, colf, cr, ci);
+                drain_chunk<KIND, KIND == 3 ? 4 : 8>(tmem + ((uint32_t)(32 * gq) << 16) + (uint32_t)(buf * 2 * TN + 64 * h), sa, colf, cr, ci);
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(tfree0[buf]);
@@ -1502,27 +1503,20 @@ __global__ void __launch_bounds__(NT_, KIND >= 0 ? 1 : 2) k_persist(const __grid
                                           root_tb);
                 }
                 break;
-            case PT_ACC: {
-                const AccParams& ap = P.acc[tk.idx];
-                double2* const dst = P.out0 ? P.out0 : ap.out;
-                const int64_t R = 1ll << ap.pp.obits;
-                for (int64_t r = tid; r < R; r += NT_) {
-                    const int64_t src = f32dev::bits_offset(r, ap.pp.ostride, ap.pp.obits, 0);
-                    double2 acc = make_double2(0.0, 0.0);
-                    for (int i = 0; i < ap.count; ++i) {
-                        const double2 v = ap.partials[(int64_t)i * R + src];
-                        acc.x += v.x;
-                        acc.y += v.y;
-                    }
-                    dst[r].x += acc.x;
-                    dst[r].y += acc.y;
+            case PT_ACC:
+                if (tid < 256) {
+                    const AccParams& ap = P.acc[tk.idx];
+                    double2* const dst = P.out0 ? P.out0 : ap.out;
+                    const int64_t items = (int64_t)f32dev::acc_lanes(ap.count) << ap.pp.obits;
+                    for (int64_t it = 0; it < items; it += 256)
+                        f32dev::accumulate_items<1>(ap.partials, ap.count, ap.pp, it, dst, root_red);
                 }
-            } break;
-            case PT_SUM: {
+                break;
+            case PT_SUM: {  // item: first of kSumOutputs outputs
                 const SumTaskParams& sp = P.sum[tk.idx];
                 double2* const dst = P.out0 ? P.out0 : sp.out;
-                const int64_t R = 1ll << sp.sp.obits;
-                for (int64_t r = tid; r < R; r += NT_) {
+                const int64_t R = 1ll << sp.sp.obits, r1 = tk.item + kSumOutputs < R ? tk.item + kSumOutputs : R;
+                for (int64_t r = tk.item + tid; r < r1; r += NT_) {
                     const int64_t off = f32dev::bits_offset(r, sp.sp.ostride, sp.sp.obits, 0);
                     double2 acc = make_double2(0.0, 0.0);
                     for (int z = 0; z < sp.batch; ++z) {
