@@ -149,6 +149,47 @@ struct DeviceWorkList {
     }
 };
 
+// The adjoint pass of a plan by tree levels (host_backward.cpp): its launches in
+// order, with their parameters in device tables.
+struct BackwardOp {
+    enum Type { GROUP, NODE, LEAF, INV_SUM, INV_READ, SEED } type = GROUP;
+    // GROUP: FP32 contractions in one launch; LEAF, INV_*: entries of the fold tables
+    int first = 0, n = 0, off_first = 0;
+    int64_t blocks = 0;
+    double cmacs = 0.0;  // per batch entry
+    bool per_slice = false;
+    // NODE: one contraction on its own (tensor cores, or a large or long FP32 one)
+    tnc::GemmParams g{};
+    int node = -1, choice = 0;
+    int64_t pa = -1, pb = -1;  // split planes
+    tnc::SeedParams seed{};
+};
+struct BackwardPlan {
+    std::vector<BackwardOp> inv_fwd, slices[2], inv_rev;  // slices: a whole batch, and the smaller last one
+    std::vector<tnc::GemmParams> gemm;
+    std::vector<tnc::LeafEnvParams> leaf;
+    std::vector<tnc::InvEnvParams> inv;
+    std::vector<int64_t> off;                             // prefix counts of every grouped launch
+    int64_t top = 0;                                      // workspace bytes
+    int64_t zero_bytes = 0;                               // FP64 sums at the workspace's start, leaf gradients first
+    // device copies
+    void* mem = nullptr;
+    const tnc::GemmParams* d_gemm = nullptr;
+    const tnc::LeafEnvParams* d_leaf = nullptr;
+    const tnc::InvEnvParams* d_inv = nullptr;
+    const int64_t* d_off = nullptr;
+    ~BackwardPlan() {
+        if (mem) cudaFree(mem);
+    }
+};
+// Batch, checkpoint spacing and workspace that the adjoint pass chose for a call.
+struct BackwardSizes {
+    int keep_every = 1;
+    int64_t nb = 0;        // 0: one slice does not fit the budget
+    size_t need = 0;       // node by node
+    size_t need_levels = 0;  // by levels (0: not run that way)
+};
+
 inline int64_t stride_of(const std::vector<std::pair<int, int64_t>>& s, int mode) {
     for (auto& p : s)
         if (p.first == mode) return p.second;
@@ -244,6 +285,8 @@ struct tnc_net {
     mutable std::map<std::string, Arena> arena_cache;  // plan_arena results by their inputs
     std::map<std::string, std::pair<double, double>> cost_cache;  // level_cost results (launches, seconds)
     std::map<std::string, std::unique_ptr<DeviceWorkList>> worklists;
+    std::map<std::string, BackwardSizes> backward_sizes;                     // by what they depend on
+    std::map<std::string, std::unique_ptr<BackwardPlan>> backward_plans;     // and the workspace
     double timed_persist_tc_cmacs = 0.0;  // tensor-core share of the timed persistent launches
     unsigned long long* d_prof = nullptr;  // "persist_profile": per task type time, count, wait
 

@@ -51,48 +51,18 @@ int64_t layout_stride(const std::vector<int>& layout, int mode) {
     return -1;
 }
 
-// Environment of child `c` of node np from the node's environment.
-tnc_status env_child(Backward& bw, const NodePlan& np, int c, int64_t b, int64_t slice0) {
-    tnc_net* net = bw.net;
+// The contraction that gives the environment of child c of node np (into
+// env_off[c]) from the node's environment and the sibling's value.
+tnc::GemmParams env_gemm(const Backward& bw, const NodePlan& np, int c, int64_t b) {
+    const tnc_net* net = bw.net;
     const Plan& P = net->plan;
     const bool is_a = (c == np.A);
-    const int sib = is_a ? np.B : np.A;
-    std::vector<int> lay;
-    if (is_a) {
-        lay = np.mm;
-        lay.insert(lay.end(), np.km.begin(), np.km.end());
-    } else {
-        lay = np.km;
-        lay.insert(lay.end(), np.nm.begin(), np.nm.end());
-    }
-    bw.env_layout[c] = lay;
-    const bool per = P.per_slice[c] != 0;
-    const int64_t elems = 1ll << lay.size();
-    const int64_t bb = per ? b : b;  // per-slice environments of every child, batch b
-    int64_t off = bw.A.alloc(bb * elems * 8);
-    bw.env_off[c] = off;
-    // GEMM dims of this environment: E_A is (mb, kb) over nb; E_B is (kb, nb) over mb
-    const int gmb = is_a ? np.mb : np.kb, gnb = is_a ? np.kb : np.nb, gkb = is_a ? np.nb : np.mb;
-    const int env_choice = shape_choice(net, bw.mode, gmb, gnb, gkb, false);
-    const bool tc = env_choice != 0;
-    int64_t pa = -1, pb = -1;
-    if (tc) {  // split-precision planes (allocated in the sizing pass too)
-        pa = bw.A.alloc(tc_bytes_a(bw.net, bw.mode, gmb, gnb, gkb, b));
-        pb = bw.A.alloc(tc_bytes_b(bw.net, bw.mode, gmb, gnb, gkb, b));
-    }
-    if (!bw.exec) {
-        if (tc) {
-            bw.A.release(pa);
-            bw.A.release(pb);
-        }
-        return TNC_OK;
-    }
     tnc::GemmParams g{};
     const std::vector<int>& ev = bw.env_layout[np.v];
     tnc::Operand E{};
     E.ptr = reinterpret_cast<const float2*>(bw.ws + bw.env_off[np.v]);
     E.batch_stride = P.per_slice[np.v] || np.is_root ? ((int64_t)1 << ev.size()) : 0;
-    tnc::Operand S = operand(net, bw.fwd, bw.ws, sib, b);
+    tnc::Operand S = operand(net, bw.fwd, bw.ws, is_a ? np.B : np.A, b);
     if (is_a) {
         // E_A[m, k] = sum_n E_v[m, n] B[k, n]
         g.A = E;
@@ -120,8 +90,61 @@ tnc_status env_child(Backward& bw, const NodePlan& np, int c, int64_t b, int64_t
         }
         for (int j = 0; j < np.nb; ++j) g.bn[j] = layout_stride(ev, np.nm[np.nb - 1 - j]);
     }
-    g.C = reinterpret_cast<float2*>(bw.ws + off);
-    g.c_batch_stride = elems;
+    g.C = reinterpret_cast<float2*>(bw.ws + bw.env_off[c]);
+    g.c_batch_stride = 1ll << bw.env_layout[c].size();
+    return g;
+}
+
+// Layout of child c's environment: its modes in np's order.
+std::vector<int> env_child_layout(const NodePlan& np, int c) {
+    std::vector<int> lay = c == np.A ? np.mm : np.km;
+    const std::vector<int>& rest = c == np.A ? np.km : np.nm;
+    lay.insert(lay.end(), rest.begin(), rest.end());
+    return lay;
+}
+
+// Parameters that fold leaf c's environments into its FP64 gradient.
+tnc::LeafEnvParams leaf_env_params(const Backward& bw, int c) {
+    const tnc_net* net = bw.net;
+    tnc::LeafEnvParams lp{};
+    lp.env = reinterpret_cast<const float2*>(bw.ws + bw.env_off[c]);
+    lp.env_batch_stride = 1ll << bw.env_layout[c].size();
+    int q = 0;
+    for (int64_t e : net->leaf_idx[c])
+        for (int bit = 0; bit < net->logd[e]; ++bit, ++q) {
+            const int mode = net->mode_base[e] + bit;
+            lp.sl_bit[q] = net->plan.slice_bit_of_mode[mode];
+            lp.env_stride[q] = lp.sl_bit[q] >= 0 ? 0 : layout_stride(bw.env_layout[c], mode);
+        }
+    lp.L = q;
+    lp.grad = reinterpret_cast<double2*>(bw.ws + bw.leaf_grad) + net->leaf_off[c];
+    return lp;
+}
+
+// Environment of child `c` of node np from the node's environment.
+tnc_status env_child(Backward& bw, const NodePlan& np, int c, int64_t b, int64_t slice0) {
+    tnc_net* net = bw.net;
+    const bool is_a = (c == np.A);
+    bw.env_layout[c] = env_child_layout(np, c);
+    const int64_t elems = 1ll << bw.env_layout[c].size();
+    bw.env_off[c] = bw.A.alloc(b * elems * 8);  // environments of every child, batch b
+    // GEMM dims of this environment: E_A is (mb, kb) over nb; E_B is (kb, nb) over mb
+    const int gmb = is_a ? np.mb : np.kb, gnb = is_a ? np.kb : np.nb, gkb = is_a ? np.nb : np.mb;
+    const int env_choice = shape_choice(net, bw.mode, gmb, gnb, gkb, false);
+    const bool tc = env_choice != 0;
+    int64_t pa = -1, pb = -1;
+    if (tc) {  // split-precision planes (allocated in the sizing pass too)
+        pa = bw.A.alloc(tc_bytes_a(bw.net, bw.mode, gmb, gnb, gkb, b));
+        pb = bw.A.alloc(tc_bytes_b(bw.net, bw.mode, gmb, gnb, gkb, b));
+    }
+    if (!bw.exec) {
+        if (tc) {
+            bw.A.release(pa);
+            bw.A.release(pb);
+        }
+        return TNC_OK;
+    }
+    tnc::GemmParams g = env_gemm(bw, np, c, b);
     g.slice0 = slice0;
     if (tc) {
         // split precision with FP32 accumulation, as in the forward
@@ -147,19 +170,8 @@ tnc_status env_fold(Backward& bw, int c, int64_t b, int64_t slice0, bool from_pe
     const int64_t elems = 1ll << bw.env_layout[c].size();
     if (c < net->n_leaves) {
         if (bw.exec) {
-            tnc::LeafEnvParams lp{};
-            lp.env = reinterpret_cast<const float2*>(bw.ws + bw.env_off[c]);
-            lp.env_batch_stride = elems;
-            int q = 0;
-            for (int64_t e : net->leaf_idx[c])
-                for (int bit = 0; bit < net->logd[e]; ++bit, ++q) {
-                    const int mode = net->mode_base[e] + bit;
-                    lp.sl_bit[q] = P.slice_bit_of_mode[mode];
-                    lp.env_stride[q] = lp.sl_bit[q] >= 0 ? 0 : layout_stride(bw.env_layout[c], mode);
-                }
-            lp.L = q;
+            tnc::LeafEnvParams lp = leaf_env_params(bw, c);
             lp.slice0 = slice0;
-            lp.grad = reinterpret_cast<double2*>(bw.ws + bw.leaf_grad) + net->leaf_off[c];
             CUDA_TRY(timed_begin(net, c, -2, (int)b, bw.s, 0.0));
             CUDA_TRY(tnc::launch_leaf_env_accum(lp, (int)b, bw.s));
             CUDA_TRY(timed_end(net, bw.s));
@@ -354,6 +366,305 @@ tnc_status backward_run(Backward& bw, int64_t lo, int64_t hi, const double* grad
 }
 
 
+// ------------------------------------------------------ adjoint pass by levels
+//
+// The same computation in few launches: the contractions of a tree level, forward
+// and reverse, run as one grouped launch (those of the tensor cores, of 256 tiles
+// or more, or of a long K on their own), and so do the folds of the
+// environments that a level produces. Node by node, a 16-qubit gradient took
+// 659 launches, planned anew (and sized several times) on every call. Every
+// contraction and every FP64 sum is the same as node by node.
+// This way is taken when every intermediate is kept (no checkpoints) and its
+// workspace fits the budget at the batch that the node-by-node pass would take.
+
+struct LevelBuilder {
+    Backward& bw;
+    BackwardPlan& bp;
+
+    // an FP32 or tensor-core contraction (node: its record in the timings)
+    void add(std::vector<std::pair<tnc::GemmParams, int>>& grouped, std::vector<BackwardOp>& singles, const tnc::GemmParams& g,
+             int node, bool per_slice) {
+        const tnc_net* net = bw.net;
+        const int choice = shape_choice(net, bw.mode, g.mb, g.nb, g.kb, false);
+        if (!choice && tnc::gemm_f32_tiles(g.mb, g.nb) < 256 && !tnc::gemm_f32_long(g.kb)) {
+            grouped.emplace_back(g, node);
+            return;
+        }
+        BackwardOp op;
+        op.type = BackwardOp::NODE;
+        op.per_slice = per_slice;
+        op.g = g;
+        op.node = node;
+        op.choice = choice;
+        op.cmacs = std::ldexp(1.0, g.mb + g.nb + g.kb);
+        singles.push_back(op);
+    }
+    // the level's launches, the grouped one first. Called when every output of the
+    // level has its place: a contraction's planes may then take any free bytes,
+    // the next one's planes the same ones.
+    void emit(std::vector<BackwardOp>& ops, const std::vector<std::pair<tnc::GemmParams, int>>& grouped,
+              std::vector<BackwardOp>& singles, bool per_slice, int64_t b) {
+        const tnc_net* net = bw.net;
+        for (BackwardOp& op : singles) {
+            if (!op.choice) continue;
+            op.pa = bw.A.alloc(tc_bytes_a(net, bw.mode, op.g.mb, op.g.nb, op.g.kb, b));
+            op.pb = bw.A.alloc(tc_bytes_b(net, bw.mode, op.g.mb, op.g.nb, op.g.kb, b));
+            bw.A.release(op.pa);
+            bw.A.release(op.pb);
+        }
+        if (!grouped.empty()) {
+            BackwardOp op;
+            op.per_slice = per_slice;
+            op.first = (int)bp.gemm.size();
+            op.off_first = (int)bp.off.size();
+            op.n = (int)grouped.size();
+            for (const auto& [g, node] : grouped) {
+                bp.off.push_back(op.blocks);
+                op.blocks += tnc::gemm_f32_group_tiles(g.mb, g.nb);
+                op.cmacs += std::ldexp(1.0, g.mb + g.nb + g.kb);
+                bp.gemm.push_back(g);
+            }
+            bp.off.push_back(op.blocks);
+            ops.push_back(op);
+        }
+        for (BackwardOp& op : singles) ops.push_back(std::move(op));
+        singles.clear();
+    }
+    // one launch over the entries [first, table size) of a fold table, elems elements each
+    void emit_fold(std::vector<BackwardOp>& ops, BackwardOp::Type type, int first, const std::vector<int64_t>& elems) {
+        if (elems.empty()) return;
+        BackwardOp op;
+        op.type = type;
+        op.first = first;
+        op.n = (int)elems.size();
+        op.off_first = (int)bp.off.size();
+        for (int64_t n : elems) {
+            bp.off.push_back(op.blocks);
+            op.blocks += (n + 255) / 256;
+        }
+        bp.off.push_back(op.blocks);
+        ops.push_back(op);
+    }
+    // forward contractions of one class, every output kept
+    void forward(std::vector<BackwardOp>& ops, bool per_slice, int64_t b) {
+        tnc_net* net = bw.net;
+        const Plan& P = net->plan;
+        for (const Group& lg : level_groups(net, bw.mode, per_slice)) {
+            std::vector<std::pair<tnc::GemmParams, int>> grouped;
+            std::vector<BackwardOp> singles;
+            for (auto* list : {&lg.fp32, &lg.tc})
+                for (int v : *list) {
+                    const NodePlan& np = P.nodes[v - net->n_leaves];
+                    bw.fwd.off[v] = bw.A.alloc((per_slice ? b : 1) * tensor_bytes(P, v));
+                    tnc::GemmParams g = gemm_params(net, bw.fwd, bw.ws, np, b);
+                    g.C = reinterpret_cast<float2*>(bw.ws + bw.fwd.off[v]);
+                    g.c_batch_stride = per_slice ? tensor_bytes(P, v) / 8 : 0;
+                    add(grouped, singles, g, v, per_slice);
+                }
+            emit(ops, grouped, singles, per_slice, per_slice ? b : 1);
+        }
+    }
+    // reverse walk of one class, a level of nodes at a time (level 0: the root, or
+    // the invariant tensors whose environments were summed)
+    void reverse(std::vector<BackwardOp>& ops, bool per_slice, int64_t b) {
+        tnc_net* net = bw.net;
+        const Plan& P = net->plan;
+        const int nl = net->n_leaves;
+        std::vector<int> level(net->tree->n_tensors(), 0);
+        std::vector<std::vector<int>> by_level;
+        for (int i = (int)P.nodes.size() - 1; i >= 0; --i) {
+            const NodePlan& np = P.nodes[i];
+            if (np.per_slice != per_slice || !bw.needs[np.v]) continue;
+            const int l = level[np.v];
+            if ((int)by_level.size() <= l) by_level.resize(l + 1);
+            by_level[l].push_back(i);
+            for (int c : {np.A, np.B})
+                if (c >= nl && (P.per_slice[c] != 0) == per_slice) level[c] = l + 1;
+        }
+        for (const auto& nodes : by_level) {
+            std::vector<std::pair<tnc::GemmParams, int>> grouped;
+            std::vector<BackwardOp> singles;
+            std::vector<int64_t> leaf_elems, inv_elems;
+            const int leaf0 = (int)bp.leaf.size(), inv0 = (int)bp.inv.size();
+            std::vector<int> folded;
+            for (int i : nodes) {
+                const NodePlan& np = P.nodes[i];
+                for (int c : {np.A, np.B}) {
+                    if (!bw.needs[c]) continue;
+                    bw.env_layout[c] = env_child_layout(np, c);
+                    const int64_t elems = 1ll << bw.env_layout[c].size();
+                    bw.env_off[c] = bw.A.alloc(b * elems * 8);
+                    add(grouped, singles, env_gemm(bw, np, c, b), np.v, per_slice);
+                    if (c < nl) {
+                        bp.leaf.push_back(leaf_env_params(bw, c));
+                        leaf_elems.push_back(net->leaf_elems[c]);
+                        folded.push_back(c);
+                    } else if (per_slice && !P.per_slice[c]) {
+                        tnc::InvEnvParams ip{};
+                        ip.env = reinterpret_cast<float2*>(bw.ws + bw.env_off[c]);
+                        ip.acc = reinterpret_cast<double2*>(bw.ws + bw.inv_acc[c]);
+                        ip.n = elems;
+                        bp.inv.push_back(ip);
+                        inv_elems.push_back(elems);
+                        folded.push_back(c);
+                    }
+                }
+            }
+            emit(ops, grouped, singles, per_slice, b);
+            emit_fold(ops, BackwardOp::LEAF, leaf0, leaf_elems);
+            emit_fold(ops, BackwardOp::INV_SUM, inv0, inv_elems);
+            for (int c : folded) bw.A.release(bw.env_off[c]);
+            for (int i : nodes) {
+                const NodePlan& np = P.nodes[i];
+                bw.A.release(bw.env_off[np.v]);
+                if (per_slice)  // the children's values are not needed again
+                    for (int c : {np.A, np.B})
+                        if (c >= nl && P.per_slice[c]) bw.A.release(bw.fwd.off[c]);
+            }
+        }
+    }
+};
+
+// The whole pass for batches of nb slices and a last one of `tail` (0: none); bw.ws
+// may be null to size the workspace.
+void build_backward_plan(Backward& bw, int64_t nb, int64_t tail, BackwardPlan& bp) {
+    tnc_net* net = bw.net;
+    const Plan& P = net->plan;
+    const tnc::Tree& T = *net->tree;
+    struct NoFuse {  // no fused stem groups in the forward levels
+        tnc_net* net;
+        bool was;
+        explicit NoFuse(tnc_net* n) : net(n), was(n->in_many) { n->in_many = true; }
+        ~NoFuse() { net->in_many = was; }
+    } no_fuse(net);
+    LevelBuilder lb{bw, bp};
+    bw.fwd.off.assign(T.n_tensors(), -1);
+    bw.env_layout.assign(T.n_tensors(), {});
+    bw.env_off.assign(T.n_tensors(), -1);
+    bw.inv_acc.assign(T.n_tensors(), -1);
+    bw.leaf_grad = bw.A.alloc(net->total_leaf_elems * 16);
+    bp.zero_bytes = bw.leaf_grad + align_up(std::max<int64_t>(net->total_leaf_elems * 16, 1));
+    for (int v = net->n_leaves; v < T.n_tensors(); ++v) {
+        if (P.per_slice[v] || v == T.root || !bw.needs[v]) continue;
+        const int par = T.parent[v];
+        if (par < 0 || !(P.per_slice[par] || par == T.root)) continue;
+        bw.inv_acc[v] = bw.A.alloc((int64_t)16 << P.layout[v].size());  // right behind the one before
+        bp.zero_bytes = bw.inv_acc[v] + align_up((int64_t)16 << P.layout[v].size());
+    }
+    lb.forward(bp.inv_fwd, false, 1);
+    const FitAlloc saved = bw.A;
+    for (int q = 0; q < (tail ? 2 : 1); ++q) {
+        const int64_t b = q ? tail : nb;
+        auto& ops = bp.slices[q];
+        lb.forward(ops, true, b);
+        bw.env_layout[T.root] = P.layout[T.root];
+        const int64_t relems = 1ll << P.layout[T.root].size();
+        bw.env_off[T.root] = bw.A.alloc(b * relems * 8);
+        BackwardOp seed;
+        seed.type = BackwardOp::SEED;
+        seed.seed.obits = P.obits;
+        for (int j = 0; j < P.obits; ++j) seed.seed.ostride[j] = P.out_stride[j];
+        seed.seed.E = reinterpret_cast<float2*>(bw.ws + bw.env_off[T.root]);
+        seed.seed.batch_stride = relems;
+        ops.push_back(seed);
+        lb.reverse(ops, true, b);
+        bw.A.used = saved.used;  // the batch's buffers are dead; keep the peak
+    }
+    const int inv0 = (int)bp.inv.size();
+    std::vector<int64_t> inv_elems;
+    for (int v = net->n_leaves; v < T.n_tensors(); ++v) {
+        if (bw.inv_acc[v] < 0) continue;
+        if (bw.env_layout[v].empty() && !P.layout[v].empty()) bw.env_layout[v] = P.layout[v];
+        const int64_t elems = (int64_t)1 << P.layout[v].size();
+        bw.env_off[v] = bw.A.alloc(elems * 8);
+        tnc::InvEnvParams ip{};
+        ip.env = reinterpret_cast<float2*>(bw.ws + bw.env_off[v]);
+        ip.acc = reinterpret_cast<double2*>(bw.ws + bw.inv_acc[v]);
+        ip.n = elems;
+        bp.inv.push_back(ip);
+        inv_elems.push_back(elems);
+    }
+    lb.emit_fold(bp.inv_rev, BackwardOp::INV_READ, inv0, inv_elems);
+    lb.reverse(bp.inv_rev, false, 1);
+    bp.top = bw.A.top;
+}
+
+tnc_status upload_backward_plan(BackwardPlan& bp, cudaStream_t s) {
+    size_t off = 0;
+    auto slot = [&](size_t bytes) {
+        const size_t o = off;
+        off += (bytes + 255) / 256 * 256;
+        return o;
+    };
+    const size_t o_gemm = slot(bp.gemm.size() * sizeof(bp.gemm[0])), o_leaf = slot(bp.leaf.size() * sizeof(bp.leaf[0])),
+                 o_inv = slot(bp.inv.size() * sizeof(bp.inv[0])), o_off = slot(bp.off.size() * sizeof(bp.off[0]));
+    CUDA_TRY(cudaMalloc(&bp.mem, std::max<size_t>(off, 256)));
+    char* base = static_cast<char*>(bp.mem);
+    auto up = [&](size_t o, const void* src, size_t bytes) -> cudaError_t {
+        return bytes ? cudaMemcpyAsync(base + o, src, bytes, cudaMemcpyHostToDevice, s) : cudaSuccess;
+    };
+    CUDA_TRY(up(o_gemm, bp.gemm.data(), bp.gemm.size() * sizeof(bp.gemm[0])));
+    CUDA_TRY(up(o_leaf, bp.leaf.data(), bp.leaf.size() * sizeof(bp.leaf[0])));
+    CUDA_TRY(up(o_inv, bp.inv.data(), bp.inv.size() * sizeof(bp.inv[0])));
+    CUDA_TRY(up(o_off, bp.off.data(), bp.off.size() * sizeof(bp.off[0])));
+    CUDA_TRY(cudaStreamSynchronize(s));  // the host vectors may go
+    bp.d_gemm = reinterpret_cast<const tnc::GemmParams*>(base + o_gemm);
+    bp.d_leaf = reinterpret_cast<const tnc::LeafEnvParams*>(base + o_leaf);
+    bp.d_inv = reinterpret_cast<const tnc::InvEnvParams*>(base + o_inv);
+    bp.d_off = reinterpret_cast<const int64_t*>(base + o_off);
+    bp.gemm.clear();
+    bp.leaf.clear();
+    bp.inv.clear();
+    return TNC_OK;
+}
+
+tnc_status run_backward_ops(tnc_net* net, const BackwardPlan& bp, const std::vector<BackwardOp>& ops, int64_t batch,
+                            int64_t slice0, int mode, const double* grad_out, char* ws, cudaStream_t s) {
+    tnc_status st;
+    for (const BackwardOp& op : ops) {
+        const int b = op.per_slice ? (int)batch : 1;
+        switch (op.type) {
+            case BackwardOp::GROUP:
+                CUDA_TRY(timed_begin(net, -1, K_GEMM_F32, b, s, op.cmacs * b));
+                CUDA_TRY(tnc::launch_gemm_f32_group(bp.d_gemm + op.first, bp.d_off + op.off_first, op.n, op.blocks, slice0, b, s));
+                CUDA_TRY(timed_end(net, s));
+                break;
+            case BackwardOp::NODE: {
+                tnc::GemmParams g = op.g;
+                g.slice0 = slice0;
+                if (op.choice) {
+                    if ((st = launch_tc_contraction(net, g, b, mode, ws + op.pa, ws + op.pb, op.node, s, op.choice, b)) != TNC_OK)
+                        return st;
+                } else {
+                    CUDA_TRY(timed_begin(net, op.node, K_GEMM_F32, b, s, op.cmacs * b));
+                    CUDA_TRY(tnc::launch_gemm_f32(g, b, s));
+                    CUDA_TRY(timed_end(net, s));
+                }
+                break;
+            }
+            case BackwardOp::LEAF:
+                CUDA_TRY(timed_begin(net, -1, -2, (int)batch, s, 0.0));
+                CUDA_TRY(tnc::launch_leaf_env_accum_group(bp.d_leaf + op.first, bp.d_off + op.off_first, op.n, op.blocks, slice0,
+                                                          (int)batch, s));
+                CUDA_TRY(timed_end(net, s));
+                break;
+            case BackwardOp::INV_SUM:
+            case BackwardOp::INV_READ:
+                net->launches += 1;
+                CUDA_TRY(tnc::launch_inv_env_group(bp.d_inv + op.first, bp.d_off + op.off_first, op.n, op.blocks,
+                                                   op.type == BackwardOp::INV_SUM ? (int)batch : 0, s));
+                break;
+            case BackwardOp::SEED: {
+                tnc::SeedParams sp = op.seed;
+                sp.grad = reinterpret_cast<const double2*>(grad_out);
+                net->launches += 1;
+                CUDA_TRY(tnc::launch_env_seed(sp, (int)batch, s));
+                break;
+            }
+        }
+    }
+    return TNC_OK;
+}
 
 }  // namespace tnc_host
 
@@ -389,45 +700,81 @@ tnc_status tnc_contract_backward(tnc_net_t net, int64_t lo, int64_t hi, int mode
         CUDA_TRY(cudaMemsetAsync(grad_leaves_c64, 0, net->total_leaf_elems * 8, s));
         return TNC_OK;
     }
-    // checkpoint spacing, then the largest slice batch, that fit the budget (dry runs)
-    int keep_every = 1;
-    auto need_for = [&](int64_t nb) {
-        Backward d = bw;
-        d.exec = false;
-        d.nb = nb;
-        d.keep_every = keep_every;
-        backward_run(d, lo, std::min(hi, lo + nb), grad_out_c128);
-        return (size_t)d.A.top;
-    };
-    int64_t nb = 1;
-    if (net->backward_keep_every > 0) keep_every = net->backward_keep_every;
-    else
-        while (need_for(1) > budget_bytes && keep_every < 64) keep_every *= 2;
-    if (need_for(1) > budget_bytes)
-        return fail(TNC_E_OOM, "backward workspace for one slice exceeds the budget (" +
-                                   std::to_string(need_for(1)) + " bytes)");
-    net->last_keep_every = keep_every;
-    int64_t hi_b = std::min<int64_t>(hi - lo, 1024);
-    while (nb < hi_b) {
-        int64_t nx = std::min<int64_t>(nb * 2, hi_b);
-        if (need_for(nx) > budget_bytes) break;
-        nb = nx;
+    // checkpoint spacing, then the largest slice batch, that fit the budget (dry runs;
+    // kept for calls alike)
+    const std::string mask(bw.needs.begin(), bw.needs.begin() + net->n_leaves);
+    const std::string key = plan_key(net, mode, 0) + ":" + std::to_string(budget_bytes) + ":" + std::to_string(hi - lo) + ":" +
+                            std::to_string(net->backward_keep_every) + ":" + mask;
+    auto known = net->backward_sizes.find(key);
+    if (known == net->backward_sizes.end()) {
+        BackwardSizes sz;
+        int keep_every = 1;
+        auto need_for = [&](int64_t nb) {
+            Backward d = bw;
+            d.exec = false;
+            d.nb = nb;
+            d.keep_every = keep_every;
+            backward_run(d, lo, std::min(hi, lo + nb), grad_out_c128);
+            return (size_t)d.A.top;
+        };
+        if (net->backward_keep_every > 0) keep_every = net->backward_keep_every;
+        else
+            while (need_for(1) > budget_bytes && keep_every < 64) keep_every *= 2;
+        sz.need = need_for(1);
+        sz.keep_every = keep_every;
+        if (sz.need <= budget_bytes) {
+            int64_t nb = 1;
+            const int64_t hi_b = std::min<int64_t>(hi - lo, 1024);
+            while (nb < hi_b) {
+                int64_t nx = std::min<int64_t>(nb * 2, hi_b);
+                const size_t need = need_for(nx);
+                if (need > budget_bytes) break;
+                nb = nx;
+                sz.need = need;
+            }
+            sz.nb = nb;
+            if (keep_every == 1 && T.root >= net->n_leaves) {
+                Backward d = bw;
+                BackwardPlan dry;
+                build_backward_plan(d, nb, (hi - lo) % nb, dry);
+                if ((size_t)dry.top <= budget_bytes) sz.need_levels = (size_t)dry.top;
+            }
+        }
+        if (net->backward_sizes.size() >= 64) net->backward_sizes.clear();
+        known = net->backward_sizes.emplace(key, sz).first;
     }
-    const size_t need = need_for(nb);
-    net->last_backward_bytes = need;
+    const BackwardSizes sz = known->second;
+    if (sz.nb == 0)
+        return fail(TNC_E_OOM, "backward workspace for one slice exceeds the budget (" + std::to_string(sz.need) + " bytes)");
+    net->last_keep_every = sz.keep_every;
+    const int64_t nb = sz.nb;
+    // by levels when its workspace is there or can be had
+    bool levels = sz.need_levels > 0;
+    size_t need = levels ? sz.need_levels : sz.need;
     char* ws = nullptr;
     if (net->ws_user && net->ws_user_bytes >= need) {
+        ws = (char*)net->ws_user;
+    } else if (levels && net->ws_user && net->ws_user_bytes >= sz.need) {  // the caller's fits node by node only
+        levels = false;
+        need = sz.need;
         ws = (char*)net->ws_user;
     } else {
         if (net->ws_own_bytes < need) {
             if (net->ws_own) CUDA_TRY(cudaFree(net->ws_own));
             net->ws_own = nullptr;
             net->ws_own_bytes = 0;
-            CUDA_TRY(cudaMalloc(&net->ws_own, need));
+            if (levels && need > sz.need && cudaMalloc(&net->ws_own, need) != cudaSuccess) {
+                (void)cudaGetLastError();
+                net->ws_own = nullptr;
+                levels = false;
+                need = sz.need;
+            }
+            if (!net->ws_own) CUDA_TRY(cudaMalloc(&net->ws_own, need));
             net->ws_own_bytes = need;
         }
         ws = (char*)net->ws_own;
     }
+    net->last_backward_bytes = need;
     net->last_batch = nb;
     net->group_key.clear();  // the workspace may now hold other data
     net->inv_key.clear();
@@ -435,8 +782,34 @@ tnc_status tnc_contract_backward(tnc_net_t net, int64_t lo, int64_t hi, int mode
     bw.exec = true;
     bw.nb = nb;
     bw.ws = ws;
-    bw.keep_every = keep_every;
-    if ((st = backward_run(bw, lo, hi, grad_out_c128)) != TNC_OK) return st;
+    bw.keep_every = sz.keep_every;
+    if (levels) {
+        const int64_t tail = (hi - lo) % nb;
+        const std::string pkey = plan_key(net, mode, nb) + ":" + std::to_string(tail) + ":" + std::to_string((uintptr_t)ws) +
+                                 ":" + std::to_string((uintptr_t)net->d_leaves) + ":" + mask;
+        auto it = net->backward_plans.find(pkey);
+        if (it == net->backward_plans.end()) {
+            auto bp = std::make_unique<BackwardPlan>();
+            build_backward_plan(bw, nb, tail, *bp);
+            if ((st = upload_backward_plan(*bp, s)) != TNC_OK) return st;
+            if (net->backward_plans.size() >= 4) net->backward_plans.clear();
+            it = net->backward_plans.emplace(pkey, std::move(bp)).first;
+        }
+        const BackwardPlan& bp = *it->second;
+        bw.leaf_grad = 0;
+        CUDA_TRY(cudaMemsetAsync(ws, 0, bp.zero_bytes, s));
+        auto run = [&](const std::vector<BackwardOp>& ops, int64_t batch, int64_t s0) {
+            return run_backward_ops(net, bp, ops, batch, s0, mode, grad_out_c128, ws, s);
+        };
+        if ((st = run(bp.inv_fwd, 1, 0)) != TNC_OK) return st;
+        for (int64_t s0 = lo; s0 < hi; s0 += nb) {
+            const int64_t b = std::min<int64_t>(nb, hi - s0);
+            if ((st = run(bp.slices[b < nb ? 1 : 0], b, s0)) != TNC_OK) return st;
+        }
+        if ((st = run(bp.inv_rev, 1, 0)) != TNC_OK) return st;
+    } else if ((st = backward_run(bw, lo, hi, grad_out_c128)) != TNC_OK) {
+        return st;
+    }
     CUDA_TRY(tnc::launch_f64_to_f32(reinterpret_cast<const double2*>(ws + bw.leaf_grad), net->total_leaf_elems,
                                     reinterpret_cast<float2*>(grad_leaves_c64), s));
     net->launches += 1;

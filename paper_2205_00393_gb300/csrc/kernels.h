@@ -136,7 +136,21 @@ struct LeafEnvParams {
     double2* grad;
 };
 
+// Environment (of every batch entry, n elements apart) and FP64 sum of one
+// slice-invariant tensor of n elements.
+struct InvEnvParams {
+    float2* env;
+    double2* acc;
+    int64_t n;
+};
+
 cudaError_t launch_env_seed(const SeedParams& p, int batch, cudaStream_t s);
+// Several leaves (tensors) per launch: off holds n + 1 prefix counts of blocks of 256 elements.
+cudaError_t launch_leaf_env_accum_group(const LeafEnvParams* d_params, const int64_t* d_off, int n, int64_t blocks,
+                                        int64_t slice0, int batch, cudaStream_t s);
+// batch >= 1: acc += the sum of the batch's environments; batch 0: env = acc in FP32
+cudaError_t launch_inv_env_group(const InvEnvParams* d_params, const int64_t* d_off, int n, int64_t blocks, int batch,
+                                 cudaStream_t s);
 cudaError_t launch_leaf_env_accum(const LeafEnvParams& p, int batch, cudaStream_t s);
 cudaError_t launch_accum_batch_f64(const float2* E, int64_t n, int batch, int64_t bs, double2* acc,
                                    cudaStream_t s);

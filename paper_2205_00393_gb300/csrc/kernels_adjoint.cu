@@ -34,13 +34,11 @@ __global__ void k_env_seed(const __grid_constant__ SeedParams p, int batch) {
 
 // grad[e] += sum over slices z of the batch whose sliced bits match leaf
 // element e of E_z[unsliced part of e]; one thread per leaf element, z in order.
-__global__ void k_leaf_env_accum(const __grid_constant__ LeafEnvParams p, int batch) {
-    const int64_t n = 1ll << p.L;
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
+__device__ __forceinline__ void leaf_env_accum(const LeafEnvParams& p, int64_t e, int64_t slice0, int batch) {
+    if (e >= 1ll << p.L) return;
     double ax = 0.0, ay = 0.0;
     for (int z = 0; z < batch; ++z) {
-        const int64_t s = p.slice0 + z;
+        const int64_t s = slice0 + z;
         bool ok = true;
         int64_t off = 0;
         for (int q = 0; q < p.L; ++q) {
@@ -64,10 +62,31 @@ __global__ void k_leaf_env_accum(const __grid_constant__ LeafEnvParams p, int ba
     p.grad[e].y += ay;
 }
 
+__global__ void k_leaf_env_accum(const __grid_constant__ LeafEnvParams p, int batch) {
+    leaf_env_accum(p, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, p.slice0, batch);
+}
+
+// entry of a group that block b serves: off[i] <= b < off[i + 1]
+__device__ __forceinline__ int group_entry(const int64_t* __restrict__ off, int n, int64_t b) {
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (off[mid] <= b) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+// The leaves whose environments one tree level produces, in one launch: a launch
+// per leaf took 4.4 us for 16 elements.
+__global__ void k_leaf_env_accum_group(const LeafEnvParams* __restrict__ params, const int64_t* __restrict__ off, int n,
+                                       int64_t slice0, int batch) {
+    const int i = group_entry(off, n, blockIdx.x);
+    leaf_env_accum(params[i], (blockIdx.x - off[i]) * blockDim.x + threadIdx.x, slice0, batch);
+}
+
 // acc[i] += sum_z E[z * bs + i] in FP64, z in order.
-__global__ void k_accum_batch_f64(const float2* __restrict__ E, int64_t n, int batch, int64_t bs,
-                                  double2* __restrict__ acc) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void accum_batch(const float2* E, int64_t n, int batch, int64_t bs, double2* acc, int64_t i) {
     if (i >= n) return;
     double ax = 0.0, ay = 0.0;
     for (int z = 0; z < batch; ++z) {
@@ -79,9 +98,24 @@ __global__ void k_accum_batch_f64(const float2* __restrict__ E, int64_t n, int b
     acc[i].y += ay;
 }
 
+__global__ void k_accum_batch_f64(const float2* __restrict__ E, int64_t n, int batch, int64_t bs,
+                                  double2* __restrict__ acc) {
+    accum_batch(E, n, batch, bs, acc, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+}
+
 __global__ void k_f64_to_f32(const double2* __restrict__ src, int64_t n, float2* __restrict__ dst) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) dst[i] = make_float2((float)src[i].x, (float)src[i].y);
+}
+
+// Environments of slice-invariant tensors: folded into their FP64 sums (batch >= 1),
+// or read back from them as FP32 (batch 0), several in one launch.
+__global__ void k_inv_env_group(const InvEnvParams* __restrict__ params, const int64_t* __restrict__ off, int n, int batch) {
+    const int q = group_entry(off, n, blockIdx.x);
+    const InvEnvParams p = params[q];
+    const int64_t i = (blockIdx.x - off[q]) * blockDim.x + threadIdx.x;
+    if (batch > 0) accum_batch(p.env, p.n, batch, p.n, p.acc, i);
+    else if (i < p.n) p.env[i] = make_float2((float)p.acc[i].x, (float)p.acc[i].y);
 }
 
 // out[q] = sum_e env[env_off[q] + e] * d[d_off[q] + e], e < size[q], in FP64.
@@ -123,6 +157,20 @@ cudaError_t launch_env_seed(const SeedParams& p, int batch, cudaStream_t s) {
 cudaError_t launch_leaf_env_accum(const LeafEnvParams& p, int batch, cudaStream_t s) {
     if (p.L > 31) return cudaErrorInvalidValue;
     k_leaf_env_accum<<<blocks_for(1ll << p.L), 256, 0, s>>>(p, batch);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_leaf_env_accum_group(const LeafEnvParams* d_params, const int64_t* d_off, int n, int64_t blocks,
+                                        int64_t slice0, int batch, cudaStream_t s) {
+    if (n < 1 || blocks < 1 || blocks > 0x7fffffffll) return cudaErrorInvalidConfiguration;
+    k_leaf_env_accum_group<<<(unsigned)blocks, 256, 0, s>>>(d_params, d_off, n, slice0, batch);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_inv_env_group(const InvEnvParams* d_params, const int64_t* d_off, int n, int64_t blocks, int batch,
+                                 cudaStream_t s) {
+    if (n < 1 || blocks < 1 || blocks > 0x7fffffffll) return cudaErrorInvalidConfiguration;
+    k_inv_env_group<<<(unsigned)blocks, 256, 0, s>>>(d_params, d_off, n, batch);
     return cudaGetLastError();
 }
 
