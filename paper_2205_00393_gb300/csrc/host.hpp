@@ -121,7 +121,7 @@ struct Group {
     std::vector<int> tc;     // nodes launched one by one: tensor-core nodes, and FP32 nodes that are large or of long K
     std::vector<int> stems;  // fused stem groups ending at this level (Plan::stems indices)
     int first = 0;           // first entry of the group's parameters in the table
-    int off_first = 0;       // first entry of its n + 1 tile offsets
+    int64_t map_first = 0;   // first entry of its CTA map
     int64_t tiles = 0;
     double cmacs = 0.0;      // per slice
 };
@@ -129,7 +129,7 @@ struct Group {
 struct GroupPlan {
     std::vector<Group> inv, ps;
     std::vector<tnc::GemmParams> params;
-    std::vector<int64_t> tile_off;
+    std::vector<int2> map;               // node (within its group) and tile of every CTA of the grouped launches
     std::vector<tnc::StemParams> stem_params;  // per Plan::stems entry (device copy in d_stem)
     std::vector<std::unique_ptr<tnc::StemRegParams>> stem_reg;  // the groups that run in registers (else null)
 };
@@ -154,7 +154,8 @@ struct DeviceWorkList {
 struct BackwardOp {
     enum Type { GROUP, NODE, LEAF, INV_SUM, INV_READ, SEED } type = GROUP;
     // GROUP: FP32 contractions in one launch; LEAF, INV_*: entries of the fold tables
-    int first = 0, n = 0, off_first = 0;
+    int first = 0, n = 0;
+    int64_t off_first = 0;  // first entry of its CTA map (GROUP) or of its n + 1 block offsets
     int64_t blocks = 0;
     double cmacs = 0.0;  // per batch entry
     bool per_slice = false;
@@ -169,7 +170,8 @@ struct BackwardPlan {
     std::vector<tnc::GemmParams> gemm;
     std::vector<tnc::LeafEnvParams> leaf;
     std::vector<tnc::InvEnvParams> inv;
-    std::vector<int64_t> off;                             // prefix counts of every grouped launch
+    std::vector<int64_t> off;                             // prefix counts of every grouped fold
+    std::vector<int2> map;                                // CTA maps of the grouped contractions
     int64_t top = 0;                                      // workspace bytes
     int64_t zero_bytes = 0;                               // FP64 sums at the workspace's start, leaf gradients first
     // device copies
@@ -178,6 +180,7 @@ struct BackwardPlan {
     const tnc::LeafEnvParams* d_leaf = nullptr;
     const tnc::InvEnvParams* d_inv = nullptr;
     const int64_t* d_off = nullptr;
+    const int2* d_map = nullptr;
     ~BackwardPlan() {
         if (mem) cudaFree(mem);
     }
@@ -265,8 +268,8 @@ struct tnc_net {
     std::string group_key;
     GroupPlan groups;
     tnc::GemmParams* d_params = nullptr;
-    int64_t* d_tile_off = nullptr;
-    size_t d_params_cap = 0, d_tile_cap = 0;
+    int2* d_map = nullptr;
+    size_t d_params_cap = 0, d_map_cap = 0;
     int64_t* d_pg = nullptr;  // parameter-gradient offsets
     size_t pg_cap = 0;
     // per-launch timing (tnc_set_timing) and launch accounting
@@ -294,7 +297,7 @@ struct tnc_net {
         if (d_leaves) cudaFree(d_leaves);
         if (d_err) cudaFree(d_err);
         if (d_params) cudaFree(d_params);
-        if (d_tile_off) cudaFree(d_tile_off);
+        if (d_map) cudaFree(d_map);
         if (d_pg) cudaFree(d_pg);
         if (d_stem) cudaFree(d_stem);
         if (d_stem_reg) cudaFree(d_stem_reg);

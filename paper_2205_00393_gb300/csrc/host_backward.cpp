@@ -416,15 +416,14 @@ struct LevelBuilder {
             BackwardOp op;
             op.per_slice = per_slice;
             op.first = (int)bp.gemm.size();
-            op.off_first = (int)bp.off.size();
+            op.off_first = (int64_t)bp.map.size();
             op.n = (int)grouped.size();
             for (const auto& [g, node] : grouped) {
-                bp.off.push_back(op.blocks);
-                op.blocks += tnc::gemm_f32_group_tiles(g.mb, g.nb);
-                op.cmacs += std::ldexp(1.0, g.mb + g.nb + g.kb);
                 bp.gemm.push_back(g);
+                tnc::gemm_f32_group_map(bp.map, (int)bp.gemm.size() - 1 - op.first, g.mb, g.nb);
+                op.cmacs += std::ldexp(1.0, g.mb + g.nb + g.kb);
             }
-            bp.off.push_back(op.blocks);
+            op.blocks = (int64_t)bp.map.size() - op.off_first;
             ops.push_back(op);
         }
         for (BackwardOp& op : singles) ops.push_back(std::move(op));
@@ -437,7 +436,7 @@ struct LevelBuilder {
         op.type = type;
         op.first = first;
         op.n = (int)elems.size();
-        op.off_first = (int)bp.off.size();
+        op.off_first = (int64_t)bp.off.size();
         for (int64_t n : elems) {
             bp.off.push_back(op.blocks);
             op.blocks += (n + 255) / 256;
@@ -597,7 +596,8 @@ tnc_status upload_backward_plan(BackwardPlan& bp, cudaStream_t s) {
         return o;
     };
     const size_t o_gemm = slot(bp.gemm.size() * sizeof(bp.gemm[0])), o_leaf = slot(bp.leaf.size() * sizeof(bp.leaf[0])),
-                 o_inv = slot(bp.inv.size() * sizeof(bp.inv[0])), o_off = slot(bp.off.size() * sizeof(bp.off[0]));
+                 o_inv = slot(bp.inv.size() * sizeof(bp.inv[0])), o_off = slot(bp.off.size() * sizeof(bp.off[0])),
+                 o_map = slot(bp.map.size() * sizeof(bp.map[0]));
     CUDA_TRY(cudaMalloc(&bp.mem, std::max<size_t>(off, 256)));
     char* base = static_cast<char*>(bp.mem);
     auto up = [&](size_t o, const void* src, size_t bytes) -> cudaError_t {
@@ -607,14 +607,17 @@ tnc_status upload_backward_plan(BackwardPlan& bp, cudaStream_t s) {
     CUDA_TRY(up(o_leaf, bp.leaf.data(), bp.leaf.size() * sizeof(bp.leaf[0])));
     CUDA_TRY(up(o_inv, bp.inv.data(), bp.inv.size() * sizeof(bp.inv[0])));
     CUDA_TRY(up(o_off, bp.off.data(), bp.off.size() * sizeof(bp.off[0])));
+    CUDA_TRY(up(o_map, bp.map.data(), bp.map.size() * sizeof(bp.map[0])));
     CUDA_TRY(cudaStreamSynchronize(s));  // the host vectors may go
     bp.d_gemm = reinterpret_cast<const tnc::GemmParams*>(base + o_gemm);
     bp.d_leaf = reinterpret_cast<const tnc::LeafEnvParams*>(base + o_leaf);
     bp.d_inv = reinterpret_cast<const tnc::InvEnvParams*>(base + o_inv);
     bp.d_off = reinterpret_cast<const int64_t*>(base + o_off);
+    bp.d_map = reinterpret_cast<const int2*>(base + o_map);
     bp.gemm.clear();
     bp.leaf.clear();
     bp.inv.clear();
+    bp.map.clear();
     return TNC_OK;
 }
 
@@ -626,7 +629,7 @@ tnc_status run_backward_ops(tnc_net* net, const BackwardPlan& bp, const std::vec
         switch (op.type) {
             case BackwardOp::GROUP:
                 CUDA_TRY(timed_begin(net, -1, K_GEMM_F32, b, s, op.cmacs * b));
-                CUDA_TRY(tnc::launch_gemm_f32_group(bp.d_gemm + op.first, bp.d_off + op.off_first, op.n, op.blocks, slice0, b, s));
+                CUDA_TRY(tnc::launch_gemm_f32_group(bp.d_gemm + op.first, bp.d_map + op.off_first, op.blocks, slice0, b, s));
                 CUDA_TRY(timed_end(net, s));
                 break;
             case BackwardOp::NODE: {

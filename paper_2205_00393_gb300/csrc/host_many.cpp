@@ -13,7 +13,8 @@ namespace tnc_host {
 // sequence is captured once into a CUDA graph and replayed for identical calls.
 struct ManyCall {
     struct MGroup {
-        int first = 0, n = 0, off_first = 0;
+        int first = 0, n = 0;
+        int64_t map_first = 0;
         int64_t tiles = 0;
         int max_b = 1;
         std::vector<std::pair<int, int>> singles;  // (network, node) launched one by one
@@ -33,7 +34,7 @@ struct ManyCall {
     // device tables
     void* d_mem = nullptr;
     tnc::GemmParams* d_params = nullptr;
-    int64_t* d_tile_off = nullptr;
+    int2* d_map = nullptr;
     int* d_net = nullptr;
     int64_t* d_rs0 = nullptr;
     int* d_rb = nullptr;
@@ -89,8 +90,7 @@ tnc_status many_run(ManyCall& mc, cudaStream_t s) {
                           const int64_t* h_rs0, const int* h_rb, bool per_slice) -> tnc_status {
         for (const auto& g : groups) {
             if (g.n > 0) {
-                CUDA_TRY(tnc::launch_gemm_f32_group_multi(mc.d_params + g.first, mc.d_tile_off + g.off_first, g.n,
-                                                          g.tiles, mc.d_net + g.first, rs0, rb, g.max_b, s));
+                CUDA_TRY(tnc::launch_gemm_f32_group_multi(mc.d_params + g.first, mc.d_map + g.map_first, g.tiles, mc.d_net + g.first, rs0, rb, g.max_b, s));
                 mc.kernels += 1;
             }
             for (auto [i, v] : g.singles) {
@@ -226,14 +226,13 @@ tnc_status many_build(ManyCall& mc, cudaStream_t s) {
     }
     // merged groups and their parameter tables
     std::vector<tnc::GemmParams> params;
-    std::vector<int64_t> tile_off;
+    std::vector<int2> map;
     std::vector<int> netidx;
     auto merge = [&](bool per_slice, int levels, std::vector<ManyCall::MGroup>& out) {
         for (int L = 0; L < levels; ++L) {
             ManyCall::MGroup mg;
             mg.first = (int)params.size();
-            mg.off_first = (int)tile_off.size();
-            int64_t tiles = 0;
+            mg.map_first = (int64_t)map.size();
             for (int i = 0; i < n; ++i) {
                 tnc_net* net = mc.nets[i];
                 const auto& list = per_slice ? net->groups.ps : net->groups.inv;
@@ -243,15 +242,13 @@ tnc_status many_build(ManyCall& mc, cudaStream_t s) {
                     const NodePlan& np = net->plan.nodes[g.fp32[k] - net->n_leaves];
                     params.push_back(net->groups.params[g.first + k]);
                     netidx.push_back(i);
-                    tile_off.push_back(tiles);
-                    tiles += tnc::gemm_f32_group_tiles(np.mb, np.nb);
+                    tnc::gemm_f32_group_map(map, (int)params.size() - 1 - mg.first, np.mb, np.nb);
                 }
                 for (int v : g.tc) mg.singles.emplace_back(i, v);
                 if (per_slice) mg.max_b = std::max<int>(mg.max_b, (int)mc.nb[i]);
             }
-            tile_off.push_back(tiles);
             mg.n = (int)params.size() - mg.first;
-            mg.tiles = tiles;
+            mg.tiles = (int64_t)map.size() - mg.map_first;
             out.push_back(mg);
         }
     };
@@ -295,7 +292,7 @@ tnc_status many_build(ManyCall& mc, cudaStream_t s) {
         return o;
     };
     const size_t o_params = slot(params.size() * sizeof(tnc::GemmParams));
-    const size_t o_tile = slot(tile_off.size() * sizeof(int64_t));
+    const size_t o_map = slot(map.size() * sizeof(int2));
     const size_t o_net = slot(netidx.size() * sizeof(int));
     const size_t o_rs0 = slot(mc.h_rs0.size() * sizeof(int64_t));
     const size_t o_rb = slot(mc.h_rb.size() * sizeof(int));
@@ -307,7 +304,7 @@ tnc_status many_build(ManyCall& mc, cudaStream_t s) {
     CUDA_TRY(cudaMalloc(&mc.d_mem, std::max<size_t>(off, 256)));
     char* base = (char*)mc.d_mem;
     mc.d_params = reinterpret_cast<tnc::GemmParams*>(base + o_params);
-    mc.d_tile_off = reinterpret_cast<int64_t*>(base + o_tile);
+    mc.d_map = reinterpret_cast<int2*>(base + o_map);
     mc.d_net = reinterpret_cast<int*>(base + o_net);
     mc.d_rs0 = reinterpret_cast<int64_t*>(base + o_rs0);
     mc.d_rb = reinterpret_cast<int*>(base + o_rb);
@@ -320,7 +317,7 @@ tnc_status many_build(ManyCall& mc, cudaStream_t s) {
         return bytes ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s) : cudaSuccess;
     };
     CUDA_TRY(up(mc.d_params, params.data(), params.size() * sizeof(tnc::GemmParams)));
-    CUDA_TRY(up(mc.d_tile_off, tile_off.data(), tile_off.size() * sizeof(int64_t)));
+    CUDA_TRY(up(mc.d_map, map.data(), map.size() * sizeof(int2)));
     CUDA_TRY(up(mc.d_net, netidx.data(), netidx.size() * sizeof(int)));
     CUDA_TRY(up(mc.d_rs0, mc.h_rs0.data(), mc.h_rs0.size() * sizeof(int64_t)));
     CUDA_TRY(up(mc.d_rb, mc.h_rb.data(), mc.h_rb.size() * sizeof(int)));

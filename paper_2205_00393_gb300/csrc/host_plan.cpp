@@ -693,8 +693,7 @@ tnc_status ensure_groups(tnc_net* net, const Arena& ar, char* ws, int mode, int6
     for (auto* list : {&G.inv, &G.ps}) {
         for (Group& g : *list) {
             g.first = (int)G.params.size();
-            g.off_first = (int)G.tile_off.size();
-            int64_t tiles = 0;
+            g.map_first = (int64_t)G.map.size();
             for (int v : g.fp32) {
                 const NodePlan& np = net->plan.nodes[v - net->n_leaves];
                 tnc::GemmParams gp = gemm_params(net, ar, ws, np, g.per_slice ? nb : 1);
@@ -702,12 +701,10 @@ tnc_status ensure_groups(tnc_net* net, const Arena& ar, char* ws, int mode, int6
                 gp.c_batch_stride = g.per_slice ? tensor_bytes(net->plan, np.v) / 8 : 0;
                 gp.slice0 = 0;
                 G.params.push_back(gp);
-                G.tile_off.push_back(tiles);
-                tiles += tnc::gemm_f32_group_tiles(np.mb, np.nb);
+                tnc::gemm_f32_group_map(G.map, (int)G.params.size() - 1 - g.first, np.mb, np.nb);
                 g.cmacs += std::ldexp(1.0, np.mb + np.nb + np.kb);
             }
-            G.tile_off.push_back(tiles);
-            g.tiles = tiles;
+            g.tiles = (int64_t)G.map.size() - g.map_first;
         }
     }
     std::vector<tnc::StemRegBranches> branches;
@@ -748,17 +745,17 @@ tnc_status ensure_groups(tnc_net* net, const Arena& ar, char* ws, int mode, int6
         CUDA_TRY(cudaMalloc(&net->d_params, std::max<size_t>(1, G.params.size()) * sizeof(tnc::GemmParams)));
         net->d_params_cap = G.params.size();
     }
-    if (G.tile_off.size() > net->d_tile_cap) {
-        if (net->d_tile_off) CUDA_TRY(cudaFree(net->d_tile_off));
-        net->d_tile_off = nullptr;
-        CUDA_TRY(cudaMalloc(&net->d_tile_off, std::max<size_t>(1, G.tile_off.size()) * sizeof(int64_t)));
-        net->d_tile_cap = G.tile_off.size();
+    if (G.map.size() > net->d_map_cap) {
+        if (net->d_map) CUDA_TRY(cudaFree(net->d_map));
+        net->d_map = nullptr;
+        CUDA_TRY(cudaMalloc(&net->d_map, std::max<size_t>(1, G.map.size()) * sizeof(int2)));
+        net->d_map_cap = G.map.size();
     }
     if (!G.params.empty())
         CUDA_TRY(cudaMemcpyAsync(net->d_params, G.params.data(), G.params.size() * sizeof(tnc::GemmParams),
                                  cudaMemcpyHostToDevice, s));
-    if (!G.tile_off.empty())
-        CUDA_TRY(cudaMemcpyAsync(net->d_tile_off, G.tile_off.data(), G.tile_off.size() * sizeof(int64_t),
+    if (!G.map.empty())
+        CUDA_TRY(cudaMemcpyAsync(net->d_map, G.map.data(), G.map.size() * sizeof(int2),
                                  cudaMemcpyHostToDevice, s));
     CUDA_TRY(cudaStreamSynchronize(s));  // host staging vectors are freed below
     net->groups = std::move(G);
@@ -882,8 +879,7 @@ tnc_status run_group(tnc_net* net, const Arena& ar, char* ws, const Group& g, in
     tnc_status st;
     if (!g.fp32.empty()) {
         CUDA_TRY(timed_begin(net, -1, K_GEMM_F32, b, s, g.cmacs * b));
-        CUDA_TRY(tnc::launch_gemm_f32_group(net->d_params + g.first, net->d_tile_off + g.off_first,
-                                            (int)g.fp32.size(), g.tiles, slice0, b, s));
+        CUDA_TRY(tnc::launch_gemm_f32_group(net->d_params + g.first, net->d_map + g.map_first, g.tiles, slice0, b, s));
         CUDA_TRY(timed_end(net, s));
     }
     for (int v : g.tc) {

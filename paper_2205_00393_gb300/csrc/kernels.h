@@ -15,6 +15,7 @@
 
 #include <cstdint>
 #include <string>
+#include <vector>
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -375,16 +376,21 @@ int64_t gemm_f32_group_tiles(int mb, int nb);
 // 35 us on one CTA and 14 us on a cluster; at K = 128 the difference (22 against
 // 18 us) is that of one more launch.
 bool gemm_f32_long(int kb);
-// Independent FP32 contractions in one launch; params and tile_off (n + 1
-// prefix offsets of their tile counts) are device arrays.
-cudaError_t launch_gemm_f32_group(const GemmParams* d_params, const int64_t* d_tile_off, int n,
-                                  int64_t total_tiles, int64_t slice0, int batch, cudaStream_t s);
+// Independent FP32 contractions in one launch; params and map (node and tile of
+// every CTA: gemm_f32_group_map) are device arrays.
+cudaError_t launch_gemm_f32_group(const GemmParams* d_params, const int2* d_map, int64_t total_tiles, int64_t slice0,
+                                  int batch, cudaStream_t s);
+// Appends node's tiles to a group's map.
+inline void gemm_f32_group_map(std::vector<int2>& map, int node, int mb, int nb) {
+    const int64_t tiles = gemm_f32_group_tiles(mb, nb);
+    for (int64_t t = 0; t < tiles; ++t) map.push_back(make_int2(node, (int)t));
+}
 cudaError_t launch_root_partials(const RootParams& p, int batch, double2* partials, cudaStream_t s);
 // Several networks per launch: node i of a grouped launch belongs to network
 // net[i]; rs0[w] / rb[w] are network w's first slice and batch of the round.
-cudaError_t launch_gemm_f32_group_multi(const GemmParams* d_params, const int64_t* d_tile_off, int n,
-                                        int64_t total_tiles, const int* d_net, const int64_t* d_rs0,
-                                        const int* d_rb, int max_batch, cudaStream_t s);
+cudaError_t launch_gemm_f32_group_multi(const GemmParams* d_params, const int2* d_map, int64_t total_tiles,
+                                        const int* d_net, const int64_t* d_rs0, const int* d_rb, int max_batch,
+                                        cudaStream_t s);
 // Final reductions of n networks (FP64 partials, then ordered sums into outs).
 cudaError_t launch_root_multi(const RootParams* d_roots, double2* const* d_partials, const int64_t* d_blk_off,
                               int n, int64_t total_blocks, const PermParams* d_perms, double2* const* d_outs,
