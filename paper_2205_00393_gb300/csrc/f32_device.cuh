@@ -6,6 +6,7 @@
 #pragma once
 
 #include "kernels.h"
+#include "launch.cuh"
 
 namespace tnc {
 namespace f32dev {
@@ -286,6 +287,7 @@ __device__ __forceinline__ void gemm_tile(const GemmParams& p, int64_t tile, int
     constexpr int RP = W::RP;
     const int tid = threadIdx.x;
     W w(p, tile, z, slice0, sm);
+    if constexpr (BAR == 0) dep_wait();
     bar_sync<BAR>();
     f32x2 acc[2][RP][4], part[2][RP][4];
 #pragma unroll
@@ -401,6 +403,7 @@ __device__ __forceinline__ void gemm_tile_cluster(const GemmParams& p, int64_t t
         w.khA = bits_offset(k, p.ak, p.kb, LOG_BK);
         w.khB = bits_offset(k, p.bk, p.kb, LOG_BK);
     };
+    dep_wait();
     __syncthreads();
     seek(0);
     w.gather();

@@ -9,6 +9,7 @@
 // environments of slice-invariant tensors, and apply the chain rule to gate
 // parameters. Accumulation over slices is FP64.
 #include "kernels.h"
+#include "launch.cuh"
 
 namespace tnc {
 
@@ -23,6 +24,8 @@ __device__ __forceinline__ int64_t bits_offset(int64_t x, const int64_t* str, in
 
 // E_z[root offset of r] = g[r] for every slice z of the batch (FP32).
 __global__ void k_env_seed(const __grid_constant__ SeedParams p, int batch) {
+    dep_trigger();
+    dep_wait();
     const int64_t R = 1ll << p.obits;
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= R) return;
@@ -63,6 +66,8 @@ __device__ __forceinline__ void leaf_env_accum(const LeafEnvParams& p, int64_t e
 }
 
 __global__ void k_leaf_env_accum(const __grid_constant__ LeafEnvParams p, int batch) {
+    dep_trigger();
+    dep_wait();
     leaf_env_accum(p, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, p.slice0, batch);
 }
 
@@ -81,6 +86,8 @@ __device__ __forceinline__ int group_entry(const int64_t* __restrict__ off, int 
 // per leaf took 4.4 us for 16 elements.
 __global__ void k_leaf_env_accum_group(const LeafEnvParams* __restrict__ params, const int64_t* __restrict__ off, int n,
                                        int64_t slice0, int batch) {
+    dep_trigger();
+    dep_wait();
     const int i = group_entry(off, n, blockIdx.x);
     leaf_env_accum(params[i], (blockIdx.x - off[i]) * blockDim.x + threadIdx.x, slice0, batch);
 }
@@ -98,12 +105,15 @@ __device__ __forceinline__ void accum_batch(const float2* E, int64_t n, int batc
     acc[i].y += ay;
 }
 
-__global__ void k_accum_batch_f64(const float2* __restrict__ E, int64_t n, int batch, int64_t bs,
-                                  double2* __restrict__ acc) {
+__global__ void k_accum_batch_f64(const float2* E, int64_t n, int batch, int64_t bs, double2* acc) {
+    dep_trigger();
+    dep_wait();
     accum_batch(E, n, batch, bs, acc, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
-__global__ void k_f64_to_f32(const double2* __restrict__ src, int64_t n, float2* __restrict__ dst) {
+__global__ void k_f64_to_f32(const double2* src, int64_t n, float2* dst) {
+    dep_trigger();
+    dep_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) dst[i] = make_float2((float)src[i].x, (float)src[i].y);
 }
@@ -111,6 +121,8 @@ __global__ void k_f64_to_f32(const double2* __restrict__ src, int64_t n, float2*
 // Environments of slice-invariant tensors: folded into their FP64 sums (batch >= 1),
 // or read back from them as FP32 (batch 0), several in one launch.
 __global__ void k_inv_env_group(const InvEnvParams* __restrict__ params, const int64_t* __restrict__ off, int n, int batch) {
+    dep_trigger();
+    dep_wait();
     const int q = group_entry(off, n, blockIdx.x);
     const InvEnvParams p = params[q];
     const int64_t i = (blockIdx.x - off[q]) * blockDim.x + threadIdx.x;
@@ -150,39 +162,33 @@ unsigned blocks_for(int64_t n) { return (unsigned)((n + 255) / 256); }
 }  // namespace
 
 cudaError_t launch_env_seed(const SeedParams& p, int batch, cudaStream_t s) {
-    k_env_seed<<<blocks_for(1ll << p.obits), 256, 0, s>>>(p, batch);
-    return cudaGetLastError();
+    return launch_dependent(k_env_seed, dim3(blocks_for(1ll << p.obits)), dim3(256), 0, s, 1, p, batch);
 }
 
 cudaError_t launch_leaf_env_accum(const LeafEnvParams& p, int batch, cudaStream_t s) {
     if (p.L > 31) return cudaErrorInvalidValue;
-    k_leaf_env_accum<<<blocks_for(1ll << p.L), 256, 0, s>>>(p, batch);
-    return cudaGetLastError();
+    return launch_dependent(k_leaf_env_accum, dim3(blocks_for(1ll << p.L)), dim3(256), 0, s, 1, p, batch);
 }
 
 cudaError_t launch_leaf_env_accum_group(const LeafEnvParams* d_params, const int64_t* d_off, int n, int64_t blocks,
                                         int64_t slice0, int batch, cudaStream_t s) {
     if (n < 1 || blocks < 1 || blocks > 0x7fffffffll) return cudaErrorInvalidConfiguration;
-    k_leaf_env_accum_group<<<(unsigned)blocks, 256, 0, s>>>(d_params, d_off, n, slice0, batch);
-    return cudaGetLastError();
+    return launch_dependent(k_leaf_env_accum_group, dim3((unsigned)blocks), dim3(256), 0, s, 1, d_params, d_off, n, slice0, batch);
 }
 
 cudaError_t launch_inv_env_group(const InvEnvParams* d_params, const int64_t* d_off, int n, int64_t blocks, int batch,
                                  cudaStream_t s) {
     if (n < 1 || blocks < 1 || blocks > 0x7fffffffll) return cudaErrorInvalidConfiguration;
-    k_inv_env_group<<<(unsigned)blocks, 256, 0, s>>>(d_params, d_off, n, batch);
-    return cudaGetLastError();
+    return launch_dependent(k_inv_env_group, dim3((unsigned)blocks), dim3(256), 0, s, 1, d_params, d_off, n, batch);
 }
 
 cudaError_t launch_accum_batch_f64(const float2* E, int64_t n, int batch, int64_t bs, double2* acc,
                                    cudaStream_t s) {
-    k_accum_batch_f64<<<blocks_for(n), 256, 0, s>>>(E, n, batch, bs, acc);
-    return cudaGetLastError();
+    return launch_dependent(k_accum_batch_f64, dim3(blocks_for(n)), dim3(256), 0, s, 1, E, n, batch, bs, acc);
 }
 
 cudaError_t launch_f64_to_f32(const double2* src, int64_t n, float2* dst, cudaStream_t s) {
-    k_f64_to_f32<<<blocks_for(n), 256, 0, s>>>(src, n, dst);
-    return cudaGetLastError();
+    return launch_dependent(k_f64_to_f32, dim3(blocks_for(n)), dim3(256), 0, s, 1, src, n, dst);
 }
 
 cudaError_t launch_param_grads(int n, const int64_t* env_off, const int64_t* d_off, const int64_t* size,

@@ -19,12 +19,14 @@ using namespace f32dev;
 
 template <int NTH, int RM, int WN, int MINB>
 __global__ void __launch_bounds__(NTH, MINB) k_gemm_f32(const __grid_constant__ GemmParams p) {
+    dep_trigger();
     extern __shared__ __align__(16) uint8_t gemm_dyn[];
     gemm_tile<0, NTH, RM, WN>(p, blockIdx.x, blockIdx.z, p.slice0, *reinterpret_cast<GemmSmemT<NTH, RM, WN>*>(gemm_dyn));
 }
 
 template <int NTH, int WN, int CL>
 __global__ void __launch_bounds__(NTH, 3) k_gemm_f32_cluster(const __grid_constant__ GemmParams p) {
+    dep_trigger();
     extern __shared__ __align__(16) uint8_t gemm_dyn[];
     gemm_tile_cluster<NTH, WN, CL>(p, blockIdx.x / CL, blockIdx.x % CL, blockIdx.z, p.slice0,
                                    *reinterpret_cast<GemmClusterSmem<NTH, WN>*>(gemm_dyn));
@@ -61,6 +63,7 @@ __device__ __forceinline__ const GemmParams& stage_params(const GemmParams* src,
 // b serves tile map[b].y of node map[b].x.
 __global__ void __launch_bounds__(GT, 4) k_gemm_f32_group(const GemmParams* __restrict__ params,
                                                        const int2* __restrict__ map, int64_t slice0) {
+    dep_trigger();
     extern __shared__ __align__(16) uint8_t gemm_dyn[];
     GroupCta& cta = *reinterpret_cast<GroupCta*>(gemm_dyn);
     const int2 nt = map[blockIdx.x];
@@ -70,6 +73,8 @@ __global__ void __launch_bounds__(GT, 4) k_gemm_f32_group(const GemmParams* __re
 // FP64 partial sums of a contraction with R = M*N <= 64 outputs.
 __global__ void __launch_bounds__(256) k_root_partials(const __grid_constant__ RootParams rp,
                                                        double2* __restrict__ partials) {
+    dep_trigger();
+    dep_wait();
     __shared__ double2 red[256];
     __shared__ int64_t root_ta[5][256], root_tb[5][256];  // offsets of 8-bit groups of j (K <= 2^40)
     const int R = 1 << (rp.g.mb + rp.g.nb);
@@ -79,15 +84,19 @@ __global__ void __launch_bounds__(256) k_root_partials(const __grid_constant__ R
 }
 
 // out[r] += sum_i partials[i][perm(r)] (a fixed order: accumulate_items)
-__global__ void __launch_bounds__(256) k_accumulate_partials(const double2* __restrict__ partials, int count,
+__global__ void __launch_bounds__(256) k_accumulate_partials(const double2* partials, int count,
                                                              const __grid_constant__ PermParams pp,
                                                              double2* __restrict__ out) {
+    dep_trigger();
+    dep_wait();
     __shared__ double2 red[256];
     accumulate_items<0>(partials, count, pp, (int64_t)blockIdx.x * 256, out, red);
 }
 
 // out[r] += sum_z src_z[perm(r)] in FP64, z ascending
 __global__ void k_slice_sum_f32(const __grid_constant__ SumParams p, int batch, double2* __restrict__ out) {
+    dep_trigger();
+    dep_wait();
     const int64_t R = 1ll << p.obits;
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= R) return;
@@ -134,8 +143,7 @@ static cudaError_t launch_gemm_f32_tiles(const GemmParams& p, int batch, cudaStr
     const int64_t M = 1ll << p.mb, N = 1ll << p.nb;
     const int64_t tiles = ((M + Cfg::BM - 1) / Cfg::BM) * ((N + Cfg::BN - 1) / Cfg::BN);
     if (tiles > 0x7fffffffll || batch < 1 || batch > 65535) return cudaErrorInvalidConfiguration;
-    k_gemm_f32<NTH, RM, WN, MINB><<<dim3((unsigned)tiles, 1, batch), NTH, sizeof(Smem), s>>>(p);
-    return cudaGetLastError();
+    return launch_dependent(k_gemm_f32<NTH, RM, WN, MINB>, dim3((unsigned)tiles, 1, batch), dim3(NTH), sizeof(Smem), s, 1, p);
 }
 
 template <int NTH, int WN, int CL>
@@ -148,18 +156,8 @@ static cudaError_t launch_gemm_f32_cluster(const GemmParams& p, int batch, cudaS
     const int64_t M = 1ll << p.mb, N = 1ll << p.nb;
     const int64_t tiles = ((M + Cfg::BM - 1) / Cfg::BM) * ((N + Cfg::BN - 1) / Cfg::BN);
     if (tiles > 0x7fffffffll / CL || batch < 1 || batch > 65535) return cudaErrorInvalidConfiguration;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(tiles * CL), 1, batch);
-    cfg.blockDim = dim3(NTH);
-    cfg.dynamicSmemBytes = sizeof(Smem);
-    cfg.stream = s;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = CL;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_gemm_f32_cluster<NTH, WN, CL>, p);
+    return launch_dependent(k_gemm_f32_cluster<NTH, WN, CL>, dim3((unsigned)(tiles * CL), 1, batch), dim3(NTH), sizeof(Smem),
+                            s, CL, p);
 }
 
 // Choice of the tile, by the number T of CTAs that 32 x 64 tiles (64 x 32 where
@@ -207,11 +205,15 @@ __global__ void __launch_bounds__(GT, 4) k_gemm_f32_group_multi(const GemmParams
                                                              const int2* __restrict__ map, const int* __restrict__ net,
                                                              const int64_t* __restrict__ rs0,
                                                              const int* __restrict__ rb) {
+    dep_trigger();
     extern __shared__ __align__(16) uint8_t gemm_dyn[];
     GroupCta& cta = *reinterpret_cast<GroupCta*>(gemm_dyn);
     const int2 nt = map[blockIdx.x];
     const int w = net[nt.x];
-    if ((int)blockIdx.z >= rb[w]) return;
+    if ((int)blockIdx.z >= rb[w]) {
+        dep_wait();
+        return;
+    }
     gemm_tile<0, GT, 4, 2>(stage_params(params + nt.x, cta), nt.y, blockIdx.z, rs0[w], cta.tile);
 }
 
@@ -222,6 +224,8 @@ __global__ void __launch_bounds__(256) k_root_partials_multi(const RootParams* _
                                                              const int64_t* __restrict__ blk_off, int n,
                                                              const int64_t* __restrict__ rs0,
                                                              const int* __restrict__ rb) {
+    dep_trigger();
+    dep_wait();
     __shared__ double2 red[256];
     __shared__ int64_t root_ta[5][256], root_tb[5][256];
     const int64_t x = blockIdx.x;
@@ -245,6 +249,8 @@ __global__ void __launch_bounds__(256) k_accumulate_multi(const RootParams* __re
                                                           double2* const* __restrict__ partials,
                                                           const PermParams* __restrict__ perms,
                                                           double2* const* __restrict__ outs, const int* __restrict__ rb) {
+    dep_trigger();
+    dep_wait();
     __shared__ double2 red[256];
     const int i = blockIdx.x;
     const PermParams& pp = perms[i];
@@ -270,8 +276,8 @@ cudaError_t launch_gemm_f32_group(const GemmParams* d_params, const int2* d_map,
     if (total_tiles < 1 || total_tiles > 0x7fffffffll || batch < 1 || batch > 65535) return cudaErrorInvalidConfiguration;
     cudaError_t e = gemm_smem_attr();
     if (e != cudaSuccess) return e;
-    k_gemm_f32_group<<<dim3((unsigned)total_tiles, 1, batch), GT, sizeof(GroupCta), s>>>(d_params, d_map, slice0);
-    return cudaGetLastError();
+    return launch_dependent(k_gemm_f32_group, dim3((unsigned)total_tiles, 1, batch), dim3(GT), sizeof(GroupCta), s, 1, d_params,
+                            d_map, slice0);
 }
 
 cudaError_t launch_gemm_f32_group_multi(const GemmParams* d_params, const int2* d_map, int64_t total_tiles,
@@ -281,9 +287,8 @@ cudaError_t launch_gemm_f32_group_multi(const GemmParams* d_params, const int2* 
         return cudaErrorInvalidConfiguration;
     cudaError_t e = gemm_smem_attr();
     if (e != cudaSuccess) return e;
-    k_gemm_f32_group_multi<<<dim3((unsigned)total_tiles, 1, max_batch), GT, sizeof(GroupCta), s>>>(d_params, d_map, d_net,
-                                                                                                d_rs0, d_rb);
-    return cudaGetLastError();
+    return launch_dependent(k_gemm_f32_group_multi, dim3((unsigned)total_tiles, 1, max_batch), dim3(GT), sizeof(GroupCta), s, 1,
+                            d_params, d_map, d_net, d_rs0, d_rb);
 }
 
 cudaError_t launch_root_multi(const RootParams* d_roots, double2* const* d_partials, const int64_t* d_blk_off,
@@ -291,31 +296,27 @@ cudaError_t launch_root_multi(const RootParams* d_roots, double2* const* d_parti
                               const int64_t* d_rs0, const int* d_rb, int max_batch, cudaStream_t s) {
     if (n < 1 || total_blocks < 1 || total_blocks > 0x7fffffffll || max_batch < 1 || max_batch > 65535)
         return cudaErrorInvalidConfiguration;
-    k_root_partials_multi<<<dim3((unsigned)total_blocks, 1, max_batch), 256, 0, s>>>(d_roots, d_partials, d_blk_off,
-                                                                                   n, d_rs0, d_rb);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_dependent(k_root_partials_multi, dim3((unsigned)total_blocks, 1, max_batch), dim3(256), 0, s, 1, d_roots,
+                                     d_partials, d_blk_off, n, d_rs0, d_rb);
     if (e != cudaSuccess) return e;
-    k_accumulate_multi<<<n, 256, 0, s>>>(d_roots, d_partials, d_perms, d_outs, d_rb);
-    return cudaGetLastError();
+    return launch_dependent(k_accumulate_multi, dim3(n), dim3(256), 0, s, 1, d_roots, d_partials, d_perms, d_outs, d_rb);
 }
 
 cudaError_t launch_root_partials(const RootParams& p, int batch, double2* partials, cudaStream_t s) {
     if (p.g.mb + p.g.nb > 6 || batch < 1 || batch > 65535) return cudaErrorInvalidConfiguration;
-    k_root_partials<<<dim3(p.chunks, batch), 256, 0, s>>>(p, partials);
-    return cudaGetLastError();
+    return launch_dependent(k_root_partials, dim3(p.chunks, batch), dim3(256), 0, s, 1, p, partials);
 }
 
 cudaError_t launch_accumulate_partials(const double2* partials, int count, const PermParams& pp,
                                        double2* out, cudaStream_t s) {
     const int64_t items = (int64_t)acc_lanes(count) << pp.obits;
-    k_accumulate_partials<<<(unsigned)((items + 255) / 256), 256, 0, s>>>(partials, count, pp, out);
-    return cudaGetLastError();
+    return launch_dependent(k_accumulate_partials, dim3((unsigned)((items + 255) / 256)), dim3(256), 0, s, 1, partials, count, pp,
+                            out);
 }
 
 cudaError_t launch_slice_sum_f32(const SumParams& p, int batch, double2* out, cudaStream_t s) {
     int64_t R = 1ll << p.obits;
-    k_slice_sum_f32<<<(unsigned)((R + 255) / 256), 256, 0, s>>>(p, batch, out);
-    return cudaGetLastError();
+    return launch_dependent(k_slice_sum_f32, dim3((unsigned)((R + 255) / 256)), dim3(256), 0, s, 1, p, batch, out);
 }
 
 }  // namespace tnc

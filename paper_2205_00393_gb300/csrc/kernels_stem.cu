@@ -10,6 +10,7 @@
 #include <type_traits>
 
 #include "kernels.h"
+#include "launch.cuh"
 
 namespace tnc {
 
@@ -85,6 +86,7 @@ __device__ __forceinline__ void inplace_step(float2* cur, const float2* bd, cons
 // X_i) and the dense [K][N] copies of every step's branch.
 __global__ void __launch_bounds__(NT, 4) k_stem_fused(const StemParams* __restrict__ P, int cap_log2,
                                                    int64_t slice0) {
+    dep_wait();
     extern __shared__ float2 stem_smem[];
     const StemParams& p = *P;
     float2* cur = stem_smem;
@@ -368,6 +370,7 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_stem_reg(const __grid_consta
             ib += p.ustr_in[b];
             ob += p.ustr_out[b];
         }
+    dep_wait();
     float2 x[RE];
     for (int q = 0; q < p.npass; ++q) {
         const StemRegPass& ps = p.pass[q];
@@ -387,7 +390,7 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_stem_reg(const __grid_consta
 #pragma unroll
                 for (int a = 0; a < kStemRegBits; ++a) st[a] = p.rstr_in[a];
                 reg_walk(g, st, ps.unborn,
-                         [&](int r, uint64_t a) { x[r] = __ldg(reinterpret_cast<const float2*>(a)); });
+                         [&](int r, uint64_t a) { x[r] = *reinterpret_cast<const float2*>(a); });
             }
             // dense copies of this slice's branches, while the loads are in flight
             for (int e = tid; e < p.nentries; e += NTH) {
@@ -446,8 +449,7 @@ cudaError_t launch_stem_reg_impl(const StemRegParams& p, const StemRegBranches* 
         k_stem_reg<NTH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
         (int)(((NTH * RE > (1 << kStemRegMinN) ? NTH * RE : (1 << kStemRegMinN)) + kStemRegMaxEntries) * sizeof(float2)));
     if (attr != cudaSuccess) return attr;
-    k_stem_reg<NTH><<<dim3(1u << p.nu, 1, batch), NTH, smem, s>>>(p, br, slice0);
-    return cudaGetLastError();
+    return launch_dependent(k_stem_reg<NTH>, dim3(1u << p.nu, 1, batch), dim3(NTH), smem, s, 1, p, br, slice0);
 }
 
 }  // namespace
@@ -485,8 +487,7 @@ cudaError_t launch_stem_fused(const StemParams* d_params, const StemParams& hp, 
         if (e != cudaSuccess) return e;
         set_for = (int)smem;
     }
-    k_stem_fused<<<dim3(1u << hp.nu, 1, batch), NT, smem, s>>>(d_params, cap_log2, slice0);
-    return cudaGetLastError();
+    return launch_dependent(k_stem_fused, dim3(1u << hp.nu, 1, batch), dim3(NT), smem, s, 1, d_params, cap_log2, slice0);
 }
 
 namespace {

@@ -538,6 +538,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                const __grid_constant__ TcGemmParams p) {
     extern __shared__ __align__(1024) uint8_t dsmem[];
     __shared__ TcShared sh;
+    if (gridDim.x * gridDim.y * gridDim.z <= 152) dep_trigger();  // a single wave
     const int warp = threadIdx.x >> 5;
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dsmem) + 1023) & ~uintptr_t(1023));
     if (threadIdx.x == 0) tc_init(sh);
@@ -552,6 +553,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = sh.tmem_base;
     TcPipe pipe;
+    dep_wait();
     tc_tile<KIND, ROWB>(&tmA, &tmB, p, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z, smem, sh, tmem, pipe);
     __syncthreads();
     if (warp == MMA_WARP) {
@@ -694,6 +696,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     cluster_sync();  // both CTAs' barriers are initialised
+    dep_wait();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = sh.tmem_base;
 
@@ -1143,6 +1146,7 @@ __device__ __forceinline__ void split_one_block(const SplitParams& p, int64_t bl
     const float2* src = p.src.ptr + z * p.src.batch_stride + slice_offset(p.src, slice0 + z);
     float4 v[8];
     split_offsets(p, g, block, roff, koff);
+    if constexpr (BAR == 0) dep_wait();
     tc_bar<BAR>();
     split_gather(p, g, src, roff, koff, v);
     split_stage(p, g, v, tile);
@@ -1196,6 +1200,7 @@ __device__ __forceinline__ void split_blocks(const SplitParams& p, int64_t block
 
 template <int KIND>
 __global__ void __launch_bounds__(256) k_split_operand(const __grid_constant__ SplitParams p) {
+    dep_trigger();
     extern __shared__ float2 tile[];
     __shared__ int64_t roff[128], koff[256];
     split_one_block<KIND, 0>(p, blockIdx.x, blockIdx.z, p.slice0, tile, roff, koff);
@@ -1204,9 +1209,11 @@ __global__ void __launch_bounds__(256) k_split_operand(const __grid_constant__ S
 // ------------------------------------------------------------ K-split reduction
 // C[z][m][n] (+)= sum over splits, in order, of partial[split][z][m][n]: FP64
 // sums rounded once, two complex elements per thread step.
-__global__ void __launch_bounds__(256) k_ksplit_reduce(const float4* __restrict__ partial, int nsplit, int batch,
+__global__ void __launch_bounds__(256) k_ksplit_reduce(const float4* partial, int nsplit, int batch,
                                                        int64_t mn2, int nb, float2* C, int64_t c_batch_stride,
                                                        int64_t c_ld, int accumulate) {
+    dep_trigger();
+    dep_wait();
     const int z = blockIdx.y;
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < mn2; i += (int64_t)gridDim.x * 256) {
         double a0 = 0, a1 = 0, a2 = 0, a3 = 0;
@@ -1290,8 +1297,8 @@ cudaError_t launch_tc_impl(const TcGemmParams& p, const void* planesA, const voi
     const int64_t kcta = K >> p.ksplit_bits;  // K of one CTA: whole k-blocks, whole chunks
     if (kcta < C_::BK || (kcta > KC_ELEMS && kcta % KC_ELEMS) || (p.ksplit_bits && (!p.partial || p.accumulate)))
         return cudaErrorInvalidValue;
-    k_cgemm_tc<KIND, ROWB><<<dim3((unsigned)tiles, 1u << p.ksplit_bits, batch), NTHREADS, smem, s>>>(ta, tb, p);
-    return cudaGetLastError();
+    return launch_dependent(k_cgemm_tc<KIND, ROWB>, dim3((unsigned)tiles, 1u << p.ksplit_bits, batch), dim3(NTHREADS), smem, s, 1,
+                            ta, tb, p);
 }
 
 template <int KIND, int ROWB>
@@ -1313,8 +1320,7 @@ cudaError_t launch_pair_impl(const TcGemmParams& p, const void* planesA, const v
         return cudaErrorInvalidValue;
     const int64_t items = ((int64_t)batch << p.ksplit_bits) << (p.mb - 8 + p.nb - 7);
     const int64_t pairs = items < sms / 2 ? items : sms / 2;
-    k_cgemm_pair<KIND, ROWB><<<dim3((unsigned)(2 * pairs)), NTHREADS, C_::SMEM, s>>>(ta, tb, p, batch);
-    return cudaGetLastError();
+    return launch_dependent(k_cgemm_pair<KIND, ROWB>, dim3((unsigned)(2 * pairs)), dim3(NTHREADS), C_::SMEM, s, 1, ta, tb, p, batch);
 }
 
 // Pairs from one item per two SMs on, or for K of at least 1024 per item: below
@@ -1619,15 +1625,13 @@ cudaError_t launch_split(const SplitParams& p_in, int mode, int batch, cudaStrea
     const dim3 grid((unsigned)blocks, 1, batch);
     const size_t smem = (size_t)SR * split_ld((int)SK) * sizeof(float2);
     switch (kind_of(mode)) {
-        case 0: k_split_operand<0><<<grid, 256, smem, s>>>(p); break;
-        case 1: k_split_operand<1><<<grid, 256, smem, s>>>(p); break;
+        case 0: return launch_dependent(k_split_operand<0>, grid, dim3(256), smem, s, 1, p);
+        case 1: return launch_dependent(k_split_operand<1>, grid, dim3(256), smem, s, 1, p);
         case 3:
             if (!p.sexp) return cudaErrorInvalidValue;
-            k_split_operand<3><<<grid, 256, smem, s>>>(p);
-            break;
-        default: k_split_operand<2><<<grid, 256, smem, s>>>(p); break;
+            return launch_dependent(k_split_operand<3>, grid, dim3(256), smem, s, 1, p);
+        default: return launch_dependent(k_split_operand<2>, grid, dim3(256), smem, s, 1, p);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_ksplit_reduce(const float2* partial, int ksplit_bits, int batch, int mb, int nb, float2* C,
@@ -1636,9 +1640,8 @@ cudaError_t launch_ksplit_reduce(const float2* partial, int ksplit_bits, int bat
     const int64_t mn2 = (1ll << (mb + nb)) / 2;  // float4 steps of two complex elements
     const int64_t want = (mn2 + 255) / 256;
     const unsigned blocks = (unsigned)(want < 152 * 16 ? want : 152 * 16);
-    k_ksplit_reduce<<<dim3(blocks, batch), 256, 0, s>>>(reinterpret_cast<const float4*>(partial), 1 << ksplit_bits,
-                                                        batch, mn2, nb, C, c_batch_stride, c_ld, accumulate);
-    return cudaGetLastError();
+    return launch_dependent(k_ksplit_reduce, dim3(blocks, batch), dim3(256), 0, s, 1, reinterpret_cast<const float4*>(partial),
+                            1 << ksplit_bits, batch, mn2, nb, C, c_batch_stride, c_ld, accumulate);
 }
 
 cudaError_t launch_persist(const PersistParams& p, int mode, cudaStream_t s) {
