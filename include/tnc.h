@@ -351,7 +351,13 @@ tnc_status tnc_worklist_many_json(int n, const tnc_net_t* nets, int64_t batch, i
  *                  for the tasks that produce its inputs (see
  *                  "persist_deps"). Results equal the per-level launches' up to
  *                  the order of FP32 additions in a K split; other calls, and
- *                  0, use one launch per tree level. 2: the persistent
+ *                  0, use one launch per tree level. 2: tnc_contract and
+ *                  tnc_contract_variants run a network whose leaves,
+ *                  intermediates and tables fit one CTA's shared memory with
+ *                  a CTA per slice, every slice of every variant in one
+ *                  launch and a sum (timing record of kind 9), if a slice
+ *                  has at most 3 2^16 complex multiply-accumulates (3 2^17
+ *                  for calls of 64 slices and more); the persistent
  *                  executor when the per-level launches of a batch would
  *                  carry less than 0.1 us of work each on average (a
  *                  contraction estimated at the larger of its flops at 300
@@ -414,8 +420,8 @@ tnc_status tnc_set_timing(tnc_net_t net, int enable);
  * launch the node's tensor id, kernel kind (0 FP32 GEMM, 1 FP64 root reduction,
  * 2 GEMM root + FP64 slice sum, 3 tensor-core GEMM, 4 operand split,
  * 7 reduction of a tensor-core GEMM's K-split partials, 8 fused stem group (node = its
- * output tensor), 9 persistent executor (node -1; one launch per slice batch), -1 leaf
- * slice sum), slice batch, complex multiply-accumulates of the
+ * output tensor), 9 persistent executor (node -1; one launch per slice batch) or a network
+ * on one CTA per slice ("persistent" = 2; node -1), -1 leaf slice sum), slice batch, complex multiply-accumulates of the
  * launch (all its nodes and slices) and milliseconds; a grouped launch of
  * several nodes of one tree level reports node -1. Any output array may be NULL. *n_out receives the number
  * of records (TNC_E_INVALID if it exceeds cap); *n_launches (may be NULL) the

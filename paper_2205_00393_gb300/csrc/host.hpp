@@ -149,6 +149,21 @@ struct DeviceWorkList {
     }
 };
 
+// A tiny network's tables on the device (host_tiny.cpp); no memory: the network
+// does not run that way.
+struct TinyPlan {
+    tnc::TinyParams prm{};
+    void* mem = nullptr;
+    double cmacs = 0;  // of a slice, invariants included
+    // what the last call's sizes come to for the other executors (statistics; a
+    // workspace that is too small stays an error): slices asked for, workspace given
+    int64_t want = -1, nb = 0;
+    size_t given = 0, arena[2] = {0, 0};
+    ~TinyPlan() {
+        if (mem) cudaFree(mem);
+    }
+};
+
 // The adjoint pass of a plan by tree levels (host_backward.cpp): its launches in
 // order, with their parameters in device tables.
 struct BackwardOp {
@@ -288,6 +303,9 @@ struct tnc_net {
     mutable std::map<std::string, Arena> arena_cache;  // plan_arena results by their inputs
     std::map<std::string, std::pair<double, double>> cost_cache;  // level_cost results (launches, seconds)
     std::map<std::string, std::unique_ptr<DeviceWorkList>> worklists;
+    std::map<std::string, std::unique_ptr<TinyPlan>> tiny_plans;
+    double2* d_tiny = nullptr;       // its partial results
+    size_t d_tiny_cap = 0;
     std::map<std::string, BackwardSizes> backward_sizes;                     // by what they depend on
     std::map<std::string, std::unique_ptr<BackwardPlan>> backward_plans;     // and the workspace
     double timed_persist_tc_cmacs = 0.0;  // tensor-core share of the timed persistent launches
@@ -304,6 +322,7 @@ struct tnc_net {
         if (ws_own) cudaFree(ws_own);
         if (d_prof) cudaFree(d_prof);
         if (d_var) cudaFree(d_var);
+        if (d_tiny) cudaFree(d_tiny);
         for (cudaEvent_t e : ev_pool) cudaEventDestroy(e);
     }
 };
@@ -450,6 +469,14 @@ tnc_status wl_upload(const WorkList& W, DeviceWorkList& D, int* err, uint64_t wa
 cudaError_t wl_launch(const DeviceWorkList& D, int mode, int64_t slice0, const int64_t* rs0, cudaStream_t s, unsigned long long* prof, double* out0);
 bool wl_validate(const tnc_net* net, const WorkList& W, const char* ws, size_t ws_bytes, const double* out, int mode, std::string* why);
 DeviceWorkList* contract_worklist(tnc_net* net, const Arena& ar, char* ws, int b, int mode, bool with_inv, double* out, cudaStream_t s, tnc_status* st);
+
+// Slices per batch of a call of `want` slices, 0 if the given workspace does not hold one.
+int64_t call_batch(const tnc_net* net, int64_t want, int mode);
+
+// tiny networks (host_tiny.cpp): slice ids first + g stride + j (j < per) summed into
+// result g < groups; *done false: the network or the call is not for it
+tnc_status tiny_contract(tnc_net* net, int mode, int64_t first, int64_t stride, int64_t per, int64_t groups, double2* out,
+                         cudaStream_t s, bool* done);
 
 // many-network calls (host_many.cpp)
 void many_forget(uint64_t uid);

@@ -13,6 +13,7 @@
 // the operand load, never a separate pass. The output is row-major [m][n].
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -361,6 +362,35 @@ bool tc_make_node(TcNode* node, const TcGemmParams& p, int mode, const void* pla
 int64_t tc_node_tiles(const TcGemmParams& p);
 // Split blocks of one batch entry; the split's pair-load flag is set.
 int64_t tc_split_prepare(SplitParams& p);
+
+// ------------------------------------------------- tiny networks
+//
+// A network whose leaves, intermediates and tables fit one CTA's shared memory
+// (kernels_tiny.cu). The tables are 32-bit words: per contraction kTinyOpWords
+// [A, B: tensors; output: element offset; mb | nb << 8 | kb << 16; first words of the
+// row offsets of A, of the column offsets of B, of the K offsets (A's | B's << 16);
+// first item of its level]; per level [items, first word of its map], the map
+// naming the contraction of every four items (16 bits each).
+constexpr int kTinyThreads = 512;
+constexpr int kTinyOpWords = 8;
+constexpr size_t kTinySmem = 200 * 1024;
+
+struct TinyParams {
+    const float2* leaves;
+    const float2* variants;
+    const uint32_t* tables;
+    int words, data_elems, leaf_elems;
+    int inv_levels, levels;      // slice-invariant levels first
+    int o_ops, o_levels, o_base, o_static, o_sliced, n_sliced, o_var, n_var, o_root;
+    // slice ids first + g * stride + j, j < per, for groups g, each with a result of its own
+    int64_t first, stride, per, groups;
+    int sbits, obits;            // variant = slice id >> sbits; 2^obits outputs
+    double2* partials;           // [groups * per][outputs]
+    double2* out;                // [groups][outputs]
+    int* err;                    // cleared (nothing here waits on another CTA)
+};
+size_t tiny_smem_bytes(int64_t data_elems, int64_t words);
+cudaError_t launch_tiny(const TinyParams& p, const PermParams& pp, cudaStream_t s);
 
 // Message returned by tnc_last_error() on this thread.
 void set_last_error(const std::string& msg);

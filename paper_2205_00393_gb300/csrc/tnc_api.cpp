@@ -132,6 +132,9 @@ tnc_status tnc_set_leaf_variants(tnc_net_t net, int n, const int* leaf_ids, int6
     return TNC_OK;
 }
 
+static tnc_status contract_range(tnc_net* net, int64_t lo, int64_t hi, int mode, double* out_c128, void* stream,
+                                 int64_t groups, bool* done);
+
 tnc_status tnc_contract_variants(tnc_net_t net, int64_t v_lo, int64_t v_hi, int64_t lo, int64_t hi, int mode,
                                  double* out_c128, void* stream) {
     if (!net) return fail(TNC_E_INVALID, "NULL network");
@@ -144,6 +147,12 @@ tnc_status tnc_contract_variants(tnc_net_t net, int64_t v_lo, int64_t v_hi, int6
     const int64_t ns = 1ll << sbits;
     if (lo < 0 || hi < lo || hi > ns) return fail(TNC_E_INVALID, "slice range outside [0, 2^|S|]");
     const int64_t n_out = 1ll << net->plan.obits;
+    // a tiny network: every variant in one launch
+    if (v_hi - v_lo > 1) {
+        bool done = false;
+        st = contract_range(net, (v_lo << sbits) + lo, (v_lo << sbits) + hi, mode, out_c128, stream, v_hi - v_lo, &done);
+        if (st != TNC_OK || done) return st;
+    }
     // the slice-invariant tensors are computed by the first variant and kept
     // in the workspace for the others
     const int keep = net->cache_invariants;
@@ -275,6 +284,15 @@ tnc_status tnc_set_workspace(tnc_net_t net, void* dev_ptr, size_t bytes) {
 }
 
 tnc_status tnc_contract(tnc_net_t net, int64_t lo, int64_t hi, int mode, double* out_c128, void* stream) {
+    bool done = false;
+    return contract_range(net, lo, hi, mode, out_c128, stream, 1, &done);
+}
+
+// tnc_contract for the slices [lo, hi) of `groups` consecutive variants, one result
+// each. More than one variant only where one launch serves them all (a tiny
+// network); else *done stays false.
+static tnc_status contract_range(tnc_net* net, int64_t lo, int64_t hi, int mode, double* out_c128, void* stream,
+                                 int64_t groups, bool* done) {
     if (!net) return fail(TNC_E_INVALID, "NULL network");
     if (!out_c128) return fail(TNC_E_INVALID, "NULL output");
     if (mode < TNC_FP32 || mode > TNC_SPLIT_FP16X2) return fail(TNC_E_INVALID, "unknown mode");
@@ -286,22 +304,29 @@ tnc_status tnc_contract(tnc_net_t net, int64_t lo, int64_t hi, int mode, double*
     cudaStream_t s = (cudaStream_t)stream;
     const Plan& P = net->plan;
     const int64_t R = 1ll << P.obits;
-    CUDA_TRY(cudaMemsetAsync(out_c128, 0, R * 16, s));
-    if (hi == lo) return TNC_OK;
-    if ((st = ensure_leaves(net, s)) != TNC_OK) return st;
+    if (hi > lo) {
+        if ((st = ensure_leaves(net, s)) != TNC_OK) return st;
+        if (persist_eligible(net) && net->persistent == 2) {  // a network that fits one CTA: a CTA per slice
+            const int64_t stride = 1ll << std::min<size_t>(net->S_sorted.size(), 62);
+            st = tiny_contract(net, mode, lo, stride, hi - lo, groups, reinterpret_cast<double2*>(out_c128), s, done);
+            if (st != TNC_OK || *done) return st;
+        }
+        if (groups > 1) return TNC_OK;
+    }
+    CUDA_TRY(cudaMemsetAsync(out_c128, 0, groups * R * 16, s));
+    if (hi == lo) {
+        *done = true;
+        return TNC_OK;
+    }
 
     // workspace and batch
     char* ws = nullptr;
     int64_t nb = 0;
-    const int64_t want = hi - lo;
+    nb = call_batch(net, hi - lo, mode);
     if (net->ws_user) {
-        nb = pick_batch(net, want, net->ws_user_bytes, mode);
         if (nb < 1) return fail(TNC_E_OOM, "workspace too small for one slice");
         ws = (char*)net->ws_user;
     } else {
-        size_t one = (size_t)plan_arena(net, 1, mode).peak;
-        size_t budget = std::max<size_t>(one, (size_t)1 << 30);
-        nb = pick_batch(net, std::min<int64_t>(want, 1024), budget, mode);
         size_t need = (size_t)plan_arena(net, nb, mode).peak;
         if (net->ws_own_bytes < need) {
             if (net->ws_own) CUDA_TRY(cudaFree(net->ws_own));
