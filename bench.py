@@ -42,7 +42,7 @@ TENSOR_FLOPS_PER_CMAC = {"bf16": 4 * 6 * 2, "tf32": 4 * 3 * 2, "bf16x2": 4 * 3 *
 # dense TF32 / BF16 nominal rate ratio (1.1 vs 2.25 PFLOP/s per GPU)
 TF32_OVER_BF16 = 1.1 / 2.25
 KIND_NAMES = {0: "k_gemm_f32", 1: "k_root_partials", 2: "k_gemm_f32+slice_sum", 3: "k_cgemm_tc",
-              4: "k_split_operand", 7: "k_ksplit_reduce", 8: "k_stem_fused", 9: "k_persist", -1: "k_slice_sum_f32", -2: "k_leaf_env_accum"}
+              4: "k_split_operand", 7: "k_ksplit_reduce", 8: "k_stem_fused", 9: "k_tiny or k_persist", -1: "k_slice_sum_f32", -2: "k_leaf_env_accum"}
 
 
 def workload_name():
@@ -355,7 +355,7 @@ def persist_profile_of(prof):
 
 
 def executor_of(by_kind):
-    return "persistent (k_persist, one launch per slice batch)" if 9 in by_kind else "one launch per tree level"
+    return "one launch per call or slice batch (k_tiny, k_persist)" if 9 in by_kind else "one launch per tree level"
 
 
 def single_node(args):
@@ -738,7 +738,7 @@ def executor_sweep(args):
                 if B > net.n_slices or (t >= 24 and B > 1) or (t >= 27 and mode == 0):
                     continue
                 ms, deps = {}, None
-                for name, p in (("persistent", 1), ("per_level", 0)):
+                for name, p in (("persistent", 1), ("per_level", 0), ("automatic", 2)):
                     net.set_option("persistent", p)
                     calls = 12 if t < 24 else 4
                     for _ in range(3):
@@ -760,7 +760,7 @@ def executor_sweep(args):
                 net.set_timing(True)
                 net.contract(0, B, mode, out=out)
                 torch.cuda.synchronize()
-                auto = "persistent" if 9 in {r["kind"] for r in net.last_timings()[0]} else "per_level"
+                auto = "cta_per_slice" if 9 in {r["kind"] for r in net.last_timings()[0]} else "per_level"
                 net.set_timing(False)
                 launches, est_s = net.stats()["level_cost"][str(mode)]
                 print(json.dumps({"metric": "executor sweep: ms per call", "workload":
@@ -769,8 +769,10 @@ def executor_sweep(args):
                                   "per_level_launches": launches, "estimated_us_per_launch": 1e6 * est_s / max(launches, 1),
                                   "ms_persistent": ms["persistent"], "ms_per_level": ms["per_level"],
                                   "per_level_over_persistent": ms["per_level"] / ms["persistent"],
-                                  "automatic_choice": auto, "automatic_choice_is_faster":
-                                  ms[auto] <= min(ms.values()), "persist_deps": deps}), flush=True)
+                                  "ms_automatic": ms["automatic"], "automatic_choice": auto,
+                                  "automatic_choice_is_faster": auto == "cta_per_slice" and
+                                  ms["automatic"] <= min(ms.values()) or auto == "per_level" and
+                                  ms["per_level"] <= ms["persistent"], "persist_deps": deps}), flush=True)
         del net
     return 0
 

@@ -294,7 +294,7 @@ struct tnc_net {
     std::vector<TimedLaunch> timed;
     int64_t launches = 0;
     // persistent executor (one launch per slice batch); its device work lists by key
-    int persistent = 2;  // 0 per-level launches, 1 persistent kernel, 2 automatic choice
+    int persistent = 2;  // 0 per-level launches, 1 persistent kernel, 2 a CTA per slice or per-level launches
     uint64_t persist_wait_ns = 0;    // bound of one dependency wait (0: 10 s)
     int persist_test_stall = 0;      // tests only: one task waits on a counter nothing signals
     int persist_deps = 1;            // per-slice node dependencies (no level chain) when their arena fits
@@ -406,16 +406,14 @@ struct WorkList {
     }
 };
 
-// The automatic executor choice: the persistent kernel when the per-level
-// launches would carry less than 0.1 us of estimated work each on average.
-// The estimate is nominal (peak rates); measured on GB300, the persistent
-// kernel is ahead on calls whose every contraction is tiny (1.3-1.8x at
-// 12-16 qubits, estimates of at most 0.03 us per launch), within about 10% of
-// the per-level launches near 0.1 us, and 6-35% behind from 0.4 us up:
-// there, each launch already runs for tens of microseconds and the
-// one-CTA-per-SM tasks do the same work less efficiently than the separate
-// kernels.
-constexpr double kPersistAutoSecondsPerLaunch = 0.1e-6;
+// The automatic executor choice ("persistent" = 2): a CTA per slice where the network
+// fits (host_tiny.cpp), else one launch per tree level. The persistent executor runs
+// only where it is asked for: it was ahead (1.3-1.8x at 12-16 qubits) when a launch
+// waited for its predecessor's end and its own decoding; with dependent launches,
+// staged parameters and CTA maps a level of tiny contractions costs 2.5 us against
+// its 4, and it is behind on every call measured, from 12 qubits (64 us against 76)
+// over 20 to 25 (71 against 119, 108 against 234, 178 against 355, 236 against 918)
+// to many circuits in one call (223 against 283, 453 against 587).
 
 // planning, arena, level groups and launches (host_plan.cpp)
 int net_plane_cap_log2(const tnc_net* net);

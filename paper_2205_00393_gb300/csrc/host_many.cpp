@@ -172,18 +172,9 @@ tnc_status many_build(ManyCall& mc, cudaStream_t s) {
         mc.nb[i] = nb;
         mc.wss[i] = ws;
     }
-    // persistent executor when every network has it on: forced, or the
-    // automatic choice over the whole call
-    bool pers = true, forced = true;
-    for (tnc_net* net : mc.nets) {
-        pers &= net->persistent != 0;
-        forced &= net->persistent == 1;
-    }
-    if (pers && !forced) {
-        double launches = 0, seconds = 0;
-        for (int i = 0; i < n; ++i) level_cost(mc.nets[i], mc.mode, mc.nb[i], true, &launches, &seconds);
-        pers = seconds < kPersistAutoSecondsPerLaunch * std::max(launches, 1.0);
-    }
+    // persistent executor when every network asks for it
+    bool pers = true;
+    for (tnc_net* net : mc.nets) pers &= net->persistent == 1;
     for (int i = 0; i < n; ++i) {
         tnc_net* net = mc.nets[i];
         const int64_t nb = mc.nb[i];

@@ -357,16 +357,10 @@ static tnc_status contract_range(tnc_net* net, int64_t lo, int64_t hi, int mode,
         const size_t cap = net->ws_user ? net->ws_user_bytes : std::max<size_t>(net->last_arena_bytes[0], (size_t)1 << 30);
         deps = (size_t)ar_flat.peak <= cap;
     }
-    const bool grow = deps && !net->ws_user && net->ws_own_bytes < (size_t)ar_flat.peak;
-    if (use_persist && net->persistent == 2) {
-        const std::string k = group_key_of(net, mode, nb, ws, !deps) + "|" + std::to_string(net->leaf_version);
-        const bool inv_cached = !grow && net->cache_invariants && net->inv_key == k;
-        double launches = 0, seconds = 0;
-        level_cost(net, mode, nb, !inv_cached, &launches, &seconds);
-        use_persist = seconds < kPersistAutoSecondsPerLaunch * std::max(launches, 1.0);
-    }
+    // (a stalled test task needs it)
+    use_persist = use_persist && (net->persistent == 1 || net->persist_test_stall);
     deps = deps && use_persist;
-    if (deps && grow) {  // a failed allocation keeps the reusing arena
+    if (deps && !net->ws_user && net->ws_own_bytes < (size_t)ar_flat.peak) {  // a failed allocation keeps the reusing arena
         void* p = nullptr;
         if (cudaMalloc(&p, (size_t)ar_flat.peak) == cudaSuccess) {
             if (net->ws_own) CUDA_TRY(cudaFree(net->ws_own));
@@ -715,7 +709,7 @@ tnc_status tnc_stats(tnc_net_t net, char* json, size_t cap) {
         // how each tensor-core-eligible contraction is cut up in the split
         // modes, for the last batch size (1 before any call)
         const int64_t cb = net->last_batch > 0 ? net->last_batch : 1;
-        // the automatic executor choice's estimate for that batch, invariants
+        // the per-level launches' estimate for that batch, invariants
         // included: [per-level launches, estimated seconds] per mode
         o << ",\"level_cost\":{";
         for (int mode = TNC_FP32; mode <= TNC_SPLIT_FP16X2; ++mode) {
