@@ -107,10 +107,11 @@ tnc_status tnc_set_leaf_variants(tnc_net_t net, int n, const int* leaf_ids, int6
 /* Contract variants [v_lo, v_hi) (of tnc_set_leaf_variants), each over its
  * slices [lo, hi) of [0, 2^|S|), into out_c128 (device): (v_hi - v_lo) blocks
  * of 2^(open qubits) complex128 values, variant v_lo first, each overwritten.
- * The slice-invariant tensors are computed by the first variant and reused
- * by the others (unless "cache_invariants" is on and they are still valid
- * from an earlier call, every call computes them once; the option itself is
- * left as it was). Errors: TNC_E_STATE without variants; TNC_E_INVALID for a range out
+ * The slice-invariant tensors are computed once per call (unless
+ * "cache_invariants" is on and they are still valid from an earlier call; the
+ * option itself is left as it was). Over every slice ([0, 2^|S|)) a batch holds
+ * several variants when the workspace (1 GiB without one of the caller's) has
+ * room for them, else variants run one after another, with the same bits. Errors: TNC_E_STATE without variants; TNC_E_INVALID for a range out
  * of bounds; the errors of tnc_contract. */
 tnc_status tnc_contract_variants(tnc_net_t net, int64_t v_lo, int64_t v_hi, int64_t lo, int64_t hi, int mode,
                                  double* out_c128, void* stream);

@@ -425,8 +425,9 @@ cudaError_t launch_gemm_f32_group_multi(const GemmParams* d_params, const int2* 
 cudaError_t launch_root_multi(const RootParams* d_roots, double2* const* d_partials, const int64_t* d_blk_off,
                               int n, int64_t total_blocks, const PermParams* d_perms, double2* const* d_outs,
                               const int64_t* d_rs0, const int* d_rb, int max_batch, cudaStream_t s);
+// (groups > 1: consecutive sums of count partials, batch slices each, into consecutive results)
 cudaError_t launch_accumulate_partials(const double2* partials, int count, const PermParams& pp,
-                                       double2* out, cudaStream_t s);
-cudaError_t launch_slice_sum_f32(const SumParams& p, int batch, double2* out, cudaStream_t s);
+                                       double2* out, cudaStream_t s, int groups = 1);
+cudaError_t launch_slice_sum_f32(const SumParams& p, int batch, double2* out, cudaStream_t s, int groups = 1);
 
 }  // namespace tnc

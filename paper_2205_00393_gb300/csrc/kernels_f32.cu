@@ -83,17 +83,18 @@ __global__ void __launch_bounds__(256) k_root_partials(const __grid_constant__ R
                   root_tb);
 }
 
-// out[r] += sum_i partials[i][perm(r)] (a fixed order: accumulate_items)
+// out[y][r] += sum_i partials[y][i][perm(r)], y = blockIdx.y (a fixed order: accumulate_items)
 __global__ void __launch_bounds__(256) k_accumulate_partials(const double2* partials, int count,
                                                              const __grid_constant__ PermParams pp,
                                                              double2* __restrict__ out) {
     dep_trigger();
     dep_wait();
     __shared__ double2 red[256];
-    accumulate_items<0>(partials, count, pp, (int64_t)blockIdx.x * 256, out, red);
+    const int64_t R = 1ll << pp.obits;
+    accumulate_items<0>(partials + blockIdx.y * (count * R), count, pp, (int64_t)blockIdx.x * 256, out + blockIdx.y * R, red);
 }
 
-// out[r] += sum_z src_z[perm(r)] in FP64, z ascending
+// out[y][r] += sum_z src_(y batch + z)[perm(r)] in FP64, z ascending, y = blockIdx.y
 __global__ void k_slice_sum_f32(const __grid_constant__ SumParams p, int batch, double2* __restrict__ out) {
     dep_trigger();
     dep_wait();
@@ -102,14 +103,16 @@ __global__ void k_slice_sum_f32(const __grid_constant__ SumParams p, int batch, 
     if (r >= R) return;
     const int64_t off = bits_offset(r, p.ostride, p.obits, 0);
     double2 acc = make_double2(0.0, 0.0);
-    for (int z = 0; z < batch; ++z) {
+    const int64_t z0 = (int64_t)blockIdx.y * batch;
+    for (int64_t z = z0; z < z0 + batch; ++z) {
         const float2* src = p.src.ptr + z * p.src.batch_stride + slice_offset(p.src, p.slice0 + z);
         float2 v = src[off];
         acc.x += v.x;
         acc.y += v.y;
     }
-    out[r].x += acc.x;
-    out[r].y += acc.y;
+    double2* const o = out + blockIdx.y * R + r;
+    o->x += acc.x;
+    o->y += acc.y;
 }
 
 }  // namespace
@@ -308,15 +311,15 @@ cudaError_t launch_root_partials(const RootParams& p, int batch, double2* partia
 }
 
 cudaError_t launch_accumulate_partials(const double2* partials, int count, const PermParams& pp,
-                                       double2* out, cudaStream_t s) {
+                                       double2* out, cudaStream_t s, int groups) {
     const int64_t items = (int64_t)acc_lanes(count) << pp.obits;
-    return launch_dependent(k_accumulate_partials, dim3((unsigned)((items + 255) / 256)), dim3(256), 0, s, 1, partials, count, pp,
-                            out);
+    return launch_dependent(k_accumulate_partials, dim3((unsigned)((items + 255) / 256), groups), dim3(256), 0, s, 1, partials,
+                            count, pp, out);
 }
 
-cudaError_t launch_slice_sum_f32(const SumParams& p, int batch, double2* out, cudaStream_t s) {
+cudaError_t launch_slice_sum_f32(const SumParams& p, int batch, double2* out, cudaStream_t s, int groups) {
     int64_t R = 1ll << p.obits;
-    return launch_dependent(k_slice_sum_f32, dim3((unsigned)((R + 255) / 256)), dim3(256), 0, s, 1, p, batch, out);
+    return launch_dependent(k_slice_sum_f32, dim3((unsigned)((R + 255) / 256), groups), dim3(256), 0, s, 1, p, batch, out);
 }
 
 }  // namespace tnc
