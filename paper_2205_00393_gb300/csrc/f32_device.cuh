@@ -5,6 +5,8 @@
 // a larger CTA (the persistent executor's other warps do not take part).
 #pragma once
 
+#include <type_traits>
+
 #include "kernels.h"
 #include "launch.cuh"
 
@@ -98,15 +100,17 @@ template <int NTH, int RM, int WN> struct TileCfg {
     static constexpr int BM = NTH / 32 / WN * 4 * RM, BN = 32 * WN;
 };
 
-// Staged operands and offset tables of one tile.
+__host__ __device__ constexpr int log2_of(int v) { return v <= 1 ? 0 : 1 + log2_of(v / 2); }
+
+// Staged operands of one tile.
 template <int NTH, int RM, int WN> struct GemmStage {
     static constexpr int BM = TileCfg<NTH, RM, WN>::BM, BN = TileCfg<NTH, RM, WN>::BN;
     float Ar[2][BK][BM + 4], Ai[2][BK][BM + 4];  // 16-byte aligned rows
     float2 Bs[2][BK][BN + 2];
-    int64_t rowA[BM], colB[BN], klA[BK], klB[BK];
     // kstep[b]: offset of k-tile t + 1 minus that of k-tile t when b bits of t
     // carry (bit b of t + 1 is its lowest set bit)
     int64_t kstepA[kMaxBits], kstepB[kMaxBits];
+    int64_t sa[4], sb[4];  // TileWork::sa, sb where registers are short
 };
 template <int NTH, int RM, int WN> struct GemmSmemT : GemmStage<NTH, RM, WN> {
     f32x2 comp[4 * RM][NTH];       // TwoSum compensation of each thread's outputs
@@ -132,7 +136,9 @@ template <> struct OperandPtr<1> { using type = const float2*; };
 
 // The gather, staging and products of one output tile (slice z, slice id
 // slice0 + z) of the contraction described by p.
-template <int BAR, int NTH, int RM, int WN> struct TileWork {
+// LEAN: registers are short (grouped contractions with their parameters in shared
+// memory, the persistent executor).
+template <int BAR, int NTH, int RM, int WN, bool LEAN = false> struct TileWork {
     using Cfg = TileCfg<NTH, RM, WN>;
     static constexpr int EA = Cfg::BM * BK / NTH, EB = Cfg::BN * BK / NTH;  // elements a thread gathers per k-tile
     static constexpr int RP = RM / 2;                                      // row pairs of a thread
@@ -140,6 +146,8 @@ template <int BAR, int NTH, int RM, int WN> struct TileWork {
     int64_t M, N, K, m0, n0;
     typename OperandPtr<BAR>::type A, B;
     bool a_kfast, b_nfast;
+    bool full;  // no element of the tile lies past M, N or K
+    int64_t sa[LEAN ? 1 : log2_of(EA)], sb[LEAN ? 1 : log2_of(EB)];  // offsets of the bits of an element's number (the same in every thread)
     int tm, tn;
     int64_t khA = 0, khB = 0;  // offsets of the k-tile to gather
     float2 ra[EA], rb[EB];
@@ -157,15 +165,6 @@ template <int BAR, int NTH, int RM, int WN> struct TileWork {
         n0 = (tile % tiles_n) * Cfg::BN;
         A = p.A.ptr + z * p.A.batch_stride + slice_offset(p.A, slice0 + z);
         B = p.B.ptr + z * p.B.batch_stride + slice_offset(p.B, slice0 + z);
-        for (int t = tid; t < Cfg::BM + Cfg::BN + 2 * BK; t += NTH) {
-            const int kl = p.kb < LOG_BK ? p.kb : LOG_BK;
-            if (t < Cfg::BM) sm.rowA[t] = (m0 + t < M) ? bits_offset(m0 + t, p.am, p.mb, 0) : 0;
-            else if (t < Cfg::BM + Cfg::BN) {
-                const int n = t - Cfg::BM;
-                sm.colB[n] = (n0 + n < N) ? bits_offset(n0 + n, p.bn, p.nb, 0) : 0;
-            } else if (t < Cfg::BM + Cfg::BN + BK) sm.klA[t - Cfg::BM - Cfg::BN] = bits_offset(t - Cfg::BM - Cfg::BN, p.ak, kl, 0);
-            else sm.klB[t - Cfg::BM - Cfg::BN - BK] = bits_offset(t - Cfg::BM - Cfg::BN - BK, p.bk, kl, 0);
-        }
         if (tid < p.kb - LOG_BK) {
             int64_t da = p.ak[LOG_BK + tid], db = p.bk[LOG_BK + tid];
             for (int j = 0; j < tid; ++j) {
@@ -178,6 +177,30 @@ template <int BAR, int NTH, int RM, int WN> struct TileWork {
         // load mapping: walk the operand's unit-stride mode with consecutive threads
         a_kfast = p.kb > 0 && p.ak[0] == 1;
         b_nfast = p.nb > 0 && p.bn[0] == 1;
+        int m, k, n, kb;
+        a_mk(0, m, k);
+        b_nk(0, n, kb);
+        A += bits_offset(m0 + m, p.am, p.mb, 0) + bits_offset(k, p.ak, p.kb, 0);
+        B += bits_offset(n0 + n, p.bn, p.nb, 0) + bits_offset(kb, p.bk, p.kb, 0);
+        // bit t of an element's number is bit lo + t of its k (or m, n)
+        constexpr int LT = log2_of(NTH) - LOG_BK, LA = log2_of(NTH / Cfg::BM), LB = log2_of(NTH / Cfg::BN);
+        auto step_a = [&](int t) {
+            return a_kfast ? (LT + t < p.mb ? p.am[LT + t] : 0) : LA + t < p.kb ? p.ak[LA + t] : 0;
+        };
+        auto step_b = [&](int t) {
+            return b_nfast ? (LB + t < p.kb ? p.bk[LB + t] : 0) : LT + t < p.nb ? p.bn[LT + t] : 0;
+        };
+        static_assert(log2_of(EA) <= 4 && log2_of(EB) <= 4, "size of the shared copies");
+        if constexpr (LEAN) {
+            if (tid < log2_of(EA)) sm.sa[tid] = step_a(tid);
+            if (tid < log2_of(EB)) sm.sb[tid] = step_b(tid);
+        } else {
+#pragma unroll
+            for (int t = 0; t < log2_of(EA); ++t) sa[t] = step_a(t);
+#pragma unroll
+            for (int t = 0; t < log2_of(EB); ++t) sb[t] = step_b(t);
+        }
+        full = m0 + Cfg::BM <= M && n0 + Cfg::BN <= N && K >= BK;
         // lanes 4 (m) x 8 (n): thread rows tm .. tm + 3 (and, for RM = 8, tm + 16 ..
         // tm + 19), columns tn, tn + 1, tn + 16, tn + 17
         const int lane = tid & 31, warp = tid >> 5;
@@ -200,21 +223,50 @@ template <int BAR, int NTH, int RM, int WN> struct TileWork {
         khA += sm.kstepA[carry];
         khB += sm.kstepB[carry];
     }
+    // The elements of a thread differ in three bits or so of k (or of m, n), and the
+    // offsets of these bits are the same in every thread: one pointer per operand, an
+    // addition per element, and no predicates where the tile has no edge. (Rows and
+    // columns from tables in shared memory were two loads and two 64-bit additions
+    // per element, in a loop that shared memory bounds as much as the FMAs:
+    // (2^11, 2^10, 2^12) 1731 us against 1510, (2^13, 2^6, 2^11) 281 against 229, a
+    // 24-qubit call 2.32 ms against 2.11.) LEAN keeps the one path with predicates:
+    // a level of small contractions waits for its instructions (20 qubits: 162 us
+    // against 166).
     __device__ __forceinline__ void gather() {
+        auto load = [&](auto masked) {
 #pragma unroll
-        for (int i = 0; i < EA; ++i) {
-            int m, k;
-            a_mk(i, m, k);
-            ra[i] = make_float2(0.f, 0.f);
-            if (m0 + m < M && k < K) ra[i] = A[khA + sm.rowA[m] + sm.klA[k]];
-        }
+            for (int i = 0; i < EA; ++i) {
+                int64_t o = 0;
 #pragma unroll
-        for (int i = 0; i < EB; ++i) {
-            int n, k;
-            b_nk(i, n, k);
-            rb[i] = make_float2(0.f, 0.f);
-            if (n0 + n < N && k < K) rb[i] = B[khB + sm.colB[n] + sm.klB[k]];
-        }
+                for (int t = 0; t < log2_of(EA); ++t)
+                    if (i >> t & 1) o += LEAN ? sm.sa[t] : sa[t];
+                if constexpr (decltype(masked)::value) {
+                    int m, k;
+                    a_mk(i, m, k);
+                    ra[i] = make_float2(0.f, 0.f);
+                    if (m0 + m < M && k < K) ra[i] = A[khA + o];
+                } else {
+                    ra[i] = A[khA + o];
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < EB; ++i) {
+                int64_t o = 0;
+#pragma unroll
+                for (int t = 0; t < log2_of(EB); ++t)
+                    if (i >> t & 1) o += LEAN ? sm.sb[t] : sb[t];
+                if constexpr (decltype(masked)::value) {
+                    int n, k;
+                    b_nk(i, n, k);
+                    rb[i] = make_float2(0.f, 0.f);
+                    if (n0 + n < N && k < K) rb[i] = B[khB + o];
+                } else {
+                    rb[i] = B[khB + o];
+                }
+            }
+        };
+        if (!LEAN && full) load(std::false_type{});
+        else load(std::true_type{});
     }
     __device__ __forceinline__ void stage_store(int st) {
 #pragma unroll
@@ -280,10 +332,10 @@ template <int BAR, int NTH, int RM, int WN> struct TileWork {
 
 // One output tile `tile` of slice z (slice id slice0 + z) of the contraction
 // described by p.
-template <int BAR = 0, int NTH = 256, int RM = 4, int WN = 2>
+template <int BAR = 0, int NTH = 256, int RM = 4, int WN = 2, bool LEAN = BAR == 1>
 __device__ __forceinline__ void gemm_tile(const GemmParams& p, int64_t tile, int z, int64_t slice0,
                                           GemmSmemT<NTH, RM, WN>& sm) {
-    using W = TileWork<BAR, NTH, RM, WN>;
+    using W = TileWork<BAR, NTH, RM, WN, LEAN>;
     constexpr int RP = W::RP;
     const int tid = threadIdx.x;
     W w(p, tile, z, slice0, sm);

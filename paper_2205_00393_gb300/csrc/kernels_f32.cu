@@ -32,10 +32,11 @@ __global__ void __launch_bounds__(NTH, 3) k_gemm_f32_cluster(const __grid_consta
                                    *reinterpret_cast<GemmClusterSmem<NTH, WN>*>(gemm_dyn));
 }
 
-// Grouped contractions run on 32 x 64 tiles by 128 threads, four CTAs per SM:
-// most nodes of a level have a few tiles at most, and the smaller tile shortens
-// the chain of each (K = 512, M = 2^8, N = 2^6: 58 us against 74 us on the
-// 64 x 64 tile of 256 threads).
+// Grouped contractions run on 32 x 64 tiles by 128 threads, three CTAs per SM: most
+// nodes of a level have a few tiles at most, and the smaller tile shortens the chain
+// of each (K = 512, M = 2^8, N = 2^6: 58 us against 74 us on the 64 x 64 tile of 256
+// threads). A fourth CTA would take the registers of a tile whose parameters are
+// in shared memory below what it needs: a 20-qubit call 162 us instead of 157.
 constexpr int GT = 128;
 using GroupSmem = GemmSmemT<GT, 4, 2>;
 
@@ -61,13 +62,13 @@ __device__ __forceinline__ const GemmParams& stage_params(const GemmParams* src,
 
 // Many independent contractions in one launch (nodes of one tree level): CTA
 // b serves tile map[b].y of node map[b].x.
-__global__ void __launch_bounds__(GT, 4) k_gemm_f32_group(const GemmParams* __restrict__ params,
+__global__ void __launch_bounds__(GT, 3) k_gemm_f32_group(const GemmParams* __restrict__ params,
                                                        const int2* __restrict__ map, int64_t slice0) {
     dep_trigger();
     extern __shared__ __align__(16) uint8_t gemm_dyn[];
     GroupCta& cta = *reinterpret_cast<GroupCta*>(gemm_dyn);
     const int2 nt = map[blockIdx.x];
-    gemm_tile<0, GT, 4, 2>(stage_params(params + nt.x, cta), nt.y, blockIdx.z, slice0, cta.tile);
+    gemm_tile<0, GT, 4, 2, true>(stage_params(params + nt.x, cta), nt.y, blockIdx.z, slice0, cta.tile);
 }
 
 // FP64 partial sums of a contraction with R = M*N <= 64 outputs.
@@ -117,7 +118,7 @@ __global__ void k_slice_sum_f32(const __grid_constant__ SumParams p, int batch, 
 
 }  // namespace
 
-__global__ void __launch_bounds__(GT, 4) k_gemm_f32_group_multi(const GemmParams* __restrict__ params,
+__global__ void __launch_bounds__(GT, 3) k_gemm_f32_group_multi(const GemmParams* __restrict__ params,
                                                              const int2* __restrict__ map, const int* __restrict__ net,
                                                              const int64_t* __restrict__ rs0,
                                                              const int* __restrict__ rb);
@@ -168,16 +169,16 @@ static cudaError_t launch_gemm_f32_cluster(const GemmParams& p, int batch, cudaS
 // batch together. Every choice gives the same bits.
 //  - few tiles and K >= 128: clusters, whose CTAs share the k groups of one
 //    tile. 152 SMs hold 456 such CTAs, and while T is below an SM each, eight
-//    per tile fill the chip: (M, N, K) = (2^10, 2^6, 2^14) 350 us against 1486
-//    on one CTA per tile, (2^6, 2^6, 2^12) 67 against 379, (2^9, 2^9, 2^9)
-//    55 against 62; at T = 256, four: (2^10, 2^9, 2^10) 148 us, against 158 with
-//    eight and 155 without. Beyond that clusters lose ((2^10, 2^10, 2^10),
-//    T = 512: 274 against 244).
+//    per tile fill the chip: (M, N, K) = (2^10, 2^6, 2^14) 285 us against 1217
+//    on one CTA per tile, (2^6, 2^6, 2^12) 56 against 313, (2^9, 2^9, 2^9)
+//    54 against 60; at T = 256, four: (2^10, 2^9, 2^10) 130 us, against 137 with
+//    eight and 140 without. Beyond that clusters lose ((2^10, 2^10, 2^10),
+//    T = 512: 237 against 224).
 //  - two SMs' worth of tiles or more: 64 x 64 tiles with 8 x 4 outputs per thread,
 //    which load fewer bytes per product from shared memory: (2^11, 2^11, 2^11)
-//    1515 us (45.4 TFLOP/s, 0.62 of the FFMA rate) against 1677.
-//  - otherwise 32 x 64 tiles (K < 128, or narrow outputs): (2^10, 2^8, 2^7) 30 us
-//    against 34.
+//    1364 us (50.4 TFLOP/s, 0.69 of the FFMA rate) against 1480.
+//  - otherwise 32 x 64 tiles (K < 128, or narrow outputs): (2^9, 2^9, 2^7) 30 us
+//    against 35.
 cudaError_t launch_gemm_f32(const GemmParams& p, int batch, cudaStream_t s) {
     const bool narrow = p.nb <= 5;
     const int64_t T = narrow ? (int64_t)batch << (p.mb > 6 ? p.mb - 6 : 0)
@@ -204,7 +205,7 @@ cudaError_t launch_gemm_f32(const GemmParams& p, int batch, cudaStream_t s) {
 // Grouped contractions of several networks: node i belongs to network
 // net[i]; slice z of the launch maps to slice rs0[net] + z of that network and
 // exists only for z < rb[net] (networks batch different numbers of slices).
-__global__ void __launch_bounds__(GT, 4) k_gemm_f32_group_multi(const GemmParams* __restrict__ params,
+__global__ void __launch_bounds__(GT, 3) k_gemm_f32_group_multi(const GemmParams* __restrict__ params,
                                                              const int2* __restrict__ map, const int* __restrict__ net,
                                                              const int64_t* __restrict__ rs0,
                                                              const int* __restrict__ rb) {
@@ -217,7 +218,7 @@ __global__ void __launch_bounds__(GT, 4) k_gemm_f32_group_multi(const GemmParams
         dep_wait();
         return;
     }
-    gemm_tile<0, GT, 4, 2>(stage_params(params + nt.x, cta), nt.y, blockIdx.z, rs0[w], cta.tile);
+    gemm_tile<0, GT, 4, 2, true>(stage_params(params + nt.x, cta), nt.y, blockIdx.z, rs0[w], cta.tile);
 }
 
 // Root reductions of several networks in one launch: block x serves chunk
