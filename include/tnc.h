@@ -228,7 +228,7 @@ tnc_status tnc_check_device(tnc_net_t net, void* stream);
  * != 0 and a non-default stream, the launch sequence is captured once into a
  * CUDA graph and replayed by later calls with identical arguments (networks,
  * ranges, outputs, workspaces, plans and options; leaf data may change between
- * calls). When every network has the "persistent" option at 1 and the
+ * calls). When the "persistent" option says so (see there) and the
  * persistent executor can run each of them, every round of slice batches is
  * instead ONE launch of the work-list kernel holding all networks' tasks,
  * ordered by tree level (level L of every network before level L + 1 of any);
@@ -358,10 +358,15 @@ tnc_status tnc_worklist_many_json(int n, const tnc_net_t* nets, int64_t batch, i
  *                  a CTA per slice, every slice of every variant in one
  *                  launch and a sum (timing record of kind 9), if a slice
  *                  has at most 3 2^16 complex multiply-accumulates (3 2^17
- *                  for calls of 64 slices and more); every other call,
- *                  and tnc_contract_many, runs one launch per level, which
- *                  is ahead of the persistent executor from 12 qubits on
- *                  (tnc_contract_many: 1 on every network takes that one)
+ *                  for calls of 64 slices and more); every other call
+ *                  runs one launch per level, which is ahead of the
+ *                  persistent executor from 12 qubits on. tnc_contract_many
+ *                  takes the persistent executor if every network has 1, or
+ *                  none has 0, the mode is a split one, there are at least
+ *                  16 networks and their per-level launches would carry less
+ *                  than 0.1 us of work each on average (a contraction
+ *                  estimated at the larger of its flops at 300 TFLOP/s and
+ *                  its 8 (MK + KN + MN) bytes per slice at 6 TB/s)
  *  "persist_deps"  0 or 1 (default 1): with 1, a tnc_contract batch run by
  *                  the persistent executor gives every tensor and temporary
  *                  of the batch bytes of their own for the launch when that

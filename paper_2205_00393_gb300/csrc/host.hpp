@@ -407,13 +407,20 @@ struct WorkList {
 };
 
 // The automatic executor choice ("persistent" = 2): a CTA per slice where the network
-// fits (host_tiny.cpp), else one launch per tree level. The persistent executor runs
-// only where it is asked for: it was ahead (1.3-1.8x at 12-16 qubits) when a launch
-// waited for its predecessor's end and its own decoding; with dependent launches,
-// staged parameters and CTA maps a level of tiny contractions costs 2.5 us against
-// its 4, and it is behind on every call measured, from 12 qubits (64 us against 76)
-// over 20 to 25 (71 against 119, 108 against 234, 178 against 355, 236 against 918)
-// to many circuits in one call (223 against 283, 453 against 587).
+// fits (host_tiny.cpp), else one launch per tree level. The persistent executor was
+// ahead (1.3-1.8x at 12-16 qubits) when a launch waited for its predecessor's end and
+// its own decoding; with dependent launches, staged parameters and CTA maps a level of
+// tiny contractions costs 2.5 us against its 4, and it is behind on every call of one
+// network measured, from 12 qubits (64 us against 76) over 20 to 25 (71 against 119,
+// 108 against 234, 178 against 355, 236 against 918). tnc_contract_many in a split mode
+// takes it from kPersistAutoNetworks networks on if its launches would carry less than
+// 0.1 us of estimated work each: there the tensor-core contractions of a level are
+// launches of their own, one network after another, and the work list runs them side
+// by side (split BF16, circuits of at most 2^26 multiply-accumulates: 10 circuits 452
+// us per level against 509, 16: 762 against 753, 24: 1013 against 966, 48: 1958
+// against 1759, 100: 3977 against 3221; FP32, 100: 2443 against 2645).
+constexpr double kPersistAutoSecondsPerLaunch = 0.1e-6;
+constexpr int kPersistAutoNetworks = 16;
 
 // planning, arena, level groups and launches (host_plan.cpp)
 int net_plane_cap_log2(const tnc_net* net);

@@ -172,9 +172,18 @@ tnc_status many_build(ManyCall& mc, cudaStream_t s) {
         mc.nb[i] = nb;
         mc.wss[i] = ws;
     }
-    // persistent executor when every network asks for it
-    bool pers = true;
-    for (tnc_net* net : mc.nets) pers &= net->persistent == 1;
+    // persistent executor when every network asks for it, or leaves the choice and the
+    // call is for it
+    bool pers = true, allowed = true;
+    for (tnc_net* net : mc.nets) {
+        pers &= net->persistent == 1;
+        allowed &= net->persistent != 0;
+    }
+    if (!pers && allowed && n >= kPersistAutoNetworks && mc.mode != TNC_FP32) {
+        double launches = 0, seconds = 0;
+        for (int i = 0; i < n; ++i) level_cost(mc.nets[i], mc.mode, mc.nb[i], true, &launches, &seconds);
+        pers = seconds < kPersistAutoSecondsPerLaunch * std::max(launches, 1.0);
+    }
     for (int i = 0; i < n; ++i) {
         tnc_net* net = mc.nets[i];
         const int64_t nb = mc.nb[i];

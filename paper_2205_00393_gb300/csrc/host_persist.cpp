@@ -230,7 +230,7 @@ static void level_cost_uncached(tnc_net* net, int mode, int64_t b, bool with_inv
 // each larger one, three per tensor-core contraction (two operand splits and the
 // GEMM), two for the final contraction. A contraction's time is estimated as
 // the larger of its flops at 300 TFLOP/s and its operand and result bytes,
-// 8 (MK + KN + MN) per slice, at 6 TB/s. For inspection (tnc_stats). Cached by plan_key.
+// 8 (MK + KN + MN) per slice, at 6 TB/s. Cached by plan_key.
 void level_cost(tnc_net* net, int mode, int64_t b, bool with_inv, double* launches, double* seconds) {
     const std::string key = plan_key(net, mode, b) + (with_inv ? ":i" : ":p");
     auto it = net->cost_cache.find(key);
