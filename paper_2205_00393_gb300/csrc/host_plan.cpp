@@ -795,8 +795,7 @@ tnc_status launch_tc_contraction(tnc_net* net, const tnc::GemmParams& g, int b, 
         sexp_a = reinterpret_cast<int8_t*>(static_cast<char*>(pa) + plane_data_bytes(mode, mbp, kbp, b));
         sexp_b = reinterpret_cast<int8_t*>(static_cast<char*>(pb) + plane_data_bytes(mode, nbp, kbp, b));
     }
-    auto split = [&](const tnc::Operand& src, int rb, const int64_t* rs, const int64_t* ks, void* dst,
-                     int8_t* sexp, int nz) -> tnc_status {
+    auto split_params = [&](const tnc::Operand& src, int rb, const int64_t* rs, const int64_t* ks, void* dst, int8_t* sexp) {
         tnc::SplitParams sp{};
         sp.src = src;
         sp.rb = rb;
@@ -806,12 +805,28 @@ tnc_status launch_tc_contraction(tnc_net* net, const tnc::GemmParams& g, int b, 
         sp.slice0 = g.slice0;
         sp.dst = dst;
         sp.sexp = sexp;
+        return sp;
+    };
+    auto split = [&](const tnc::SplitParams& sp, int nz) -> tnc_status {
         CUDA_TRY(timed_begin(net, node, K_SPLIT, nz, s, 0.0));
         CUDA_TRY(tnc::launch_split(sp, mode, nz, s));
         CUDA_TRY(timed_end(net, s));
         return TNC_OK;
     };
     tnc_status st;
+    bool both = false;  // both operands in one launch (timed as one split)
+    if (!pA && !pB && !pK) {
+        const tnc::SplitParams sa = split_params(g.A, mbp, g.am, g.ak, pa, sexp_a), sb = split_params(g.B, nbp, g.bn, g.bk, pb, sexp_b);
+        const size_t records = net->timed.size();
+        CUDA_TRY(timed_begin(net, node, K_SPLIT, std::max(nza, nzb), s, 0.0));
+        CUDA_TRY(tnc::launch_split_pair(sa, nza, sb, nzb, mode, s, &both));
+        if (both) {
+            CUDA_TRY(timed_end(net, s));
+        } else {
+            net->launches -= 1;
+            net->timed.resize(records);
+        }
+    }
     for (int64_t qk = 0; qk < (1ll << pK); ++qk) {  // K panels: the top pK bits of k fixed
         tnc::Operand Ak = g.A, Bk = g.B;
         for (int j = 0; j < pK; ++j)
@@ -823,13 +838,13 @@ tnc_status launch_tc_contraction(tnc_net* net, const tnc::GemmParams& g, int b, 
             tnc::Operand B = Bk;
             for (int j = 0; j < pB; ++j)
                 if ((qb >> j) & 1) B.ptr += g.bn[nbp + j];
-            if ((st = split(B, nbp, g.bn, g.bk, pb, sexp_b, nzb)) != TNC_OK) return st;
+            if (!both && (st = split(split_params(B, nbp, g.bn, g.bk, pb, sexp_b), nzb)) != TNC_OK) return st;
             for (int64_t qa = 0; qa < (1ll << pA); ++qa) {  // row panels of A: top pA bits of m fixed
                 tnc::Operand A = Ak;
                 for (int j = 0; j < pA; ++j)
                     if ((qa >> j) & 1) A.ptr += g.am[mbp + j];
-                if (pB == 0 || qb == 0 || pA > 0)  // else the A planes of this K panel are still in place
-                    if ((st = split(A, mbp, g.am, g.ak, pa, sexp_a, nza)) != TNC_OK) return st;
+                if (!both && (pB == 0 || qb == 0 || pA > 0))  // else the A planes of this K panel are still in place
+                    if ((st = split(split_params(A, mbp, g.am, g.ak, pa, sexp_a), nza)) != TNC_OK) return st;
                 tnc::TcGemmParams tp{};
                 tp.mb = mbp;
                 tp.nb = nbp;

@@ -109,6 +109,9 @@ int tc_min_kb(int mode);
 // split FP16x2: K chunks of 256 (one if K <= 256) that carry their own scale
 int tc_scale_chunks(int kb);
 cudaError_t launch_split(const SplitParams& p, int mode, int batch, cudaStream_t s);
+// Both operands of a contraction in one launch; *done false: too large to gain by it.
+cudaError_t launch_split_pair(const SplitParams& a, int batch_a, const SplitParams& b, int batch_b, int mode, cudaStream_t s,
+                              bool* done);
 cudaError_t launch_cgemm_tc(const TcGemmParams& p, int mode, const void* planesA, const void* planesB,
                             int batch, cudaStream_t s);
 // C[z][m][n] (+)= sum over s < 2^ksplit_bits, in order, of partial[s][z][m][n] (an FP64 sum
