@@ -116,6 +116,15 @@ tnc_status tnc_set_leaf_variants(tnc_net_t net, int n, const int* leaf_ids, int6
 tnc_status tnc_contract_variants(tnc_net_t net, int64_t v_lo, int64_t v_hi, int64_t lo, int64_t hi, int mode,
                                  double* out_c128, void* stream);
 
+/* Slices per batch (a multiple of 2^|S|, at least two variants) in which
+ * tnc_contract_variants runs n_variants variants over every slice with one launch
+ * per tree level in a workspace of workspace_bytes (0: the budget of an own one, the
+ * larger of 1 GiB and one slice's arena), or 0 if it runs them one after another.
+ * tnc_arena_json gives the bytes of a batch, which fit that workspace. Host logic,
+ * no GPU. Errors: TNC_E_INVALID for a bad argument; TNC_E_STATE before
+ * tnc_set_path. */
+tnc_status tnc_variants_batch(tnc_net_t net, int64_t n_variants, int mode, size_t workspace_bytes, int64_t* slices);
+
 /* Bytes of all leaves packed back to back in leaf order (complex64). */
 tnc_status tnc_leaf_bytes(tnc_net_t net, size_t* bytes);
 

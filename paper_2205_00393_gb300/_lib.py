@@ -51,6 +51,7 @@ def load_library():
                                   P(P(ctypes.c_float))],
         "tnc_contract_variants": [ctypes.c_void_p, ctypes.c_int64, ctypes.c_int64, ctypes.c_int64, ctypes.c_int64,
                                   ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p],
+        "tnc_variants_batch": [ctypes.c_void_p, ctypes.c_int64, ctypes.c_int, ctypes.c_size_t, c_i64p],
         "tnc_leaf_bytes": [ctypes.c_void_p, P(ctypes.c_size_t)],
         "tnc_upload_leaves": [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p],
         "tnc_greedy_path": [ctypes.c_void_p, P(ctypes.c_int)],
@@ -299,6 +300,14 @@ class Network:
                                              ctypes.c_void_p(out.data_ptr()), _stream_ptr(stream))
         _check(self._lib, st)
         return out
+
+    def variants_batch(self, count, mode=FP32, workspace_bytes=0):
+        """Slices per batch of contract_variants over every slice, 0 if the
+        variants run one after another (tnc_variants_batch)."""
+        n = ctypes.c_int64()
+        _check(self._lib, self._lib.tnc_variants_batch(self._h, int(count), int(mode), int(workspace_bytes),
+                                                       ctypes.byref(n)))
+        return n.value
 
     def set_option(self, key, value):
         """Tensor-core tuning option (see tnc_set_option in include/tnc.h)."""

@@ -475,8 +475,17 @@ cudaError_t wl_launch(const DeviceWorkList& D, int mode, int64_t slice0, const i
 bool wl_validate(const tnc_net* net, const WorkList& W, const char* ws, size_t ws_bytes, const double* out, int mode, std::string* why);
 DeviceWorkList* contract_worklist(tnc_net* net, const Arena& ar, char* ws, int b, int mode, bool with_inv, double* out, cudaStream_t s, tnc_status* st);
 
-// Slices per batch of a call of `want` slices, 0 if the given workspace does not hold one.
-int64_t call_batch(const tnc_net* net, int64_t want, int mode);
+// What a call's batch may take: the caller's workspace, or an own one of at most the
+// larger of 1 GiB and one slice's arena, and at most so many slices.
+struct Budget {
+    size_t bytes;
+    int64_t slices;
+};
+Budget own_budget(const tnc_net* net, int mode);
+Budget batch_budget(const tnc_net* net, int mode);
+// Slices per batch of a call of `want` slices, 0 if the budget does not hold one. Its
+// arena fits the budget.
+int64_t call_batch(const tnc_net* net, int64_t want, int mode, const Budget& budget);
 
 // tiny networks (host_tiny.cpp): slice ids first + g stride + j (j < per) summed into
 // result g < groups; *done false: the network or the call is not for it

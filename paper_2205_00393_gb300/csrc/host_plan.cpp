@@ -635,10 +635,16 @@ int64_t pick_batch(const tnc_net* net, int64_t want, size_t budget, int mode) {
     return lo;
 }
 
-int64_t call_batch(const tnc_net* net, int64_t want, int mode) {
-    if (net->ws_user) return pick_batch(net, want, net->ws_user_bytes, mode);
-    const size_t one = (size_t)plan_arena(net, 1, mode).peak;
-    return pick_batch(net, std::min<int64_t>(want, 1024), std::max<size_t>(one, (size_t)1 << 30), mode);
+Budget own_budget(const tnc_net* net, int mode) {
+    return {std::max<size_t>((size_t)plan_arena(net, 1, mode).peak, (size_t)1 << 30), 1024};
+}
+
+Budget batch_budget(const tnc_net* net, int mode) {
+    return net->ws_user ? Budget{net->ws_user_bytes, 65535} : own_budget(net, mode);
+}
+
+int64_t call_batch(const tnc_net* net, int64_t want, int mode, const Budget& budget) {
+    return pick_batch(net, std::min(want, budget.slices), budget.bytes, mode);
 }
 
 std::vector<Group> level_groups(const tnc_net* net, int mode, bool per_slice) {

@@ -187,7 +187,7 @@ tnc_status tiny_contract(tnc_net* net, int mode, int64_t first, int64_t stride, 
     if (tp.want != per || tp.given != given) {
         tp.want = per;
         tp.given = given;
-        tp.nb = call_batch(net, per, mode);
+        tp.nb = call_batch(net, per, mode, batch_budget(net, mode));
         for (int flat : {0, 1}) tp.arena[flat] = tp.nb < 1 ? 0 : (size_t)plan_arena(net, tp.nb, mode, flat == 0).peak;
     }
     if (tp.nb < 1) return TNC_OK;

@@ -292,15 +292,22 @@ tnc_status tnc_contract(tnc_net_t net, int64_t lo, int64_t hi, int mode, double*
 // multiple of per, or 0 if the variants run one after another: one launch per
 // level and batch then serves several variants (23 bitstrings of a 24-qubit stem:
 // 6.47 -> 5.44 ms, 284 launches -> 64; 8 of a 20-qubit circuit 469 -> 78 us).
-// Batches are as even as they can be. The batch must not change the arithmetic: the K panels and splits of a
-// tensor-core contraction are those of one variant's batch.
-static int64_t variants_batch(tnc_net* net, int mode, int64_t per, int64_t groups) {
+// Batches are as even as they can be and fit the budget: a smaller batch can need
+// more bytes than a larger one, whose operand planes pass the cap and are cut into
+// panels, so the evened batch is checked by itself and taken down by eighths until
+// it fits. The batch must not change the arithmetic: one variant's own batch holds
+// all its slices, and the K panels and splits of a tensor-core contraction are the
+// same in both.
+static int64_t variants_batch(const tnc_net* net, int mode, int64_t per, int64_t groups, const Budget& budget) {
     const Plan& P = net->plan;
-    if (P.nodes.empty() || per > 65535) return 0;
-    if (persist_eligible(net) && (net->persistent == 1 || net->persist_test_stall)) return 0;
-    const int64_t most = call_batch(net, per * groups, mode) / per;  // variants per batch
-    if (most < 2) return 0;
-    const int64_t rounds = (groups + most - 1) / most, nb = (groups + rounds - 1) / rounds * per;
+    if (P.nodes.empty() || per < 1 || per > 65535) return 0;
+    const int64_t most = call_batch(net, per * groups, mode, budget) / per;  // variants per batch
+    if (most < 2 || call_batch(net, per, mode, budget) != per) return 0;
+    const int64_t rounds = (groups + most - 1) / most;
+    int64_t v = (groups + rounds - 1) / rounds;
+    while (v >= 2 && (size_t)plan_arena(net, v * per, mode).peak > budget.bytes) v -= (v + 7) / 8;
+    if (v < 2) return 0;
+    const int64_t nb = v * per;
     for (const NodePlan& np : P.nodes)
         if (np.per_slice && shape_choice(net, mode, np.mb, np.nb, np.kb, np.is_root)) {
             const TcCut a = tc_cut(net, mode, np.mb, np.nb, np.kb, per), b = tc_cut(net, mode, np.mb, np.nb, np.kb, nb);
@@ -337,7 +344,8 @@ static tnc_status contract_range(tnc_net* net, int64_t lo, int64_t hi, int mode,
     int64_t nb = 0;
     if (groups > 1 && hi > lo) {
         const bool all = net->S_sorted.size() < 62 && per == 1ll << net->S_sorted.size();  // consecutive slice ids
-        nb = all ? variants_batch(net, mode, per, groups) : 0;
+        const bool forced = persist_eligible(net) && (net->persistent == 1 || net->persist_test_stall);
+        nb = all && !forced ? variants_batch(net, mode, per, groups, batch_budget(net, mode)) : 0;
         if (nb == 0) return TNC_OK;
         hi = lo + per * groups;
     }
@@ -349,7 +357,7 @@ static tnc_status contract_range(tnc_net* net, int64_t lo, int64_t hi, int mode,
 
     // workspace and batch
     char* ws = nullptr;
-    if (groups == 1) nb = call_batch(net, hi - lo, mode);
+    if (groups == 1) nb = call_batch(net, hi - lo, mode, batch_budget(net, mode));
     if (net->ws_user) {
         if (nb < 1) return fail(TNC_E_OOM, "workspace too small for one slice");
         ws = (char*)net->ws_user;
@@ -490,6 +498,17 @@ static tnc_status contract_range(tnc_net* net, int64_t lo, int64_t hi, int mode,
         }
     }
     *done = true;
+    return TNC_OK;
+}
+
+tnc_status tnc_variants_batch(tnc_net_t net, int64_t n_variants, int mode, size_t workspace_bytes, int64_t* slices) {
+    if (!net || !slices) return fail(TNC_E_INVALID, "NULL argument");
+    if (mode < TNC_FP32 || mode > TNC_SPLIT_FP16X2) return fail(TNC_E_INVALID, "unknown mode");
+    if (n_variants < 1 || n_variants > (1ll << 24)) return fail(TNC_E_INVALID, "n_variants must be in [1, 2^24]");
+    tnc_status st = ensure_plan(net);
+    if (st != TNC_OK) return st;
+    const Budget budget = workspace_bytes ? Budget{workspace_bytes, 65535} : own_budget(net, mode);
+    *slices = net->S_sorted.size() > 15 ? 0 : variants_batch(net, mode, 1ll << net->S_sorted.size(), n_variants, budget);
     return TNC_OK;
 }
 

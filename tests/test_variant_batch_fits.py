@@ -1,0 +1,78 @@
+"""A batch of several variants fits the workspace it was chosen for, although a
+smaller batch can need more bytes than a larger one (operands whose planes pass
+"tc_plane_cap_log2" are cut into panels). On the CPU the choice is swept over
+workspaces and counts by the library's own workspace plan; on the GPU a case whose
+evened batch needs more than the workspace equals one variant per call, bit for
+bit, and still shares launches."""
+
+import numpy as np
+import pytest
+
+from tnc_inputs import bitstring_variants, circuit_to_network, grid_rqc, random_bitstrings
+
+
+def _net(r, c, cycles, n_open, target, cap):
+    from paper_2205_00393_gb300 import Network
+    circuit = grid_rqc(r, c, cycles, 3, n_open=n_open)
+    net = Network.from_tn(circuit_to_network(circuit).as_complex64())
+    net.set_path(net.greedy_path())
+    net.set_slices(net.find_slices(target, 7))
+    if cap:
+        net.set_option("tc_plane_cap_log2", cap)
+    return circuit, net
+
+
+@pytest.mark.parametrize("r,c,cycles,n_open,target,mode,cap", [
+    (4, 5, 12, 2, 17, 2, 26), (4, 5, 12, 3, 19, 2, 25), (4, 5, 12, 4, 18, 1, 25), (4, 5, 12, 3, 17, 4, 24),
+    (4, 6, 12, 3, 23, 2, 0), (5, 5, 12, 2, 23, 2, 0), (4, 5, 12, 3, 17, 0, 0)])
+def test_batch_fits_its_workspace(libtnc, r, c, cycles, n_open, target, mode, cap):
+    _, net = _net(r, c, cycles, n_open, target, cap)
+    n = net.n_slices
+    peak = {}
+
+    def need(b):
+        if b not in peak:
+            peak[b] = net.arena(b, mode)["peak"]
+        return peak[b]
+
+    batched = 0
+    for slices in list(range(2 * n, min(48 * n, 200), max(1, n // 3))) + [19, 43]:
+        for count in (2, 3, 5, 7, 14, 28, 64):
+            got = net.variants_batch(count, mode, need(slices))
+            assert got == 0 or (got % n == 0 and got >= 2 * n and need(got) <= need(slices)), (slices, count)
+            batched += got > 0
+    assert batched
+    for count in (2, 9, 40):
+        got = net.variants_batch(count, mode)
+        assert got == 0 or need(got) <= max(need(1), 1 << 30)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_open,target,mode,cap,slices,count", [
+    (2, 17, 2, 26, 43, 14), (3, 19, 2, 25, 11, 5), (2, 17, 1, 25, 19, 3), (4, 18, 1, 26, 15, 7)])
+def test_evened_batch_needs_more_than_the_workspace(libtnc, n_open, target, mode, cap, slices, count):
+    """Workspaces that hold `slices` slices, but not the next smaller number of whole
+    variants that evens the batches out."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    circuit, net = _net(4, 5, 12, n_open, target, cap)
+    net.set_leaf_variants(*bitstring_variants(circuit, random_bitstrings(circuit, count, 5)))
+    size = net.arena(slices, mode)["peak"]
+    batch = net.variants_batch(count, mode, size)
+    assert batch == 0 or net.arena(batch, mode)["peak"] <= size  # before anything runs
+    ws = torch.empty(size, dtype=torch.uint8, device="cuda")
+    net.set_workspace(ws)
+    net.set_option("persistent", 0)
+    net.set_timing(True)
+    out = net.contract_variants(0, count, mode=mode).cpu().numpy()
+    shared = net.last_timings()[1]
+    net.check_device()
+    if batch:
+        assert net.stats()["last_batch"] == batch
+    net.set_timing(True)
+    one = np.concatenate([net.contract_variants(v, v + 1, mode=mode).cpu().numpy() for v in range(count)])
+    alone = net.last_timings()[1]
+    net.check_device()
+    assert np.array_equal(out, one)
+    assert shared < alone if batch else shared <= alone
