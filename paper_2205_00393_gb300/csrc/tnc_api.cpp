@@ -367,7 +367,14 @@ static tnc_status contract_range(tnc_net* net, int64_t lo, int64_t hi, int mode,
             if (net->ws_own) CUDA_TRY(cudaFree(net->ws_own));
             net->ws_own = nullptr;
             net->ws_own_bytes = 0;
-            CUDA_TRY(cudaMalloc(&net->ws_own, std::max<size_t>(need, kAlign)));
+            net->inv_key.clear();  // what it held is gone
+            const cudaError_t own_workspace = cudaMalloc(&net->ws_own, std::max<size_t>(need, kAlign));
+            if (own_workspace == cudaErrorMemoryAllocation && groups > 1) {  // one variant after another takes less
+                (void)cudaGetLastError();
+                net->ws_own = nullptr;
+                return TNC_OK;
+            }
+            CUDA_TRY(own_workspace);
             net->ws_own_bytes = need;
         }
         ws = (char*)net->ws_own;

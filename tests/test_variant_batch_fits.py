@@ -76,3 +76,31 @@ def test_evened_batch_needs_more_than_the_workspace(libtnc, n_open, target, mode
     net.check_device()
     assert np.array_equal(out, one)
     assert shared < alone if batch else shared <= alone
+
+
+@pytest.mark.gpu
+def test_batch_that_cannot_be_had(libtnc):
+    """On a full device the library's own workspace holds one variant's slices but not
+    the batch's: the variants then run one after another."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    mode, count = 2, 20
+    circuit, net = _net(4, 5, 12, 4, 18, 0)
+    net.set_leaf_variants(*bitstring_variants(circuit, random_bitstrings(circuit, count, 5)))
+    net.set_option("persistent", 0)
+    out = torch.empty((count, net.n_out), dtype=torch.complex128, device="cuda")
+    one = np.concatenate([net.contract_variants(v, v + 1, mode=mode).cpu().numpy() for v in range(count)])
+    batch = net.variants_batch(count, mode)
+    left = 400 << 20
+    assert net.arena(net.n_slices, mode)["peak"] < left // 4 and net.arena(batch, mode)["peak"] > left + (200 << 20)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    full = torch.empty(torch.cuda.mem_get_info()[0] - left, dtype=torch.uint8, device="cuda")
+    net.contract_variants(0, count, mode=mode, out=out)
+    net.check_device()
+    del full
+    torch.cuda.empty_cache()
+    assert np.array_equal(out.cpu().numpy(), one)
+    net.contract_variants(0, count, mode=mode, out=out)  # and in a batch again
+    assert net.stats()["last_batch"] == batch and np.array_equal(out.cpu().numpy(), one)
