@@ -127,24 +127,19 @@ __device__ __forceinline__ void two_sum_into(f32x2& a, f32x2 b, f32x2& c) {
     c = add2(c, e);
 }
 
-// Operand pointer of a tile. Alone in a launch (BAR 0) the operands were
-// written by earlier launches and may be read through the read-only path;
-// inside the persistent executor (BAR 1) other CTAs of the same launch wrote
-// them, so the loads stay on the coherent path.
-template <int BAR> struct OperandPtr { using type = const float2* __restrict__; };
-template <> struct OperandPtr<1> { using type = const float2*; };
-
 // The gather, staging and products of one output tile (slice z, slice id
 // slice0 + z) of the contraction described by p.
 // LEAN: registers are short (grouped contractions with their parameters in shared
 // memory, the persistent executor).
-template <int BAR, int NTH, int RM, int WN, bool LEAN = false> struct TileWork {
+template <int NTH, int RM, int WN, bool LEAN = false> struct TileWork {
     using Cfg = TileCfg<NTH, RM, WN>;
     static constexpr int EA = Cfg::BM * BK / NTH, EB = Cfg::BN * BK / NTH;  // elements a thread gathers per k-tile
     static constexpr int RP = RM / 2;                                      // row pairs of a thread
     GemmStage<NTH, RM, WN>& sm;
     int64_t M, N, K, m0, n0;
-    typename OperandPtr<BAR>::type A, B;
+    // plain pointers: the predecessor launch, or another CTA of the persistent executor,
+    // may write the operands while this CTA decodes its parameters (launch.cuh)
+    const float2 *A, *B;
     bool a_kfast, b_nfast;
     bool full;  // no element of the tile lies past M, N or K
     int64_t sa[LEAN ? 1 : log2_of(EA)], sb[LEAN ? 1 : log2_of(EB)];  // offsets of the bits of an element's number (the same in every thread)
@@ -152,7 +147,8 @@ template <int BAR, int NTH, int RM, int WN, bool LEAN = false> struct TileWork {
     int64_t khA = 0, khB = 0;  // offsets of the k-tile to gather
     float2 ra[EA], rb[EB];
 
-    // Fills the offset tables; a barrier must follow before the first gather.
+    // Fills kstepA, kstepB (and sm.sa, sm.sb); the wait for the predecessor and a
+    // barrier must follow before the first gather.
     __device__ __forceinline__ TileWork(const GemmParams& p, int64_t tile, int z, int64_t slice0,
                                         GemmStage<NTH, RM, WN>& stage)
         : sm(stage) {
@@ -335,7 +331,7 @@ template <int BAR, int NTH, int RM, int WN, bool LEAN = false> struct TileWork {
 template <int BAR = 0, int NTH = 256, int RM = 4, int WN = 2, bool LEAN = BAR == 1>
 __device__ __forceinline__ void gemm_tile(const GemmParams& p, int64_t tile, int z, int64_t slice0,
                                           GemmSmemT<NTH, RM, WN>& sm) {
-    using W = TileWork<BAR, NTH, RM, WN, LEAN>;
+    using W = TileWork<NTH, RM, WN, LEAN>;
     constexpr int RP = W::RP;
     const int tid = threadIdx.x;
     W w(p, tile, z, slice0, sm);
@@ -442,7 +438,7 @@ template <int NTH, int WN, int CL>
 __device__ __forceinline__ void gemm_tile_cluster(const GemmParams& p, int64_t tile, uint32_t rank, int z, int64_t slice0,
                                                   GemmClusterSmem<NTH, WN>& sm) {
     static_assert(CL == 2 || CL == 4 || CL == 8, "a CTA owns whole complex outputs");
-    using W = TileWork<0, NTH, 4, WN>;
+    using W = TileWork<NTH, 4, WN>;
     constexpr int E = 16 / CL;
     const int tid = threadIdx.x;
     W w(p, tile, z, slice0, sm);

@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(GT, 3) k_gemm_f32_group(const GemmParams* __re
 
 // FP64 partial sums of a contraction with R = M*N <= 64 outputs.
 __global__ void __launch_bounds__(256) k_root_partials(const __grid_constant__ RootParams rp,
-                                                       double2* __restrict__ partials) {
+                                                       double2* partials) {
     dep_trigger();
     dep_wait();
     __shared__ double2 red[256];
@@ -86,8 +86,7 @@ __global__ void __launch_bounds__(256) k_root_partials(const __grid_constant__ R
 
 // out[y][r] += sum_i partials[y][i][perm(r)], y = blockIdx.y (a fixed order: accumulate_items)
 __global__ void __launch_bounds__(256) k_accumulate_partials(const double2* partials, int count,
-                                                             const __grid_constant__ PermParams pp,
-                                                             double2* __restrict__ out) {
+                                                             const __grid_constant__ PermParams pp, double2* out) {
     dep_trigger();
     dep_wait();
     __shared__ double2 red[256];
@@ -96,7 +95,7 @@ __global__ void __launch_bounds__(256) k_accumulate_partials(const double2* part
 }
 
 // out[y][r] += sum_z src_(y batch + z)[perm(r)] in FP64, z ascending, y = blockIdx.y
-__global__ void k_slice_sum_f32(const __grid_constant__ SumParams p, int batch, double2* __restrict__ out) {
+__global__ void k_slice_sum_f32(const __grid_constant__ SumParams p, int batch, double2* out) {
     dep_trigger();
     dep_wait();
     const int64_t R = 1ll << p.obits;

@@ -7,8 +7,9 @@
 // with the launch itself. Every CTA of a kernel that is launched this way calls
 // dep_wait() before it ends, so that its completion implies its predecessor's.
 // Data that a predecessor writes is read through plain pointers: a load through
-// the read-only path (__ldg, __restrict__) may be moved above the wait, unless its
-// address itself comes from shared memory behind a barrier after it.
+// the read-only path (__ldg) or a __restrict__ pointer, of which nothing else is
+// supposed to write the target, may be moved above the wait. __restrict__ is for the
+// uploaded tables.
 //
 // dep_trigger() in a kernel lets its successor start early. That pays for short
 // kernels and costs in long ones, whose successor's waiting CTAs take places and
