@@ -431,6 +431,7 @@ __device__ __forceinline__ f32x2 ld_cluster(const f32x2* p, uint32_t rank) {
     return v;
 }
 __device__ __forceinline__ void cluster_barrier() {
+    __syncwarp();  // .aligned: the whole warp executes it together, also after a predicated store
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
