@@ -443,7 +443,8 @@ __device__ __forceinline__ void tc_tile(const CUtensorMap* tmA, const CUtensorMa
             any = true;
             __syncwarp();
         }
-        if (*abort_flag && any && elect_one()) {
+        // (other warps may set the flag between two lanes' reads: the warp decides together)
+        if (__any_sync(0xffffffffu, *abort_flag) && any && elect_one()) {
             mma_commit(smem_u32(&sh.drain_bar));
             for (uint32_t i = 0; i < spin && !mbar_try(smem_u32(&sh.drain_bar), 0); ++i) {
             }
@@ -776,7 +777,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                 __syncwarp();
                 if (kbi == kpc - 1) ++cgl;
             }
-        if (*abort_flag && any && elect_one()) {
+        // (other warps may set the flag between two lanes' reads: the warp decides together)
+        if (__any_sync(0xffffffffu, *abort_flag) && any && elect_one()) {
             mma_commit_pair(smem_u32(&sh.drain_bar));
             for (uint32_t i = 0; i < spin && !mbar_try(smem_u32(&sh.drain_bar), 0); ++i) {
             }

@@ -21,3 +21,13 @@ def test_aligned_cluster_barriers_follow_a_syncwarp():
     for name, src in _sources():
         for m in re.finditer(r'asm volatile\("barrier\.cluster\.[^"]*\.aligned', src):
             assert src[:m.start()].rstrip().endswith("__syncwarp();"), name
+
+
+def test_elections_do_not_depend_on_a_flag_of_another_warp():
+    found = 0
+    for name, src in _sources():
+        for line in src.splitlines():
+            if "elect_one()" in line and "bool elect_one" not in line:
+                found += 1
+                assert "abort_flag" not in line or "__any_sync(0xffffffffu, *abort_flag)" in line, (name, line.strip())
+    assert found >= 4
