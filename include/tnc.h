@@ -365,7 +365,9 @@ tnc_status tnc_worklist_many_json(int n, const tnc_net_t* nets, int64_t batch, i
  *                  tnc_contract_variants run a network whose leaves,
  *                  intermediates and tables fit one CTA's shared memory with
  *                  a CTA per slice, every slice of every variant in one
- *                  launch and a sum (timing record of kind 9), if a slice
+ *                  launch and a sum (timing record of kind 9; a caller's
+ *                  workspace holds the partial results, in rounds of as many
+ *                  as it has room for), if a slice
  *                  has at most 3 2^16 complex multiply-accumulates (3 2^17
  *                  for calls of 64 slices and more); every other call
  *                  runs one launch per level, which is ahead of the

@@ -304,7 +304,7 @@ struct tnc_net {
     std::map<std::string, std::pair<double, double>> cost_cache;  // level_cost results (launches, seconds)
     std::map<std::string, std::unique_ptr<DeviceWorkList>> worklists;
     std::map<std::string, std::unique_ptr<TinyPlan>> tiny_plans;
-    double2* d_tiny = nullptr;       // its partial results
+    double2* d_tiny = nullptr;       // their partial results without a caller's workspace
     size_t d_tiny_cap = 0;
     std::map<std::string, BackwardSizes> backward_sizes;                     // by what they depend on
     std::map<std::string, std::unique_ptr<BackwardPlan>> backward_plans;     // and the workspace

@@ -191,8 +191,13 @@ tnc_status tiny_contract(tnc_net* net, int mode, int64_t first, int64_t stride, 
         for (int flat : {0, 1}) tp.arena[flat] = tp.nb < 1 ? 0 : (size_t)plan_arena(net, tp.nb, mode, flat == 0).peak;
     }
     if (tp.nb < 1) return TNC_OK;
+    // Partial results: in the caller's workspace, in rounds of as many as it holds (calls
+    // on several streams then share no memory that their workspaces do not), or in a
+    // buffer of the network's own.
     const size_t need = (size_t)(per * groups) << P.obits;
-    if (need > net->d_tiny_cap) {
+    const int64_t room = net->ws_user ? (int64_t)(given / sizeof(double2) >> P.obits) : per * groups;
+    if (room < 1) return TNC_OK;
+    if (!net->ws_user && need > net->d_tiny_cap) {
         double2* m = nullptr;
         if (cudaMalloc(&m, need * sizeof(double2)) != cudaSuccess) {  // the workspace's executors need none
             (void)cudaGetLastError();
@@ -205,14 +210,10 @@ tnc_status tiny_contract(tnc_net* net, int mode, int64_t first, int64_t stride, 
     tnc::TinyParams p = tp.prm;
     p.leaves = net->d_leaves;
     p.variants = net->d_var;
-    p.first = first;
     p.stride = stride;
-    p.per = per;
-    p.groups = groups;
     p.sbits = (int)net->S_sorted.size();
     p.obits = P.obits;
-    p.partials = net->d_tiny;
-    p.out = out;
+    p.partials = net->ws_user ? static_cast<double2*>(net->ws_user) : net->d_tiny;
     p.err = net->d_err;
     tnc::PermParams pp{};
     pp.obits = P.obits;
@@ -222,14 +223,24 @@ tnc_status tiny_contract(tnc_net* net, int mode, int64_t first, int64_t stride, 
         for (const NodePlan& np : P.nodes)
             cm += std::ldexp(1.0, np.mb + np.nb + np.kb) * (np.per_slice ? (double)(per * groups) : 1.0);
     CUDA_TRY(timed_begin(net, -1, K_PERSIST, (int)std::min<int64_t>(per, 0x7fffffff), s, cm));
-    CUDA_TRY(tnc::launch_tiny(p, pp, s));
+    net->launches -= 1;
+    const int64_t dg = std::max<int64_t>(1, std::min(groups, room / per)), dj = std::min(per, room);
+    for (int64_t g = 0; g < groups; g += dg)
+        for (int64_t j = 0; j < per; j += dj) {
+            p.first = first + g * stride + j;
+            p.per = std::min(dj, per - j);
+            p.groups = std::min(dg, groups - g);
+            p.out = out + (g << P.obits);
+            p.clear = j == 0;
+            CUDA_TRY(tnc::launch_tiny(p, pp, s));
+            net->launches += 2;  // the slices and their sum
+        }
     CUDA_TRY(timed_end(net, s));
-    net->launches += 1;  // the sum
     net->last_batch = tp.nb;
     net->last_arena_bytes[0] = tp.arena[0];
     net->last_arena_bytes[1] = net->persist_deps ? tp.arena[1] : 0;
     net->last_persist_deps = net->persist_deps && tp.arena[1] <= (given ? given : std::max<size_t>(tp.arena[0], (size_t)1 << 30));
-    net->inv_key.clear();  // nothing of it is in the workspace
+    net->inv_key.clear();  // the workspace may hold partial results
     *done = true;
     return TNC_OK;
 }

@@ -390,6 +390,7 @@ struct TinyParams {
     int sbits, obits;            // variant = slice id >> sbits; 2^obits outputs
     double2* partials;           // [groups * per][outputs]
     double2* out;                // [groups][outputs]
+    int clear;                   // out begins at zero (else the sums are added to it)
     int* err;                    // cleared (nothing here waits on another CTA)
 };
 size_t tiny_smem_bytes(int64_t data_elems, int64_t words);

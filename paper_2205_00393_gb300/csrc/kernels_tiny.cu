@@ -59,8 +59,9 @@ __global__ void __launch_bounds__(TT) k_tiny(const __grid_constant__ TinyParams 
     const int tid = threadIdx.x;
     for (int i = tid; i < p.words / 4; i += TT) reinterpret_cast<uint4*>(W)[i] = reinterpret_cast<const uint4*>(p.tables)[i];
     for (int i = tid; i < p.leaf_elems; i += TT) data[i] = p.leaves[i];
-    for (int64_t i = (int64_t)blockIdx.x * TT + tid; i < p.groups << p.obits; i += (int64_t)gridDim.x * TT)
-        p.out[i] = make_double2(0.0, 0.0);  // k_tiny_sum adds into it
+    if (p.clear)
+        for (int64_t i = (int64_t)blockIdx.x * TT + tid; i < p.groups << p.obits; i += (int64_t)gridDim.x * TT)
+            p.out[i] = make_double2(0.0, 0.0);  // k_tiny_sum adds into it
     if (blockIdx.x == 0 && tid == 0) *p.err = 0;
     __syncthreads();
     uint32_t* const base = W + p.o_base;  // element offset of every tensor in data
