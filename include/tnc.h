@@ -26,6 +26,13 @@
  *  - `stream` is a cudaStream_t (NULL = legacy default stream). All device
  *    work of a call is enqueued on it; calls return before it completes.
  *  - A network object is not thread-safe; use one per thread.
+ *  - Stream capture: the first call of its kind (mode, sizes, workspace, options,
+ *    leaf data) plans, allocates, uploads and waits; make it before a capture. A graph
+ *    reads the leaves of its own time. It holds the addresses of the network's
+ *    tables and buffers and is valid until the network is planned anew or destroyed,
+ *    its workspace changes hands or a call of another kind rewrites the tables of
+ *    the per-level launches; those of a network that runs on one CTA per slice are
+ *    kept until the network is destroyed.
  */
 #ifndef TNC_H
 #define TNC_H

@@ -155,6 +155,7 @@ struct TinyPlan {
     tnc::TinyParams prm{};
     void* mem = nullptr;
     double cmacs = 0;  // of a slice, invariants included
+    bool captured = false;  // a graph holds its tables: they stay until the network goes
     // what the last call's sizes come to for the other executors (statistics; a
     // workspace that is too small stays an error): slices asked for, workspace given
     int64_t want = -1, nb = 0;
@@ -306,6 +307,10 @@ struct tnc_net {
     std::map<std::string, std::unique_ptr<TinyPlan>> tiny_plans;
     double2* d_tiny = nullptr;       // their partial results without a caller's workspace
     size_t d_tiny_cap = 0;
+    bool d_tiny_captured = false;    // a graph holds that buffer
+    // what captured calls hold, after its place was taken: freed with the network
+    std::vector<std::unique_ptr<TinyPlan>> tiny_kept;
+    std::vector<double2*> d_tiny_kept;
     std::map<std::string, BackwardSizes> backward_sizes;                     // by what they depend on
     std::map<std::string, std::unique_ptr<BackwardPlan>> backward_plans;     // and the workspace
     double timed_persist_tc_cmacs = 0.0;  // tensor-core share of the timed persistent launches
@@ -323,6 +328,7 @@ struct tnc_net {
         if (d_prof) cudaFree(d_prof);
         if (d_var) cudaFree(d_var);
         if (d_tiny) cudaFree(d_tiny);
+        for (double2* p : d_tiny_kept) cudaFree(p);
         for (cudaEvent_t e : ev_pool) cudaEventDestroy(e);
     }
 };
@@ -483,6 +489,9 @@ struct Budget {
 };
 Budget own_budget(const tnc_net* net, int mode);
 Budget batch_budget(const tnc_net* net, int mode);
+// Whether the stream is being captured: allocations, uploads and waits then fail (and
+// end the capture).
+bool capturing(cudaStream_t s);
 // Slices per batch of a call of `want` slices, 0 if the budget does not hold one. Its
 // arena fits the budget.
 int64_t call_batch(const tnc_net* net, int64_t want, int mode, const Budget& budget);

@@ -624,6 +624,12 @@ cudaError_t timed_end(tnc_net* net, cudaStream_t s) {
     return cudaEventRecord(net->ev_pool[net->timed.back().ev + 1], s);
 }
 
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) (void)cudaGetLastError();
+    return st != cudaStreamCaptureStatusNone;
+}
+
 int64_t pick_batch(const tnc_net* net, int64_t want, size_t budget, int mode) {
     int64_t lo = 1, hi = std::max<int64_t>(1, std::min<int64_t>(want, 65535));
     if ((size_t)plan_arena(net, 1, mode).peak > budget) return 0;

@@ -169,7 +169,12 @@ tnc_status tiny_contract(tnc_net* net, int mode, int64_t first, int64_t stride, 
     if (net->persist_test_stall || per < 1 || groups < 1 || per > fit || groups > fit / per) return TNC_OK;
     const std::string key = plan_key(net, mode, 0);
     auto it = net->tiny_plans.find(key);
+    // a graph that a call is captured into keeps the addresses of its tables and
+    // buffer: neither is made during a capture (a call alike comes before it; else
+    // the other executors see to the call), and neither is freed while the network lives
+    const bool capture = capturing(s);
     if (it == net->tiny_plans.end()) {
+        if (capture) return TNC_OK;
         auto tp = std::make_unique<TinyPlan>();
         Tables T;
         if (build_tiny(net, mode, T, tp->prm, tp->cmacs)) {
@@ -178,7 +183,11 @@ tnc_status tiny_contract(tnc_net* net, int mode, int64_t first, int64_t stride, 
             CUDA_TRY(cudaStreamSynchronize(s));  // the host words may go
             tp->prm.tables = static_cast<const uint32_t*>(tp->mem);
         }
-        if (net->tiny_plans.size() >= 8) net->tiny_plans.clear();
+        if (net->tiny_plans.size() >= 8) {
+            for (auto& [k, plan] : net->tiny_plans)
+                if (plan->captured) net->tiny_kept.push_back(std::move(plan));
+            net->tiny_plans.clear();
+        }
         it = net->tiny_plans.emplace(key, std::move(tp)).first;
     }
     TinyPlan& tp = *it->second;
@@ -198,14 +207,22 @@ tnc_status tiny_contract(tnc_net* net, int mode, int64_t first, int64_t stride, 
     const int64_t room = net->ws_user ? (int64_t)(given / sizeof(double2) >> P.obits) : per * groups;
     if (room < 1) return TNC_OK;
     if (!net->ws_user && need > net->d_tiny_cap) {
+        if (capture) return TNC_OK;
         double2* m = nullptr;
-        if (cudaMalloc(&m, need * sizeof(double2)) != cudaSuccess) {  // the workspace's executors need none
+        const size_t size = std::max(need, std::min<size_t>(2 * net->d_tiny_cap, kTinyMaxPartials));  // (so few are kept)
+        if (cudaMalloc(&m, size * sizeof(double2)) != cudaSuccess) {  // the workspace's executors need none
             (void)cudaGetLastError();
             return TNC_OK;
         }
-        if (net->d_tiny) CUDA_TRY(cudaFree(net->d_tiny));
+        if (net->d_tiny_captured) net->d_tiny_kept.push_back(net->d_tiny);
+        else if (net->d_tiny) CUDA_TRY(cudaFree(net->d_tiny));
         net->d_tiny = m;
-        net->d_tiny_cap = need;
+        net->d_tiny_cap = size;
+        net->d_tiny_captured = false;
+    }
+    if (capture) {
+        tp.captured = true;
+        net->d_tiny_captured |= !net->ws_user;
     }
     tnc::TinyParams p = tp.prm;
     p.leaves = net->d_leaves;

@@ -90,3 +90,62 @@ def test_variants_in_rounds(lib, per_slice):
     got, tiny = _one_cta(net, lambda: net.contract_variants(1, 9))
     assert tiny
     assert np.all(np.abs(got - want) <= 1e-10 * np.abs(want).max())
+
+
+def _captured(net, lo, hi, mode):
+    """A graph of one call, after a call alike."""
+    out = torch.zeros(net.n_out, dtype=torch.complex128, device="cuda")
+    net.contract(lo, hi, mode, out=out)
+    torch.cuda.synchronize()
+    want = out.cpu().numpy()
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        net.contract(lo, hi, mode, out=out)
+    return graph, out, want
+
+
+def _replays(graph, out, want):
+    out.fill_(7.0)
+    graph.replay()
+    torch.cuda.synchronize()
+    return np.array_equal(out.cpu().numpy(), want)
+
+
+def test_captured_call_outlives_larger_ones(lib):
+    """The buffer of a captured call's partial results is not freed by a longer range."""
+    net = _net(4, 5, 8, 1, 7)
+    graphs = [_captured(net, lo, hi, 0) for lo, hi in ((1, 3), (0, 200))]
+    net.contract(0, 4096)
+    hold = [torch.full((1 << 18,), 3.0, dtype=torch.float64, device="cuda") for _ in range(8)]  # over what is free
+    torch.cuda.synchronize()
+    assert all(_replays(*g) for g in graphs)
+    del hold
+
+
+def test_captured_call_outlives_other_plans(lib):
+    """Its tables are not freed by the plans of other calls that take their place."""
+    net = _net(3, 4, 8, 2, 8)
+    graph = _captured(net, 0, net.n_slices, 0)
+    want = graph[2]
+    for cap in range(16, 40):  # another plan key each
+        net.set_option("tc_plane_cap_log2", cap)
+        assert np.array_equal(net.contract().cpu().numpy(), want)
+    hold = [torch.full((1 << 14,), 3.0, dtype=torch.float64, device="cuda") for _ in range(64)]
+    assert _replays(*graph)
+    del hold
+
+
+def test_first_call_in_a_capture_falls_back(lib):
+    """A longer range than any before it, captured: nothing is allocated on this path; the
+    per-level launches, which have run alike, take the call."""
+    net = _net(3, 4, 8, 2, 8)
+    out = torch.zeros(net.n_out, dtype=torch.complex128, device="cuda")
+    net.contract(0, 1)  # one CTA per slice
+    net.set_option("persistent", 0)
+    want = net.contract(out=out).cpu().numpy()
+    net.set_option("persistent", 2)
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=stream):
+        net.contract(out=out)
+    assert _replays(graph, out, want)
