@@ -31,8 +31,8 @@
  *    reads the leaves of its own time. It holds the addresses of the network's
  *    tables and buffers and is valid until the network is planned anew or destroyed,
  *    its workspace changes hands or a call of another kind rewrites the tables of
- *    the per-level launches; those of a network that runs on one CTA per slice are
- *    kept until the network is destroyed.
+ *    the per-level launches; those of a network that runs on one CTA per slice and of
+ *    an adjoint pass are kept until the network is destroyed.
  */
 #ifndef TNC_H
 #define TNC_H

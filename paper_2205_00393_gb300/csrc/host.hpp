@@ -190,6 +190,7 @@ struct BackwardPlan {
     std::vector<int2> map;                                // CTA maps of the grouped contractions
     int64_t top = 0;                                      // workspace bytes
     int64_t zero_bytes = 0;                               // FP64 sums at the workspace's start, leaf gradients first
+    bool captured = false;  // a graph holds its tables: they stay until the network goes
     // device copies
     void* mem = nullptr;
     const tnc::GemmParams* d_gemm = nullptr;
@@ -313,6 +314,7 @@ struct tnc_net {
     std::vector<double2*> d_tiny_kept;
     std::map<std::string, BackwardSizes> backward_sizes;                     // by what they depend on
     std::map<std::string, std::unique_ptr<BackwardPlan>> backward_plans;     // and the workspace
+    std::vector<std::unique_ptr<BackwardPlan>> backward_kept;  // captured ones whose place was taken
     double timed_persist_tc_cmacs = 0.0;  // tensor-core share of the timed persistent launches
     unsigned long long* d_prof = nullptr;  // "persist_profile": per task type time, count, wait
 

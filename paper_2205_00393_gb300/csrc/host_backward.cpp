@@ -751,30 +751,40 @@ tnc_status tnc_contract_backward(tnc_net_t net, int64_t lo, int64_t hi, int mode
         return fail(TNC_E_OOM, "backward workspace for one slice exceeds the budget (" + std::to_string(sz.need) + " bytes)");
     net->last_keep_every = sz.keep_every;
     const int64_t nb = sz.nb;
-    // by levels when its workspace is there or can be had
+    // by levels when its workspace is there or can be had, and, during a capture, its
+    // plan: a plan is uploaded, the node-by-node pass has its parameters in its launches
+    const int64_t tail = (hi - lo) % nb;
+    auto place = [&](size_t bytes) -> char* {
+        if (net->ws_user && net->ws_user_bytes >= bytes) return (char*)net->ws_user;
+        return net->ws_own && net->ws_own_bytes >= bytes ? (char*)net->ws_own : nullptr;
+    };
+    auto plan_at = [&](const char* at) {
+        return plan_key(net, mode, nb) + ":" + std::to_string(tail) + ":" + std::to_string((uintptr_t)at) + ":" +
+               std::to_string((uintptr_t)net->d_leaves) + ":" + mask;
+    };
+    const bool capture = capturing(s);
     bool levels = sz.need_levels > 0;
+    if (net->ws_user && net->ws_user_bytes < sz.need_levels && net->ws_user_bytes >= sz.need)
+        levels = false;  // the caller's workspace fits node by node only
+    if (levels && capture) {
+        char* const at = place(sz.need_levels);
+        levels = at && net->backward_plans.count(plan_at(at));
+    }
     size_t need = levels ? sz.need_levels : sz.need;
-    char* ws = nullptr;
-    if (net->ws_user && net->ws_user_bytes >= need) {
-        ws = (char*)net->ws_user;
-    } else if (levels && net->ws_user && net->ws_user_bytes >= sz.need) {  // the caller's fits node by node only
-        levels = false;
-        need = sz.need;
-        ws = (char*)net->ws_user;
-    } else {
-        if (net->ws_own_bytes < need) {
-            if (net->ws_own) CUDA_TRY(cudaFree(net->ws_own));
+    char* ws = place(need);
+    if (!ws) {
+        if (net->ws_own) CUDA_TRY(cudaFree(net->ws_own));
+        net->ws_own = nullptr;
+        net->ws_own_bytes = 0;
+        size_t bytes = std::max(need, sz.need);  // (either way fits then)
+        if (bytes > sz.need && cudaMalloc(&net->ws_own, bytes) != cudaSuccess) {
+            (void)cudaGetLastError();
             net->ws_own = nullptr;
-            net->ws_own_bytes = 0;
-            if (levels && need > sz.need && cudaMalloc(&net->ws_own, need) != cudaSuccess) {
-                (void)cudaGetLastError();
-                net->ws_own = nullptr;
-                levels = false;
-                need = sz.need;
-            }
-            if (!net->ws_own) CUDA_TRY(cudaMalloc(&net->ws_own, need));
-            net->ws_own_bytes = need;
+            levels = false;
+            need = bytes = sz.need;
         }
+        if (!net->ws_own) CUDA_TRY(cudaMalloc(&net->ws_own, bytes));
+        net->ws_own_bytes = bytes;
         ws = (char*)net->ws_own;
     }
     net->last_backward_bytes = need;
@@ -787,17 +797,20 @@ tnc_status tnc_contract_backward(tnc_net_t net, int64_t lo, int64_t hi, int mode
     bw.ws = ws;
     bw.keep_every = sz.keep_every;
     if (levels) {
-        const int64_t tail = (hi - lo) % nb;
-        const std::string pkey = plan_key(net, mode, nb) + ":" + std::to_string(tail) + ":" + std::to_string((uintptr_t)ws) +
-                                 ":" + std::to_string((uintptr_t)net->d_leaves) + ":" + mask;
+        const std::string pkey = plan_at(ws);
         auto it = net->backward_plans.find(pkey);
         if (it == net->backward_plans.end()) {
             auto bp = std::make_unique<BackwardPlan>();
             build_backward_plan(bw, nb, tail, *bp);
             if ((st = upload_backward_plan(*bp, s)) != TNC_OK) return st;
-            if (net->backward_plans.size() >= 4) net->backward_plans.clear();
+            if (net->backward_plans.size() >= 4) {
+                for (auto& [k, plan] : net->backward_plans)
+                    if (plan->captured) net->backward_kept.push_back(std::move(plan));
+                net->backward_plans.clear();
+            }
             it = net->backward_plans.emplace(pkey, std::move(bp)).first;
         }
+        it->second->captured |= capture;
         const BackwardPlan& bp = *it->second;
         bw.leaf_grad = 0;
         CUDA_TRY(cudaMemsetAsync(ws, 0, bp.zero_bytes, s));
