@@ -717,7 +717,9 @@ tnc_status tnc_contract_backward(tnc_net_t net, int64_t lo, int64_t hi, int mode
             d.exec = false;
             d.nb = nb;
             d.keep_every = keep_every;
-            backward_run(d, lo, std::min(hi, lo + nb), grad_out_c128);
+            // a whole batch and the smaller last one, which can need more: its operand
+            // planes may stay below the cap at which the others are cut into panels
+            backward_run(d, lo, std::min(hi, lo + nb + (hi - lo) % nb), grad_out_c128);
             return (size_t)d.A.top;
         };
         if (net->backward_keep_every > 0) keep_every = net->backward_keep_every;
