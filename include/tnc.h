@@ -263,10 +263,11 @@ tnc_status tnc_contract_many(int n, const tnc_net_t* nets, const int64_t* slice_
  * "tc_cuts": per split mode, [node index, A row-panel bits, B row-panel bits,
  * K-panel bits, K-split bits] of every tensor-core-eligible contraction for
  * the last batch size ("tc_cut_batch"); "persistent" and "persist_deps" (the
- * options); "last_persist_deps": 1 if the last persistent tnc_contract ran
- * with per-entry dependencies; "last_workspace": [bytes of the reusing
+ * options); "last_persist_deps": 1 if the last tnc_contract ran on the persistent
+ * executor with per-entry dependencies; "last_workspace": [bytes of the reusing
  * layout, bytes without reuse (0 if not considered)] for the last
- * tnc_contract batch; "level_cost": per mode, [per-level launches,
+ * tnc_contract batch ([0, 0]: one CTA per slice, which lays out no tensors;
+ * "last_batch" is then what the workspace would hold); "level_cost": per mode, [per-level launches,
  * estimated seconds at peak rates] of that batch with the slice-invariant
  * levels; "timed_persist_tc_cmacs": the
  * complex multiply-accumulates that timed persistent launches (since

@@ -156,10 +156,10 @@ struct TinyPlan {
     void* mem = nullptr;
     double cmacs = 0;  // of a slice, invariants included
     bool captured = false;  // a graph holds its tables: they stay until the network goes
-    // what the last call's sizes come to for the other executors (statistics; a
-    // workspace that is too small stays an error): slices asked for, workspace given
+    // slices of the last call, the caller's workspace, and how many slices that holds for
+    // the other executors (none: an error, also here)
     int64_t want = -1, nb = 0;
-    size_t given = 0, arena[2] = {0, 0};
+    size_t given = 0;
     ~TinyPlan() {
         if (mem) cudaFree(mem);
     }

@@ -197,7 +197,6 @@ tnc_status tiny_contract(tnc_net* net, int mode, int64_t first, int64_t stride, 
         tp.want = per;
         tp.given = given;
         tp.nb = call_batch(net, per, mode, batch_budget(net, mode));
-        for (int flat : {0, 1}) tp.arena[flat] = tp.nb < 1 ? 0 : (size_t)plan_arena(net, tp.nb, mode, flat == 0).peak;
     }
     if (tp.nb < 1) return TNC_OK;
     // Partial results: in the caller's workspace, in rounds of as many as it holds (calls
@@ -254,9 +253,8 @@ tnc_status tiny_contract(tnc_net* net, int mode, int64_t first, int64_t stride, 
         }
     CUDA_TRY(timed_end(net, s));
     net->last_batch = tp.nb;
-    net->last_arena_bytes[0] = tp.arena[0];
-    net->last_arena_bytes[1] = net->persist_deps ? tp.arena[1] : 0;
-    net->last_persist_deps = net->persist_deps && tp.arena[1] <= (given ? given : std::max<size_t>(tp.arena[0], (size_t)1 << 30));
+    net->last_arena_bytes[0] = net->last_arena_bytes[1] = 0;  // no layout of tensors, no task dependencies
+    net->last_persist_deps = false;
     net->inv_key.clear();  // the workspace may hold partial results
     *done = true;
     return TNC_OK;

@@ -149,3 +149,18 @@ def test_first_call_in_a_capture_falls_back(lib):
     with torch.cuda.graph(graph, stream=stream):
         net.contract(out=out)
     assert _replays(graph, out, want)
+
+
+def test_statistics_of_a_one_cta_call(lib):
+    """They name no layout and no executor that did not run; a workspace of two slices is
+    still reported as one."""
+    net = _net(3, 4, 8, 2, 8)
+    net.set_option("persistent", 1)
+    net.contract()
+    st = net.stats()
+    assert st["last_persist_deps"] == 1 and min(st["last_workspace"]) > 0
+    net.set_option("persistent", 2)
+    net.set_workspace(torch.empty(net.workspace_bytes(2), dtype=torch.uint8, device="cuda"))
+    assert _one_cta(net, net.contract)[1]
+    st = net.stats()
+    assert st["last_persist_deps"] == 0 and st["last_workspace"] == [0, 0] and st["last_batch"] == 2
