@@ -225,11 +225,12 @@ static void level_cost_uncached(tnc_net* net, int mode, int64_t b, bool with_inv
 
 // Launches and estimated seconds of one batch of b slices on the per-level
 // executor (the slice-invariant levels included when with_inv), added to
-// *launches and *seconds: one grouped launch per level for its FP32
-// contractions of fewer than 256 tiles (those of long K count with it), one for
-// each larger one, three per tensor-core contraction (two operand splits and the
-// GEMM), two for the final contraction. A contraction's time is estimated as
-// the larger of its flops at 300 TFLOP/s and its operand and result bytes,
+// *launches and *seconds: one grouped launch per level for its small FP32
+// contractions, one for each of 256 tiles or more or of long K, one per fused stem
+// group, tc_launches per tensor-core contraction, two for the final contraction.
+// (tnc_contract_many merges the grouped launches of its networks, and their final
+// contractions; its choice of the executor adds up the networks' own launches.) A
+// contraction's time is estimated as the larger of its flops at 300 TFLOP/s and its operand and result bytes,
 // 8 (MK + KN + MN) per slice, at 6 TB/s. Cached by plan_key.
 void level_cost(tnc_net* net, int mode, int64_t b, bool with_inv, double* launches, double* seconds) {
     const std::string key = plan_key(net, mode, b) + (with_inv ? ":i" : ":p");
@@ -244,6 +245,22 @@ void level_cost(tnc_net* net, int mode, int64_t b, bool with_inv, double* launch
     *seconds += it->second.second;
 }
 
+// Launches of one tensor-core contraction of b slices (launch_tc_contraction).
+static double tc_launches(const tnc_net* net, int mode, const NodePlan& np, int64_t b) {
+    const Plan& P = net->plan;
+    const TcCut c = tc_cut(net, mode, np.mb, np.nb, np.kb, b);
+    auto batch = [&](int v) {  // an operand that is the same in every slice is split once
+        return v < net->n_leaves ? (P.sl[v].empty() ? 1 : (int)b) : (P.per_slice[v] ? (int)b : 1);
+    };
+    const int pA = c.pA, pB = c.pB, pK = c.pK;
+    int64_t splits = 1;
+    if (pA || pB || pK) splits = (1ll << pK) * ((1ll << pB) + (pA ? 1ll << (pA + pB) : 1));
+    else if (!tnc::split_pair_fits(tnc::split_blocks(np.mb, np.kb, np.kb > 0 && np.ak[0] == 1), batch(np.A),
+                                   tnc::split_blocks(np.nb, np.kb, np.kb > 0 && np.bk[0] == 1), batch(np.B)))
+        splits = 2;
+    return (double)splits + (double)(1ll << (pA + pB + pK)) * (c.ks ? 2 : 1);
+}
+
 static void level_cost_uncached(tnc_net* net, int mode, int64_t b, bool with_inv, double* launches,
                                 double* seconds) {
     const Plan& P = net->plan;
@@ -254,16 +271,15 @@ static void level_cost_uncached(tnc_net* net, int mode, int64_t b, bool with_inv
     for (bool per : {false, true}) {
         if (!per && !with_inv) continue;
         for (const Group& g : level_groups(net, mode, per)) {
-            bool grouped = !g.fp32.empty();
+            *launches += (g.fp32.empty() ? 0 : 1) + (double)g.stems.size();
             for (int v : g.tc) {
                 const NodePlan& np = P.nodes[v - net->n_leaves];
-                if (shape_choice(net, mode, np.mb, np.nb, np.kb, np.is_root)) *launches += 3;
-                else if (tnc::gemm_f32_tiles(np.mb, np.nb) >= 256) *launches += 1;
-                else grouped = true;
+                *launches += shape_choice(net, mode, np.mb, np.nb, np.kb, np.is_root) ? tc_launches(net, mode, np, per ? b : 1) : 1;
             }
-            if (grouped) *launches += 1;
             for (auto* list : {&g.fp32, &g.tc})
                 for (int v : *list) *seconds += node_s(P.nodes[v - net->n_leaves], per ? (double)b : 1.0);
+            for (int gi : g.stems)
+                for (int k : P.stems[gi].steps) *seconds += node_s(P.nodes[k], per ? (double)b : 1.0);
         }
     }
     for (const NodePlan& np : P.nodes)

@@ -112,6 +112,10 @@ cudaError_t launch_split(const SplitParams& p, int mode, int batch, cudaStream_t
 // Both operands of a contraction in one launch; *done false: too large to gain by it.
 cudaError_t launch_split_pair(const SplitParams& a, int batch_a, const SplitParams& b, int batch_b, int mode, cudaStream_t s,
                               bool* done);
+// Whether it takes one launch: blocks of one batch entry of the operands (of 2^rb rows
+// and 2^kb columns; k_unit: consecutive k are adjacent) and their batches.
+int64_t split_blocks(int rb, int kb, bool k_unit);
+bool split_pair_fits(int64_t blocks_a, int batch_a, int64_t blocks_b, int batch_b);
 cudaError_t launch_cgemm_tc(const TcGemmParams& p, int mode, const void* planesA, const void* planesB,
                             int batch, cudaStream_t s);
 // C[z][m][n] (+)= sum over s < 2^ksplit_bits, in order, of partial[s][z][m][n] (an FP64 sum

@@ -1631,6 +1631,10 @@ static bool split_pairs(const SplitParams& p) {
     return true;
 }
 
+int64_t split_blocks(int rb, int kb, bool k_unit) {
+    return ((1ll << rb) / split_tile_rows(kb, k_unit)) * ((1ll << kb) / split_tile_k(kb));
+}
+
 // Grid and shared memory of a split; false if it cannot run.
 static bool split_grid(SplitParams& p, int batch, int64_t& blocks, size_t& smem) {
     p.vec2 = split_pairs(p) ? 1 : 0;
@@ -1639,7 +1643,7 @@ static bool split_grid(SplitParams& p, int batch, int64_t& blocks, size_t& smem)
     const bool kfast = p.kb > 0 && p.ks[0] == 1;
     const int64_t SK = split_tile_k(p.kb), SR = split_tile_rows(p.kb, kfast);
     if (R < SR || SR > 128) return false;
-    blocks = (R / SR) * (K / SK);
+    blocks = split_blocks(p.rb, p.kb, kfast);
     smem = (size_t)SR * split_ld((int)SK) * sizeof(float2);
     return true;
 }
@@ -1665,6 +1669,9 @@ cudaError_t launch_split(const SplitParams& p_in, int mode, int batch, cudaStrea
 // split TF32 call 5.58 -> 5.33 ms). Beyond 2^16 blocks (2^27 elements and more, over
 // 0.3 ms) the operands keep a launch each.
 constexpr int64_t kSplitPairBlocks = 1 << 16;
+bool split_pair_fits(int64_t blocks_a, int batch_a, int64_t blocks_b, int batch_b) {
+    return blocks_a <= kSplitPairBlocks / batch_a && blocks_b <= kSplitPairBlocks / batch_b;
+}
 cudaError_t launch_split_pair(const SplitParams& a, int batch_a, const SplitParams& b, int batch_b, int mode, cudaStream_t s,
                               bool* done) {
     *done = false;
@@ -1675,7 +1682,7 @@ cudaError_t launch_split_pair(const SplitParams& a, int batch_a, const SplitPara
     size_t smem[2] = {0, 0};
     if (!split_grid(pp.p[0], batch_b, blocks[0], smem[0]) || !split_grid(pp.p[1], batch_a, blocks[1], smem[1]))
         return cudaErrorInvalidConfiguration;
-    if (blocks[0] > kSplitPairBlocks / batch_b || blocks[1] > kSplitPairBlocks / batch_a) return cudaSuccess;
+    if (!split_pair_fits(blocks[1], batch_a, blocks[0], batch_b)) return cudaSuccess;
     pp.blocks[0] = (int)blocks[0];
     pp.blocks[1] = (int)blocks[1];
     pp.first = pp.blocks[0] * batch_b;
