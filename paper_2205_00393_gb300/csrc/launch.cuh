@@ -13,7 +13,7 @@
 //
 // dep_trigger() in a kernel lets its successor start early. That pays for short
 // kernels and costs in long ones, whose successor's waiting CTAs take places and
-// issue slots from them: kernels of up to two waves call it, the others (and the
+// issue slots from them: kernels of up to two or three waves call it, the others (and the
 // stem and CTA-pair kernels) leave it to their CTAs' ends, which still hides the
 // launch. The 27 launches of a 20-qubit split BF16 call take 237 us one after
 // another, 180 without and 161 with early triggers; a 25-qubit split TF32 call
@@ -25,7 +25,7 @@
 
 namespace tnc {
 
-constexpr unsigned kTriggerCtas = 1216;  // 152 SMs x 4 CTAs x 2 waves
+constexpr unsigned kTriggerCtas = 1216;  // 152 SMs x 8: two waves at four CTAs per SM, 2.7 at the grouped FP32 kernels' three
 __device__ __forceinline__ void dep_trigger() {
     if (gridDim.x * gridDim.y * gridDim.z <= kTriggerCtas) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

@@ -12,8 +12,8 @@
 //     caller's complex128 result in a fixed order.
 // Intermediates live in one workspace arena whose offsets are planned on the
 // host by a first-fit simulation of the tensors' lifetimes (host_plan.cpp).
-// A launch-bound call runs each batch as one persistent launch instead
-// (host_persist.cpp).
+// A network that fits one CTA runs on a CTA per slice instead (host_tiny.cpp); with
+// "persistent" = 1 each batch is one persistent launch (host_persist.cpp).
 #include "host.hpp"
 
 #include <iomanip>
@@ -399,7 +399,8 @@ static tnc_status contract_range(tnc_net* net, int64_t lo, int64_t hi, int mode,
         const size_t cap = net->ws_user ? net->ws_user_bytes : std::max<size_t>(net->last_arena_bytes[0], (size_t)1 << 30);
         deps = (size_t)ar_flat.peak <= cap;
     }
-    // (a stalled test task needs it)
+    // "persistent" = 2 leaves this call to the launches below; a test task that stalls
+    // exists in the persistent executor only
     use_persist = use_persist && (net->persistent == 1 || net->persist_test_stall);
     deps = deps && use_persist;
     if (deps && !net->ws_user && net->ws_own_bytes < (size_t)ar_flat.peak) {  // a failed allocation keeps the reusing arena
@@ -656,8 +657,8 @@ tnc_status tnc_set_option(tnc_net_t net, const char* key, int64_t value) {
     } else if (k == "persist_test_stall") {
         net->persist_test_stall = value != 0;
     } else if (k == "stem_cap_log2") {
-        // a group with a step that is not in place holds two buffers of
-        // 2^value complex elements: 2 x 64 KB at 13 fits a CTA, 2 x 128 KB does not
+        // (plan_stems keeps groups within 2^12 elements: 13 is accepted and means 12 for
+        // them, but only steps on stems of more than 2^13 elements are fused then)
         if (value != 0 && (value < 2 || value > tnc::kStemMaxInner - 1))
             return fail(TNC_E_INVALID, "stem_cap_log2 must be 0 or in [2, 13]");
         net->stem_cap_log2 = (int)value;
