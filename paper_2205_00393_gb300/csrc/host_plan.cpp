@@ -324,7 +324,8 @@ std::string plan_key(const tnc_net* net, int mode, int64_t nb) {
            std::to_string(g_tune_version) + ":" + std::to_string(net->force_choice) + ":" +
            std::to_string(net->tc_row_bytes) + ":" + std::to_string(net->tuning ? 1 : 0) + ":" +
            std::to_string(net->in_many ? 1 : 0) + ":" + std::to_string(net->stem_cap_log2) + ":" +
-           std::to_string(net->plan.stem_cap) + ":" + std::to_string(net_plane_cap_log2(net));
+           std::to_string(net->plan.stem_cap) + ":" + std::to_string(net->stem_coalesce_bits) + ":" +
+           std::to_string(net->stem_min_outer) + ":" + std::to_string(net_plane_cap_log2(net));
 }
 
 // First-fit simulation of the workspace for a batch of `nb` slices, cached

@@ -1,0 +1,53 @@
+"""Stem options that change after a network was used: plans kept by the options they
+depend on must not serve the new ones. Tensors that a fused group keeps on chip have
+no place in its workspace plan, so a plan of other groups has none for tensors that
+are now stored."""
+
+import numpy as np
+import pytest
+
+from tnc_inputs import circuit_to_network, grid_rqc, stem_path
+
+OPTIONS = [("stem_coalesce_bits", 0), ("stem_coalesce_bits", 6), ("stem_min_outer_log2", 0), ("stem_min_outer_log2", 12),
+           ("stem_cap_log2", 10), ("stem_cap_log2", 0)]
+
+
+def _net():
+    from paper_2205_00393_gb300 import Network
+    c = grid_rqc(4, 4, 10, 3, n_open=2)
+    t = circuit_to_network(c).as_complex64()
+    net = Network.from_tn(t)
+    net.set_path(stem_path(t, c))
+    return net
+
+
+@pytest.mark.parametrize("key,value", OPTIONS)
+def test_plans_follow_the_options(libtnc, key, value):
+    def stats(net):
+        peak = net.arena(1)["peak"]  # (plans the groups)
+        st = net.stats()
+        assert st["workspace_batch1"] == net.workspace_bytes(1) == peak
+        return st
+
+    used, fresh = _net(), _net()
+    before = stats(used)  # plans made with the defaults
+    fresh.set_option(key, value)
+    used.set_option(key, value)
+    a, b = stats(used), stats(fresh)
+    assert a["stem_groups"] == b["stem_groups"] != before["stem_groups"]
+    assert a["level_cost"] == b["level_cost"] != before["level_cost"]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("key,value", OPTIONS)
+def test_results_follow_the_options(libtnc, key, value):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    net = _net()
+    want = net.contract().cpu().numpy()
+    net.set_option(key, value)
+    got = net.contract().cpu().numpy()
+    net.check_device()
+    # (sums of at most 2^4 products per step may be ordered differently: 400 steps of 2^-24)
+    assert np.max(np.abs(got - want)) <= 400 * 2.0 ** -24 * np.max(np.abs(want))
