@@ -401,11 +401,13 @@ tnc_status tnc_contract_many(int n, const tnc_net_t* nets, const int64_t* slice_
     auto it = cache.find(key.str());
     if (it != cache.end()) {
         // a network's own workspace may have been reallocated by a later call
-        // of its own: the cached sequence addresses the old one
+        // of its own: the cached sequence addresses the old one (a smaller one may
+        // have come to its place, after an allocation that failed)
         for (int i = 0; i < n && it != cache.end(); ++i) {
             const tnc_net* net = nets[i];
             const char* cur = static_cast<const char*>(net->ws_user ? net->ws_user : net->ws_own);
-            if (cur != it->second->wss[i]) {
+            const size_t bytes = net->ws_user ? net->ws_user_bytes : net->ws_own_bytes;
+            if (cur != it->second->wss[i] || bytes < (size_t)it->second->arenas[i].peak) {
                 cache.erase(it);
                 it = cache.end();
             }

@@ -104,3 +104,44 @@ def test_batch_that_cannot_be_had(libtnc):
     assert np.array_equal(out.cpu().numpy(), one)
     net.contract_variants(0, count, mode=mode, out=out)  # and in a batch again
     assert net.stats()["last_batch"] == batch and np.array_equal(out.cpu().numpy(), one)
+
+
+@pytest.mark.gpu
+def test_many_after_a_workspace_was_lost(libtnc):
+    """contract_many replays a kept sequence in the networks' own workspaces. After a batch
+    that could not be had, a network's workspace may be a smaller one (at the same
+    address, perhaps): the sequence is built anew, and results stay the same."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2205_00393_gb300 import contract_many
+    mode, count = 2, 20
+    circuit, net = _net(4, 5, 12, 4, 18, 0)
+    _, other = _net(3, 4, 8, 1, 8, 0)
+    nets = [net, other]
+    for q in nets:
+        q.set_option("persistent", 0)
+    net.set_leaf_variants(*bitstring_variants(circuit, random_bitstrings(circuit, count, 5)))
+    ranges = [(0, 8 * net.n_slices), (0, other.n_slices)]  # (slices of eight variants)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        outs = [torch.empty(q.n_out, dtype=torch.complex128, device="cuda") for q in nets]
+        out = torch.empty((count, net.n_out), dtype=torch.complex128, device="cuda")
+        for _ in range(3):  # eager, captured, replayed
+            contract_many(nets, ranges, mode, outs=outs, stream=stream)
+        stream.synchronize()
+        want = [o.cpu().numpy() for o in outs]
+        torch.cuda.empty_cache()
+        left = 400 << 20
+        full = torch.empty(torch.cuda.mem_get_info()[0] - left, dtype=torch.uint8, device="cuda")
+        net.contract_variants(0, count, mode=mode, out=out, stream=stream)
+        net.check_device(stream)
+        del full
+        torch.cuda.empty_cache()
+        for _ in range(2):
+            for o in outs:
+                o.fill_(float("nan"))
+            contract_many(nets, ranges, mode, outs=outs, stream=stream)
+            stream.synchronize()
+            # (other numbers of slices per batch: bound of test_many_gpu.py)
+            assert all(np.allclose(o.cpu().numpy(), w, rtol=1e-9, atol=1e-15) for o, w in zip(outs, want))
