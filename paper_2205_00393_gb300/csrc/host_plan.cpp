@@ -229,7 +229,9 @@ void plan_stems(tnc_net* net) {
             mx = std::max(mx, inner);
         }
         const int lim = std::min(cap, kStemGroupCap);
-        if (mx > lim || (int)U.size() < net->stem_min_outer || U.size() > 30) return false;
+        // (no inner mode: a branch that its slice makes a scalar, with no run of
+        // elements to keep together; the GEMM kernels take it)
+        if (mx < 1 || mx > lim || (int)U.size() < net->stem_min_outer || U.size() > 30) return false;
         g = StemGroupPlan();
         g.steps.assign(chain.begin() + i, chain.begin() + i + n);
         g.in = P.nodes[chain[i]].A;
