@@ -750,6 +750,7 @@ tnc_status tnc_stats(tnc_net_t net, char* json, size_t cap) {
         }
     }
     if (net->plan.valid) {
+        if (net->plan.stem_cap != net->stem_cap_log2) plan_stems(net);
         o << ",\"workspace_batch1\":" << plan_arena(net, 1, TNC_FP32).peak;
         o << ",\"last_batch\":" << net->last_batch;
         o << ",\"backward_keep_every\":" << net->last_keep_every;
@@ -792,7 +793,6 @@ tnc_status tnc_stats(tnc_net_t net, char* json, size_t cap) {
         }
         o << "}";
         // fused stem groups for the current cap: [first node, steps, outer bits, inner bits, per slice]
-        if (net->plan.stem_cap != net->stem_cap_log2) plan_stems(net);
         o << ",\"stem_cap_log2\":" << net->stem_cap_log2 << ",\"stem_groups\":[";
         for (size_t gi = 0; gi < net->plan.stems.size(); ++gi) {
             const StemGroupPlan& g = net->plan.stems[gi];

@@ -38,6 +38,15 @@ def test_plans_follow_the_options(libtnc, key, value):
     assert a["level_cost"] == b["level_cost"] != before["level_cost"]
 
 
+def test_first_statistics_are_those_of_the_groups(libtnc):
+    """tnc_stats reports the workspace and the launches of the fused groups that it lists,
+    also before anything else planned them."""
+    first, later = _net(), _net()
+    a = first.stats()
+    later.workspace_bytes(1)
+    assert a == later.stats() == first.stats()
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("key,value", OPTIONS)
 def test_results_follow_the_options(libtnc, key, value):
